@@ -1,0 +1,734 @@
+// Folding long runs of prefix rows into the interface on the tcgen05 tensor
+// cores (Sec. 2.2, Eq. global-summary, App. A.2): lsp_prefill (one request's
+// whole prefix, Fig. 3) and lsp_view_update calls whose row capacity is a
+// chunk of a prefix rather than one round's accepted tokens.  bf16 storage,
+// head dim 128, at most 16 summary queries a head and 8 query heads a KV head.
+//
+// For every tapped layer l and query head h the new rows' statistics are
+//     s_j = g_r . k_j / sqrt(d),  eta_N = log sum_j exp(s_j),
+//     m_N = sum_j exp(s_j - eta_N) v_j,
+// merged with the stored (eta_A, m_A) by Eq. summary-update (a prefill merges
+// with the empty prefix).  A unit is one (request, layer, KV head): its
+// queries are the 16 REP rows of the KV head's REP query heads (R padded to
+// 16), its keys the request's new rows in blocks of 128.
+//
+// What bounds it: the K/V rows, read once from HBM.  The arithmetic is small
+// for tcgen05 (about 0.4 of the time the rows take to arrive at REP = 4) but
+// was the bound on mma.sync, one warp a query head.
+//
+// fold_tc_kernel, one CTA per SM, an equal share of the 128-row blocks of all
+// units each (a share may end one unit and begin the next, so no last wave is
+// left over whatever the row counts are):
+//   warp 8      TMA producer: K and V blocks (32 KB each, 128-byte swizzle)
+//               through a ring of four or five slots: at least 64 KB of loads
+//               in flight an SM, what HBM's latency asks for
+//   warp 9      TMEM allocation and MMA issue.  S^T = K G^T: keys on the 128
+//               lanes, queries on N, two buffers, so the next block's scores
+//               run under this block's softmax.  O^T += V^T P^T: dims on the
+//               lanes, V as the MN-major A operand straight from its rows, P
+//               as the MN-major B operand.  Both operands of P V take the
+//               layout their producer writes, so nothing is transposed.
+//   warps 0-7   softmax: a thread owns one key (TMEM lane) and half of the
+//               queries, P = 2^((s - ref) log2(e) / sqrt(d)) is written as a
+//               bf16 high part and a bf16 remainder (two MMAs, ~16
+//               significant bits), and the sums stay in registers.
+//
+// The reference ref of each query is not the running maximum: bf16 and fp32
+// share their exponent range, so P keeps its precision under any reference
+// near the maximum.  ref is the maximum over the first block, and is raised
+// only when a score passes it by 24 in base-2 units (one compare a score and
+// one barrier a block instead of a maximum across the 128 lanes for every
+// query and block).  The accumulator is drained into registers every
+// kFlushBlocks blocks and when ref moves: tcgen05 accumulation drops low bits,
+// and a short run keeps its error below that of the 2048-row segments of the
+// mma.sync kernel this replaces.
+//
+// fold_merge_kernel merges a unit's pieces (one per CTA share that touches
+// it) and the stored state, in share order: deterministic.
+//
+// Measured (GB300, Qwen3-8B heads, 5 layers): lsp_prefill of 131072 rows
+// (2.68 GB) 745 us with the mma.sync kernel, 411 + 7 us now (6.5 TB/s, the copy
+// bandwidth); lsp_view_update of 2048 rows 232 -> 24 us for one request, 423 ->
+// 183 us for 16.  Relative error of m against 64 bits at 131072 rows: 4.6e-6 ->
+// 2.8e-6.
+#include <algorithm>
+#include <type_traits>
+
+#include "common.cuh"
+#include "lsp_internal.h"
+
+namespace lsp {
+namespace {
+
+constexpr int kFoldD = 128;                  // head dim
+constexpr int kFoldKeys = 128;               // keys per block (UMMA M)
+constexpr int kFoldSoftmax = 256;            // softmax threads (8 warps)
+constexpr int kFoldThreads = kFoldSoftmax + 64;
+constexpr int kFoldSlot = kFoldKeys * 256;   // bytes of one K or V block
+constexpr int kFoldRec = 16 + 16 * kFoldD;   // floats per (piece, query head): eta[16], m[16][d]
+constexpr int kFlushBlocks = 8;
+constexpr float kRefSlack = 24.f;            // log2 units a score may pass its reference by
+constexpr int kFoldMaxC = 64;
+constexpr int kCopyBatch = 4;                // window vectors a thread has in flight (K and V each)
+constexpr int kFoldMaxSlots = 5;
+
+struct FoldLayout {
+  int slots;
+  uint32_t off_p, off_ring, off_misc, bytes;
+};
+
+// bytes: G [2][16 REP][128 B], P high and remainder [64-query blocks][128][128 B],
+// the ring, then references, scales and 1 / sums, block counts and barriers
+__host__ __device__ constexpr FoldLayout fold_layout(int rep) {
+  FoldLayout L{};
+  const int nb = (16 * rep + 63) / 64;
+  L.off_p = (uint32_t)rep * 4096u;
+  L.off_ring = L.off_p + 2u * (uint32_t)nb * 16384u;
+  const uint32_t misc = 3u * 128u * 4u + 272u + 160u;
+  const int fit = (int)((227u * 1024u - 1024u - misc - L.off_ring) / (uint32_t)kFoldSlot);
+  L.slots = fit < kFoldMaxSlots ? fit : kFoldMaxSlots;
+  L.off_misc = L.off_ring + (uint32_t)L.slots * kFoldSlot;
+  L.bytes = L.off_misc + misc + 1024u;
+  return L;
+}
+static_assert(fold_layout(8).slots >= 4 && fold_layout(4).slots == 5, "K and V of two blocks fit the ring");
+
+__host__ __device__ constexpr uint32_t fold_tmem_cols(int rep) {
+  uint32_t c = 32;
+  while (c < 48u * (uint32_t)rep) c *= 2;    // two score buffers and the output, 16 rep columns each
+  return c;
+}
+
+// MN-major operand with 128-byte swizzling: 64 contiguous elements per 128-B
+// row, 8 rows of K per 1024-B group, `lbo` bytes between 64-element blocks.
+__device__ __forceinline__ uint64_t fold_desc_mn(uint32_t saddr, uint32_t lbo) {
+  uint64_t d = 0;
+  d |= (uint64_t)((saddr & 0x3FFFFu) >> 4);
+  d |= (uint64_t)((lbo >> 4) & 0x3FFFu) << 16;
+  d |= (uint64_t)(1024u >> 4) << 32;
+  d |= (uint64_t)1 << 46;
+  d |= (uint64_t)2 << 61;
+  return d;
+}
+
+// kind::f16, bf16 A and B, fp32 D, M = 128, N = n; `mn`: A and B MN-major.
+__device__ __forceinline__ uint32_t fold_idesc(int n, bool mn) {
+  return (1u << 4) | (1u << 7) | (1u << 10) | (mn ? (3u << 15) : 0u) | ((uint32_t)(n >> 3) << 17) |
+         ((uint32_t)(kFoldKeys >> 4) << 24);
+}
+
+__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, float* v) {
+  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
+               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
+               : "r"(taddr));
+}
+template <int N>
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float* v) {
+  static_assert(N % 8 == 0, "columns come in eights");
+#pragma unroll
+  for (int c = 0; c < N; c += 8) tmem_ld8_issue(taddr + (uint32_t)c, v + c);
+  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
+  // the values may be used only after the wait
+#pragma unroll
+  for (int c = 0; c < N; ++c) asm volatile("" : "+f"(v[c]));
+}
+
+__device__ __forceinline__ float fold_ex2(float x) {
+  float y;
+  asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return y;
+}
+
+__device__ __forceinline__ void mbar_arrive1(uint32_t bar) {
+  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
+}
+
+__device__ __forceinline__ void st_v4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+
+// Wait that gives up after kWaitLimitNs (recorded), or as soon as another
+// role of the CTA has given up: every loop below still runs to its end then.
+__device__ __forceinline__ bool fold_wait(uint32_t bar, uint32_t parity, volatile int* stop, unsigned* err) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = global_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 15u) == 0) {
+      if (*stop) return false;
+      if (global_ns() - t0 > kWaitLimitNs) {
+        set_err(err, LSP_DEV_TIMEOUT);
+        *stop = 1;
+        return false;
+      }
+    }
+  }
+}
+
+__device__ __forceinline__ bool softmax_any(bool x) {
+  uint32_t r;
+  asm volatile(
+      "{\n .reg .pred p, q;\n setp.ne.u32 p, %1, 0;\n barrier.cta.red.or.pred q, 1, %2, p;\n selp.u32 %0, 1, 0, q;\n}"
+      : "=r"(r)
+      : "r"((uint32_t)x), "n"(kFoldSoftmax)
+      : "memory");
+  return r != 0;
+}
+
+// The warp's max or sum over its 32 lanes of eight columns: lane L gets column
+// L & 7 (nine shuffles instead of five for each column).
+template <bool kMax>
+__device__ __forceinline__ float reduce8(const float* x, int lane) {
+  auto op = [](float a, float b) { return kMax ? fmaxf(a, b) : a + b; };
+  float y[4], z[2];
+#pragma unroll
+  for (int k = 0; k < 4; ++k) {
+    const float send = (lane & 4) ? x[k] : x[k + 4], keep = (lane & 4) ? x[k + 4] : x[k];
+    y[k] = op(keep, __shfl_xor_sync(0xffffffffu, send, 4));
+  }
+#pragma unroll
+  for (int k = 0; k < 2; ++k) {
+    const float send = (lane & 2) ? y[k] : y[k + 2], keep = (lane & 2) ? y[k + 2] : y[k];
+    z[k] = op(keep, __shfl_xor_sync(0xffffffffu, send, 2));
+  }
+  const float send = (lane & 1) ? z[0] : z[1], keep = (lane & 1) ? z[1] : z[0];
+  float r = op(keep, __shfl_xor_sync(0xffffffffu, send, 1));
+  r = op(r, __shfl_xor_sync(0xffffffffu, r, 8));
+  return op(r, __shfl_xor_sync(0xffffffffu, r, 16));
+}
+
+// Accepted rows of request i of this call (0 where the count is out of range).
+__device__ __forceinline__ int fold_rows(const FoldParams& p, int i) {
+  const int n = p.acc ? p.acc[i] : p.rows;
+  return n < 0 || n > p.rows ? 0 : n;
+}
+
+// pre[i] = blocks per unit of requests 0 .. i-1 (one warp; nreq <= 64).
+__device__ __forceinline__ void fold_prefix(const FoldParams& p, int* pre, int lane) {
+  auto nblk = [&](int i) { return i < p.nreq && p.R > 0 ? (fold_rows(p, i) + kFoldKeys - 1) / kFoldKeys : 0; };
+  const int a = nblk(2 * lane), b = nblk(2 * lane + 1);
+  int s = a + b;
+#pragma unroll
+  for (int o = 1; o < 32; o <<= 1) {
+    const int v = __shfl_up_sync(0xffffffffu, s, o);
+    if (lane >= o) s += v;
+  }
+  pre[2 * lane] = s - a - b;
+  pre[2 * lane + 1] = s - b;
+  if (lane == 31) pre[kFoldMaxC] = s;
+}
+
+// CTAs that get blocks: every share holds at least one (1 when there are none).
+__device__ __forceinline__ long long fold_shares(long long total, unsigned grid) {
+  return max(1ll, min(total, (long long)grid));
+}
+
+// The piece of a CTA's share [f, f_end) that begins at flattened block f: the
+// blocks of all units in order (request, layer x KV head, block).
+struct FoldPiece {
+  int req, lg, blk, n, unit;       // n blocks from block blk of unit = req * LG + lg
+};
+__device__ __forceinline__ FoldPiece fold_piece(const int* pre, int nreq, int LG, int f, int f_end) {
+  FoldPiece q;
+  int i = 0;
+  while (i + 1 < nreq && f >= pre[i + 1] * LG) ++i;
+  const int nb = pre[i + 1] - pre[i], r = f - pre[i] * LG;
+  q.req = i;
+  q.lg = r / nb;
+  q.blk = r - q.lg * nb;
+  q.n = min(nb - q.blk, f_end - f);
+  q.unit = i * LG + q.lg;
+  return q;
+}
+
+template <int REP>
+__global__ void __launch_bounds__(kFoldThreads, 1)
+    fold_tc_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv, const FoldParams p) {
+  constexpr int Q = 16 * REP, QH = 8 * REP;               // queries; a softmax thread's share of them
+  constexpr int CW = REP <= 5 ? QH : (REP == 7 ? 8 : 16); // score columns a thread holds at a time
+  constexpr FoldLayout L = fold_layout(REP);
+  constexpr int NS = L.slots, NB = (Q + 63) / 64;
+  extern __shared__ uint8_t fsm_raw[];
+  uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(fsm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
+  const uint32_t s_g = smem_u32(sm), s_p = s_g + L.off_p, s_ring = s_g + L.off_ring;
+  float* sref = reinterpret_cast<float*>(sm + L.off_misc);   // reference of each query
+  float* sscale = sref + 128;                                // factor of a reference that moved
+  float* sinv = sscale + 128;                                // 1 / sum
+  int* pre = reinterpret_cast<int*>(sinv + 128);             // [65]
+  uint64_t* bars = reinterpret_cast<uint64_t*>(pre + 68);
+  uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2 * kFoldMaxSlots + 8);
+  volatile int* stop = reinterpret_cast<volatile int*>(tslot + 1);
+  volatile int* sfresh = stop + 1;
+  float* exch = reinterpret_cast<float*>(sm + L.off_p);      // [4][Q] between warps, while P is idle
+  // new rows and first window slot of each request, in the remainder half of P
+  // until the first block's barriers (every window copy is done by then)
+  int* srows = reinterpret_cast<int*>(sm + L.off_p + NB * 16384);
+  int* sslot = srows + kFoldMaxC;
+  const uint32_t bar0 = smem_u32(bars);
+  auto b_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
+  auto b_empty = [&](int s) { return bar0 + 8u * (uint32_t)(kFoldMaxSlots + s); };
+  auto b_sfull = [&](int s) { return bar0 + 8u * (uint32_t)(2 * kFoldMaxSlots + s); };
+  auto b_sempty = [&](int s) { return bar0 + 8u * (uint32_t)(2 * kFoldMaxSlots + 2 + s); };
+  const uint32_t b_p = bar0 + 8u * (2 * kFoldMaxSlots + 4), b_pv = b_p + 8, b_g = b_p + 16, b_end = b_p + 24;
+
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  if (tid == 0) {
+    for (int s = 0; s < NS; ++s) {
+      mbar_init(b_full(s), 1);
+      mbar_init(b_empty(s), 1);
+    }
+    for (int s = 0; s < 2; ++s) {
+      mbar_init(b_sfull(s), 1);
+      mbar_init(b_sempty(s), kFoldSoftmax / 32);
+    }
+    mbar_init(b_p, kFoldSoftmax / 32);
+    mbar_init(b_pv, 1);
+    mbar_init(b_g, kFoldSoftmax / 32);
+    mbar_init(b_end, 1);
+    *stop = 0;
+    fence_barrier_init();
+    tma_prefetch_desc(&mk);
+    tma_prefetch_desc(&mv);
+  }
+  if (warp == 9) tmem_alloc(smem_u32(tslot), fold_tmem_cols(REP));
+  griddep_launch();
+  griddep_wait();
+  if (warp == 0) fold_prefix(p, pre, lane);
+  if (warp == 1)
+    for (int i = lane; i < p.nreq; i += 32) {
+      const int n = fold_rows(p, i);
+      srows[i] = n;
+      sslot[i] = p.W > 0 ? (int)(((p.replace ? 0 : p.t[p.b0 + i]) + n - min(n, p.W)) % p.W) : 0;
+    }
+  tc_fence_before();
+  __syncthreads();
+  tc_fence_after();
+  const uint32_t tmem = *tslot, t_o = tmem + 2u * Q;
+  const int LG = p.L * p.nkv;
+  const long long total = (long long)pre[kFoldMaxC] * LG;
+  const long long nshare = fold_shares(total, gridDim.x);
+  const int f0 = (int)min(total, total * blockIdx.x / nshare), f1 = (int)min(total, total * (blockIdx.x + 1) / nshare);
+
+  if (warp == 8 && lane == 0) {
+    // ------------------------------------------------------------ TMA producer
+    const uint64_t pol = policy_evict_first();
+    int q = 0;                                            // ring position: K and V of a block in turn
+    bool ok = true;
+    for (int f = f0; f < f1 && ok;) {
+      const FoldPiece pc = fold_piece(pre, p.nreq, LG, f, f1);
+      const int l = pc.lg / p.nkv, x = (pc.lg % p.nkv) * kFoldD;
+      const int y0 = (pc.req * p.L + l) * p.rows + pc.blk * kFoldKeys;
+      for (int i = 0; i < pc.n && ok; ++i)
+        for (int kv = 0; kv < 2; ++kv, ++q) {
+          const int s = q % NS;
+          if (q >= NS && !fold_wait(b_empty(s), (uint32_t)(q / NS - 1) & 1u, stop, p.err)) { ok = false; break; }
+          mbar_expect_tx(b_full(s), kFoldSlot);
+          const uint32_t dst = s_ring + (uint32_t)s * kFoldSlot;
+          const CUtensorMap* mp = kv ? &mv : &mk;
+          tma_load_2d(dst, mp, b_full(s), x, y0 + i * kFoldKeys, pol);
+          tma_load_2d(dst + kFoldSlot / 2, mp, b_full(s), x + 64, y0 + i * kFoldKeys, pol);
+        }
+      f += pc.n;
+    }
+    // every load has landed before the CTA's shared memory goes away
+    for (int i = max(0, q - NS); i < q; ++i) mbar_wait(b_full(i % NS), (uint32_t)(i / NS) & 1u, p.err);
+  } else if (warp == 9 && lane == 0) {
+    // ------------------------------------------------------------ MMA issue
+    const uint32_t id_s = fold_idesc(Q, false), id_o = fold_idesc(Q, true);
+    int n = 0, piece = 0;                                 // block and piece of this CTA
+    bool ok = true;
+    auto scores = [&](int nn) {
+      const int s = (2 * nn) % NS, buf = nn & 1;
+      ok = ok && fold_wait(b_full(s), (uint32_t)(2 * nn / NS) & 1u, stop, p.err);
+      if (nn >= 2) ok = ok && fold_wait(b_sempty(buf), (uint32_t)(nn / 2 - 1) & 1u, stop, p.err);
+      if (!ok) return;
+      tc_fence_after();
+      const uint32_t sk = s_ring + (uint32_t)s * kFoldSlot;
+#pragma unroll
+      for (int ks = 0; ks < kFoldD / 16; ++ks) {
+        const uint32_t kb = (uint32_t)(ks >> 2), in = (uint32_t)(ks & 3) * 32u;
+        umma_f16(tmem + (uint32_t)(buf * Q), sdesc_sw128(sk + kb * (kFoldSlot / 2) + in),
+                 sdesc_sw128(s_g + kb * (uint32_t)(Q * 128) + in), id_s, ks > 0 ? 1u : 0u);
+      }
+      umma_commit(b_empty(s));
+      umma_commit(b_sfull(buf));
+    };
+    for (int f = f0; f < f1; ++piece) {
+      const FoldPiece pc = fold_piece(pre, p.nreq, LG, f, f1);
+      ok = ok && fold_wait(b_g, (uint32_t)piece & 1u, stop, p.err);
+      scores(n);
+      for (int i = 0; i < pc.n; ++i, ++n) {
+        if (i + 1 < pc.n) scores(n + 1);
+        const int s = (2 * n + 1) % NS;
+        ok = ok && fold_wait(b_full(s), (uint32_t)((2 * n + 1) / NS) & 1u, stop, p.err);
+        ok = ok && fold_wait(b_p, (uint32_t)n & 1u, stop, p.err);
+        if (!ok) continue;
+        tc_fence_after();
+        const uint32_t sv = s_ring + (uint32_t)s * kFoldSlot;
+        const uint32_t keep = *sfresh ? 0u : 1u;          // fresh: the accumulator was drained
+#pragma unroll
+        for (int ks = 0; ks < kFoldKeys / 16; ++ks) {
+          const uint64_t ad = fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2);
+          umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)ks * 2048u, 16384u), id_o, ks > 0 ? 1u : keep);
+          umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)(NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o, 1u);
+        }
+        umma_commit(b_empty(s));
+        umma_commit(b_pv);
+      }
+      f += pc.n;
+    }
+    umma_commit(b_end);                                   // no MMA outlives the CTA's TMEM
+    mbar_wait(b_end, 0, p.err);
+  } else if (warp < 8) {
+    // ------------------------------------------------------------ softmax
+    const int quad = warp & 3, half = warp >> 2;
+    const int j = quad * 32 + lane;                       // key of the block (S), dim of the head (O)
+    const uint32_t tl = (uint32_t)(quad * 32) << 16;
+    const int c0 = half * QH;                             // first of this thread's queries
+    const float isd = rsqrtf((float)kFoldD), sl2 = 1.4426950408889634f * isd;
+    const uint32_t prow = s_p + (uint32_t)(j >> 3) * 1024u + (uint32_t)(j & 7) * 128u;
+    auto bar = [] { named_bar(1, kFoldSoftmax); };
+    // the queries' maxima (kMax) or sums over the block's 128 keys into out(query, value)
+    auto across = [&](auto is_max, const float* x, int cbase, int n) {
+#pragma unroll
+      for (int c = 0; c < n; c += 8) {
+        const float r = reduce8<decltype(is_max)::value>(x + c, lane);
+        if (lane < 8) exch[quad * Q + cbase + c + lane] = r;
+      }
+    };
+
+    auto load_g = [&](int lg) {
+      const int l = lg / p.nkv, g = lg % p.nkv;
+      const bf16* G = static_cast<const bf16*>(p.G) + ((size_t)l * p.nq + (size_t)g * REP) * p.R * kFoldD;
+      for (int i = tid; i < Q * 16; i += kFoldSoftmax) {
+        const int row = i >> 4, c8 = i & 15, hh = row >> 4, r = row & 15;
+        uint4 v = make_uint4(0u, 0u, 0u, 0u);
+        if (r < p.R) v = *reinterpret_cast<const uint4*>(G + ((size_t)hh * p.R + r) * kFoldD + c8 * 8);
+        st_v4(s_g + (uint32_t)((c8 >> 3) * (Q * 128) + (row >> 3) * 1024 + (row & 7) * 128 + (((c8 & 7) ^ (row & 7)) << 4)),
+              v.x, v.y, v.z, v.w);
+      }
+      fence_proxy_async_smem();
+      __syncwarp();
+      if (lane == 0) mbar_arrive1(b_g);
+    };
+    if (f0 < f1) load_g(fold_piece(pre, p.nreq, LG, f0, f1).lg);
+
+    // ---- while the first rows land: the window ring (row q of the prefix in
+    // slot q mod W), the boundary rows, counts out of range
+    if (p.acc && blockIdx.x == 0 && tid < p.nreq && (p.acc[tid] < 0 || p.acc[tid] > p.rows)) set_err(p.err, LSP_DEV_BAD_DELTA);
+    {
+      const int vpr = p.nkv * (kFoldD / 8), span = p.W * vpr;   // 16-byte vectors of a row (all KV heads), of a window
+      const int items = p.nreq * p.L * span;
+      for (int k0 = (int)blockIdx.x * (kCopyBatch * kFoldSoftmax) + tid; k0 < items; k0 += (int)gridDim.x * (kCopyBatch * kFoldSoftmax)) {
+        uint4 xk[kCopyBatch], xv[kCopyBatch];
+        size_t dst[kCopyBatch];
+        bool on[kCopyBatch];
+#pragma unroll
+        for (int u = 0; u < kCopyBatch; ++u) {
+          const int k = k0 + u * kFoldSoftmax, ul = k / span, w = k - ul * span, r = w / vpr, c = w - r * vpr;
+          const int i = ul / p.L, l = ul - i * p.L;
+          on[u] = k < items && r < min(srows[i], p.W);
+          if (on[u]) {
+            const int n = srows[i];
+            int slot = sslot[i] + r;
+            if (slot >= p.W) slot -= p.W;
+            dst[u] = ((((size_t)(p.b0 + i) * p.L + l) * p.nkv + (c >> 4)) * p.W + slot) * kFoldD + (size_t)(c & 15) * 8;
+            const size_t src = (((size_t)ul * p.rows + (n - min(n, p.W)) + r) * vpr + c) * 8;
+            xk[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.k) + src);
+            xv[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.v) + src);
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kCopyBatch; ++u)
+          if (on[u]) {
+            *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_k) + dst[u]) = xk[u];
+            *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_v) + dst[u]) = xv[u];
+          }
+      }
+      if (p.h)
+        for (int ul = (int)blockIdx.x; ul < p.nreq * p.L; ul += (int)gridDim.x) {
+          const int i = ul / p.L, n = srows[i];
+          if (n == 0) continue;
+          const bf16* hin = static_cast<const bf16*>(p.hid) + ((size_t)ul * p.h_rows + (p.h_rows == 1 ? 0 : n - 1)) * p.H;
+          bf16* hout = static_cast<bf16*>(p.h) + ((size_t)p.b0 * p.L + ul) * p.H;
+          for (int k = tid * 8; k < p.H; k += kFoldSoftmax * 8)
+            *reinterpret_cast<uint4*>(hout + k) = *reinterpret_cast<const uint4*>(hin + k);
+        }
+    }
+
+    int n = 0;
+    bool first_piece = true;
+    for (int f = f0; f < f1;) {
+      const FoldPiece pc = fold_piece(pre, p.nreq, LG, f, f1);
+      if (!first_piece) load_g(pc.lg);                    // every score MMA of the last piece has completed
+      first_piece = false;
+      const int nrows = fold_rows(p, pc.req);
+      float acc[QH], sum[QH];
+#pragma unroll
+      for (int c = 0; c < QH; ++c) acc[c] = sum[c] = 0.f;
+      int since = 0;                                      // blocks in the accumulator
+      auto drain = [&] {
+        tc_fence_after();
+        float o[CW];
+#pragma unroll
+        for (int cc = 0; cc < QH; cc += CW) {
+          tmem_ld_cols<CW>(t_o + tl + (uint32_t)(c0 + cc), o);
+#pragma unroll
+          for (int c = 0; c < CW; ++c) acc[cc + c] += o[c];
+        }
+      };
+      for (int i = 0; i < pc.n; ++i, ++n) {
+        const int buf = n & 1;
+        const int nvalid = nrows - (pc.blk + i) * kFoldKeys;   // rows of this block (may exceed 128)
+        const bool valid = j < nvalid;
+        fold_wait(b_sfull(buf), (uint32_t)(n >> 1) & 1u, stop, p.err);
+        tc_fence_after();
+        const uint32_t ts = tmem + tl + (uint32_t)(buf * Q + c0);
+        float s[CW];
+        auto load = [&](int cc) {
+          tmem_ld_cols<CW>(ts + (uint32_t)cc, s);
+          if (!valid) {
+#pragma unroll
+            for (int c = 0; c < CW; ++c) s[c] = -INFINITY;
+          }
+        };
+        // does a score pass its reference by more than the slack?
+        bool move = i == 0;
+        if (i == 0) {
+          if (CW == QH) load(0);
+        } else {
+          float mx = -INFINITY;
+#pragma unroll
+          for (int cc = 0; cc < QH; cc += CW) {
+            load(cc);
+#pragma unroll
+            for (int c = 0; c < CW; c += 4) {
+              const float4 r = *reinterpret_cast<const float4*>(sref + c0 + cc + c);
+              mx = fmaxf(mx, fmaxf(fmaxf(s[c] - r.x, s[c + 1] - r.y), fmaxf(s[c + 2] - r.z, s[c + 3] - r.w)));
+            }
+          }
+          move = softmax_any(mx * sl2 > kRefSlack);
+          // P and the accumulator are free once the previous block's MMAs are done
+          fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
+          if (move || since == kFlushBlocks) {
+            drain();
+            since = 0;
+          }
+        }
+        if (move) {
+#pragma unroll
+          for (int cc = 0; cc < QH; cc += CW) {
+            if (CW != QH) load(cc);
+            across(std::true_type{}, s, c0 + cc, CW);
+          }
+          bar();
+          if (tid < Q) {
+            float m = fmaxf(fmaxf(exch[tid], exch[Q + tid]), fmaxf(exch[2 * Q + tid], exch[3 * Q + tid]));
+            if (m == -INFINITY) m = 0.f;                  // no finite score yet
+            const float old = i == 0 ? m : sref[tid];
+            m = fmaxf(m, old);
+            sscale[tid] = fold_ex2((old - m) * sl2);
+            sref[tid] = m;
+          }
+          bar();
+          if (i > 0) {
+#pragma unroll
+            for (int c = 0; c < QH; ++c) {
+              const float a = sscale[c0 + c];
+              acc[c] *= a;
+              sum[c] *= a;
+            }
+          }
+        }
+        // P = high + remainder (bf16 each), eight queries a 16-byte store
+#pragma unroll
+        for (int cc = 0; cc < QH; cc += CW) {
+          if (CW != QH) load(cc);
+#pragma unroll
+          for (int c = 0; c < CW; c += 8) {
+            const float4 ra = *reinterpret_cast<const float4*>(sref + c0 + cc + c);
+            const float4 rb = *reinterpret_cast<const float4*>(sref + c0 + cc + c + 4);
+            const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
+            uint32_t hi[4], lo[4];
+#pragma unroll
+            for (int e = 0; e < 8; e += 2) {
+              const float x0 = fold_ex2((s[c + e] - r[e]) * sl2), x1 = fold_ex2((s[c + e + 1] - r[e + 1]) * sl2);
+              sum[cc + c + e] += x0;
+              sum[cc + c + e + 1] += x1;
+              const uint32_t h = pack_bf16(x0, x1);
+              hi[e >> 1] = h;
+              lo[e >> 1] = pack_bf16(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u));
+            }
+            const int col = c0 + cc + c;
+            const uint32_t a = prow + (uint32_t)(col >> 6) * 16384u + (uint32_t)((((col & 63) >> 3) ^ (j & 7)) << 4);
+            st_v4(a, hi[0], hi[1], hi[2], hi[3]);
+            st_v4(a + (uint32_t)(NB * 16384), lo[0], lo[1], lo[2], lo[3]);
+          }
+        }
+        tc_fence_before();
+        __syncwarp();
+        if (lane == 0) mbar_arrive1(b_sempty(buf));
+        if (nvalid < kFoldKeys) {
+          // the unit's ragged end: rows past it may hold anything, and 0 x V has to stay 0
+          const int vs = (2 * n + 1) % NS;
+          fold_wait(b_full(vs), (uint32_t)((2 * n + 1) / NS) & 1u, stop, p.err);
+          if (!valid) {
+            const uint32_t a = s_ring + (uint32_t)vs * kFoldSlot + (uint32_t)half * (kFoldSlot / 2) + (uint32_t)j * 128u;
+#pragma unroll
+            for (int c = 0; c < 8; ++c) st_v4(a + (uint32_t)c * 16u, 0u, 0u, 0u, 0u);
+          }
+        }
+        fence_proxy_async_smem();
+        if (tid == 0) *sfresh = since == 0;
+        ++since;
+        __syncwarp();
+        if (lane == 0) mbar_arrive1(b_p);
+      }
+      // ---- the piece's (eta, m) of every query
+      fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
+      drain();
+      tc_fence_before();
+      across(std::false_type{}, sum, c0, QH);
+      bar();
+      float* rec = p.ws + (size_t)((int)blockIdx.x + pc.unit) * REP * kFoldRec;
+      if (tid < Q) {
+        const float t = (exch[tid] + exch[Q + tid]) + (exch[2 * Q + tid] + exch[3 * Q + tid]);
+        sinv[tid] = 1.0f / t;
+        rec[(tid >> 4) * kFoldRec + (tid & 15)] = sref[tid] * isd + logf(t);
+      }
+      bar();
+#pragma unroll
+      for (int c = 0; c < QH; ++c) {
+        const int col = c0 + c;
+        rec[(col >> 4) * kFoldRec + 16 + (col & 15) * kFoldD + j] = acc[c] * sinv[col];
+      }
+      f += pc.n;
+    }
+  }
+
+  tc_fence_before();
+  __syncthreads();
+  if (warp == 9) {
+    tc_fence_after();
+    tmem_dealloc(tmem, fold_tmem_cols(REP));
+  }
+}
+
+// One CTA per (request, layer, query head): 16 rows x 16 groups of 8 dims.
+// The pieces' weights come from one pass over their eta, so their values are
+// all in flight at once (a chain of two-way merges waited for each in turn).
+// CTA 0 also advances t.
+constexpr int kMergeBatch = 4;
+
+__global__ void __launch_bounds__(256) fold_merge_kernel(const FoldParams p, const int grid) {
+  __shared__ int pre[kFoldMaxC + 1];
+  griddep_launch();
+  griddep_wait();
+  if (threadIdx.x < 32) fold_prefix(p, pre, threadIdx.x);
+  __syncthreads();
+  if (blockIdx.x == 0 && (int)threadIdx.x < p.nreq) {
+    const int n = fold_rows(p, threadIdx.x);
+    int64_t* t = p.t + p.b0 + threadIdx.x;
+    if (p.replace) *t = n;
+    else if (n > 0) *t += n;
+  }
+  const int i = blockIdx.x / (p.L * p.nq), lh = blockIdx.x % (p.L * p.nq);
+  const int l = lh / p.nq, h = lh % p.nq;
+  const int rep = p.nq / p.nkv, lg = l * p.nkv + h / rep, hh = h % rep;
+  const int r = threadIdx.x >> 4, c0 = (threadIdx.x & 15) * 8;
+  const int nb = pre[i + 1] - pre[i];
+  if (r >= p.R || nb == 0) return;
+  const long long LG = (long long)p.L * p.nkv, total = pre[kFoldMaxC] * LG;
+  const long long f0 = pre[i] * LG + (long long)lg * nb, nshare = fold_shares(total, grid);
+  const int s0 = (int)(((f0 + 1) * nshare - 1) / total), s1 = (int)(((f0 + nb) * nshare - 1) / total);
+  const int unit = i * (int)LG + lg;
+  auto rec = [&](int s) { return p.ws + ((size_t)(s + unit) * rep + hh) * kFoldRec; };
+  const size_t q = (((size_t)(p.b0 + i) * p.L + l) * p.nq + h) * p.R + r;
+  float* mo = p.m + q * kFoldD + c0;
+  const float ea = p.replace ? -INFINITY : p.eta[q];
+  float mx = ea;
+  for (int s = s0; s <= s1; ++s) mx = fmaxf(mx, __ldcg(rec(s) + r));
+  float w = 0.f, m[8];
+#pragma unroll
+  for (int e = 0; e < 8; ++e) m[e] = 0.f;
+  auto add = [&](float wt, const float4& a, const float4& b) {
+    w += wt;
+    const float v[8] = {a.x, a.y, a.z, a.w, b.x, b.y, b.z, b.w};
+#pragma unroll
+    for (int e = 0; e < 8; ++e) m[e] = fmaf(wt, v[e], m[e]);
+  };
+  if (!p.replace) add(expf(ea - mx), *reinterpret_cast<const float4*>(mo), *reinterpret_cast<const float4*>(mo + 4));
+  for (int s = s0; s <= s1; s += kMergeBatch) {
+    float4 a[kMergeBatch], b[kMergeBatch];
+    float e[kMergeBatch];
+#pragma unroll
+    for (int u = 0; u < kMergeBatch; ++u)
+      if (s + u <= s1) {
+        const float* x = rec(s + u);
+        e[u] = __ldcg(x + r);
+        a[u] = __ldcg(reinterpret_cast<const float4*>(x + 16 + r * kFoldD + c0));
+        b[u] = __ldcg(reinterpret_cast<const float4*>(x + 16 + r * kFoldD + c0 + 4));
+      }
+#pragma unroll
+    for (int u = 0; u < kMergeBatch; ++u)
+      if (s + u <= s1) add(expf(e[u] - mx), a[u], b[u]);
+  }
+  const float inv = 1.0f / w;
+  *reinterpret_cast<float4*>(mo) = make_float4(m[0] * inv, m[1] * inv, m[2] * inv, m[3] * inv);
+  *reinterpret_cast<float4*>(mo + 4) = make_float4(m[4] * inv, m[5] * inv, m[6] * inv, m[7] * inv);
+  // this query's eta is read by its 16 threads, all of one half-warp, above
+  __syncwarp(0xffffu << ((threadIdx.x & 16) ? 16 : 0));
+  if ((threadIdx.x & 15) == 0) p.eta[q] = mx + logf(w);
+}
+
+template <int REP>
+int launch_rep(const FoldParams& p, const CUtensorMap& mk, const CUtensorMap& mv, int grid, cudaStream_t s) {
+  constexpr FoldLayout L = fold_layout(REP);
+  static_assert(L.bytes <= 227 * 1024, "one CTA's shared memory");
+  static const cudaError_t attr =
+      cudaFuncSetAttribute(fold_tc_kernel<REP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
+  if (attr != cudaSuccess) return LSP_ERR_CUDA;
+  return launch_pdl(fold_tc_kernel<REP>, dim3(grid), dim3(kFoldThreads), L.bytes, s, mk, mv, p) == cudaSuccess ? LSP_OK
+                                                                                                               : LSP_ERR_CUDA;
+}
+
+}  // namespace
+
+bool fold_supported(int dtype, int d, int R, int nq, int nkv) {
+  return dtype == LSP_DTYPE_BF16 && d == kFoldD && R >= 0 && R <= 16 && nq / nkv <= 8;
+}
+
+// One record per query head for each (share, unit) pair a walk over the
+// flattened blocks meets: at most one more than the shares for each unit.
+size_t fold_ws_floats(int C, int L, int nq, int nkv, int num_sms) {
+  return ((size_t)num_sms + (size_t)C * L * nkv) * (nq / nkv) * kFoldRec;
+}
+
+int launch_fold(const FoldParams& p, int num_sms, cudaStream_t s) {
+  if (p.rows < 1 || p.nreq < 1 || p.nreq > kFoldMaxC || !p.ws) return LSP_ERR_UNSUPPORTED;
+  if (p.H % 8) return LSP_ERR_SHAPE;
+  CUtensorMap mk, mv;
+  const uint64_t rows = (uint64_t)p.nreq * p.L * p.rows, pitch = (uint64_t)p.nkv * kFoldD;
+  int rc;
+  if ((rc = tmap_2d_bf16_sw128(&mk, p.k, pitch, rows, pitch * 2, 64, kFoldKeys)) != LSP_OK) return rc;
+  if ((rc = tmap_2d_bf16_sw128(&mv, p.v, pitch, rows, pitch * 2, 64, kFoldKeys)) != LSP_OK) return rc;
+  // one CTA per SM, fewer when the capacity holds fewer blocks
+  const long long blocks = (long long)p.nreq * p.L * p.nkv * ((p.rows + kFoldKeys - 1) / kFoldKeys);
+  const int grid = (int)std::max(1ll, std::min((long long)num_sms, blocks));
+  switch (p.nq / p.nkv) {
+    case 1: rc = launch_rep<1>(p, mk, mv, grid, s); break;
+    case 2: rc = launch_rep<2>(p, mk, mv, grid, s); break;
+    case 3: rc = launch_rep<3>(p, mk, mv, grid, s); break;
+    case 4: rc = launch_rep<4>(p, mk, mv, grid, s); break;
+    case 5: rc = launch_rep<5>(p, mk, mv, grid, s); break;
+    case 6: rc = launch_rep<6>(p, mk, mv, grid, s); break;
+    case 7: rc = launch_rep<7>(p, mk, mv, grid, s); break;
+    case 8: rc = launch_rep<8>(p, mk, mv, grid, s); break;
+    default: return LSP_ERR_UNSUPPORTED;
+  }
+  if (rc != LSP_OK) return rc;
+  return launch_pdl(fold_merge_kernel, dim3(p.nreq * p.L * p.nq), dim3(256), 0, s, p, grid) == cudaSuccess ? LSP_OK
+                                                                                                           : LSP_ERR_CUDA;
+}
+
+}  // namespace lsp

@@ -71,7 +71,7 @@ struct lsp_state {
   size_t part_bytes = 0;
   float* part_val = nullptr;
   int* part_idx = nullptr;
-  float* prefill_ws = nullptr;       // prefill segment partials (bf16, d = 128 configs)
+  float* fold_ws = nullptr;          // piece records of long folds (configs fold_supported serves)
   float* ver_sa = nullptr;           // verification row partials and draw partials
   float* ver_sb = nullptr;
   int* ver_si = nullptr;
@@ -234,8 +234,9 @@ int lsp_state_create(const lsp_config* cfg, lsp_state** out) {
   const size_t w_pv = off; off = align256(off + (size_t)2 * st->nblk * c.C * 4);
   const size_t w_pi = off; off = align256(off + (size_t)2 * st->nblk * c.C * 4);
   const size_t w_sync = off; off = align256(off + sample_sync_bytes(c.B));
-  const bool prefill_ok = c.dtype == LSP_DTYPE_BF16 && c.d == 128;
-  const size_t w_pf = off; off = align256(off + (prefill_ok ? prefill_ws_floats(c.L, c.nq) * sizeof(float) : 0));
+  const bool fold_ok = fold_supported(c.dtype, c.d, c.R, c.nq, c.nkv);
+  const size_t w_pf = off;
+  off = align256(off + (fold_ok ? fold_ws_floats(c.C, c.L, c.nq, c.nkv, st->num_sms) * sizeof(float) : 0));
   const size_t ver_rows = (size_t)c.C * (2 * c.B + 1) * verify_max_stat_chunks(c.V);
   const size_t w_vsa = off; off = align256(off + ver_rows * sizeof(float));
   const size_t w_vsb = off; off = align256(off + ver_rows * sizeof(float));
@@ -257,7 +258,7 @@ int lsp_state_create(const lsp_config* cfg, lsp_state** out) {
   st->part_val = reinterpret_cast<float*>(w + w_pv);
   st->part_idx = reinterpret_cast<int*>(w + w_pi);
   st->sample_sync = reinterpret_cast<unsigned long long*>(w + w_sync);
-  st->prefill_ws = prefill_ok ? reinterpret_cast<float*>(w + w_pf) : nullptr;
+  st->fold_ws = fold_ok ? reinterpret_cast<float*>(w + w_pf) : nullptr;
   st->ver_sa = reinterpret_cast<float*>(w + w_vsa);
   st->ver_sb = reinterpret_cast<float*>(w + w_vsb);
   st->ver_si = reinterpret_cast<int*>(w + w_vsi);
@@ -314,12 +315,41 @@ static int feats_h_rows(const lsp_target_feats* f) {
   return f->h_rows == 1 ? 1 : -1;
 }
 
+// Row capacity from which a view update takes the segmented tcgen05 fold.  The
+// per-(request, layer, KV head) kernel walks its rows 32 at a time in one CTA
+// (about 4 us a pass); the fold pays a fixed price for each such unit an SM gets
+// a piece of.  Measured at the Qwen3-8B heads, 5 layers (per-unit kernel vs
+// fold, us): C = 1: 14.1 vs 14.7 at 64 rows, 24.0 vs 14.7 at 128; C = 4: 28.3
+// vs 23.9 at 128; C = 16: 78.9 vs 92.1 at 256, 128 vs 106 at 512.
+static bool fold_pays(const lsp_state* st, int rows) {
+  const lsp_config& c = st->cfg;
+  return st->fold_ws && c.R > 0 && rows >= 64 + 80ll * c.C * c.L * c.nkv / st->num_sms;
+}
+
+static FoldParams fold_params(const lsp_state* st, const lsp_target_feats* f) {
+  const lsp_config& c = st->cfg;
+  FoldParams p = {};
+  p.k = f->k; p.v = f->v; p.hid = f->h; p.rows = f->rows; p.h_rows = feats_h_rows(f); p.G = st->G;
+  p.win_k = st->win_k; p.win_v = st->win_v; p.m = st->m; p.eta = st->eta; p.h = st->h; p.t = st->t;
+  p.ws = st->fold_ws; p.err = st->err;
+  p.L = c.L; p.nq = c.nq; p.nkv = c.nkv; p.W = c.W; p.R = c.R; p.H = c.H;
+  return p;
+}
+
 int lsp_view_update(lsp_state* st, const lsp_target_feats* f, const int32_t* acc,
                     lsp_stream_t stream) {
   if (!st || !f || !acc || !f->k || !f->v || f->rows < 1 || feats_h_rows(f) < 0) return LSP_ERR_ARG;
   if (!f->h && st->h) return LSP_ERR_ARG;
   if (!st->initialized) return LSP_ERR_STATE;
   const lsp_config& c = st->cfg;
+  if (fold_pays(st, f->rows)) {
+    FoldParams p = fold_params(st, f);
+    p.acc = acc; p.nreq = c.C; p.b0 = 0; p.replace = 0;
+    mark(st, 0, S(stream));
+    const int rc = launch_fold(p, st->num_sms, S(stream));
+    mark(st, 1, S(stream));
+    return rc;
+  }
   ViewParams p;
   p.k_new = f->k; p.v_new = f->v; p.h_new = f->h; p.rows = f->rows; p.h_rows = feats_h_rows(f); p.acc = acc;
   p.G = st->G; p.win_k = st->win_k; p.win_v = st->win_v; p.m = st->m; p.eta = st->eta;
@@ -337,12 +367,10 @@ int lsp_prefill(lsp_state* st, int b, const lsp_target_feats* f, lsp_stream_t st
   if (!st->initialized) return LSP_ERR_STATE;
   const lsp_config& c = st->cfg;
   if (b < 0 || b >= c.C) return LSP_ERR_ARG;
-  PrefillParams p;
-  p.k = f->k; p.v = f->v; p.hid = f->h; p.rows = f->rows; p.h_rows = feats_h_rows(f); p.G = st->G;
-  p.win_k = st->win_k; p.win_v = st->win_v; p.m = st->m; p.eta = st->eta; p.h = st->h; p.t = st->t;
-  p.ws = st->prefill_ws;
-  p.b = b; p.L = c.L; p.nq = c.nq; p.nkv = c.nkv; p.d = c.d; p.W = c.W; p.R = c.R; p.H = c.H;
-  return launch_prefill(p, c.dtype, S(stream));
+  if (!st->fold_ws) return LSP_ERR_UNSUPPORTED;
+  FoldParams p = fold_params(st, f);
+  p.acc = nullptr; p.nreq = 1; p.b0 = b; p.replace = 1;
+  return launch_fold(p, st->num_sms, S(stream));
 }
 
 int lsp_verify(lsp_state* st, const float* target_logits, const float* draft_logits,

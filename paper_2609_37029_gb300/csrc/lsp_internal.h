@@ -189,26 +189,31 @@ int launch_attention_tc(const AttnParams& p, const AttnTcPlan& pl, cudaStream_t 
 int tmap_2d_bf16_sw128(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t rows, uint64_t row_bytes,
                        uint32_t box_inner, uint32_t box_rows);
 
-// ------------------------------------------------------------------ prefill
-struct PrefillParams {
-  const void* k;          // request b's prefix K: [L][rows][nkv][d] dtype
-  const void* v;          // V, same layout
-  const void* hid;        // hidden states [L][h_rows][H] dtype (h_rows = rows or 1: the last row only)
-  int rows;               // t (>= 1)
+// ------------------------------------------------------------------ folding long runs of rows
+// New rows of nreq requests (state rows b0 ..), each up to `rows` long: a
+// prefill (one request, replace = 1, acc = null: all `rows` rows) or a view
+// update over a chunk of a prefix.
+struct FoldParams {
+  const void* k;          // [nreq][L][rows][nkv][d] bf16
+  const void* v;
+  const void* hid;        // [nreq][L][h_rows][H] (h_rows = rows, or 1: the boundary row only)
+  int rows;               // row capacity per (request, layer) (>= 1)
   int h_rows;
+  const int32_t* acc;     // [nreq] new rows, or null: `rows` of each
   const void* G;          // [L][nq][R][d]
   void* win_k;            // state window [C][L][nkv][W][d]
   void* win_v;
   float* m;               // [C][L][nq][R][d]
   float* eta;             // [C][L][nq][R]
-  void* h;                // [C][L][H]
+  void* h;                // [C][L][H] or null
   int64_t* t;             // [C]
-  float* ws;              // prefill_ws_floats(L, nq) segment partials
-  int b, L, nq, nkv, d, W, R, H;
+  float* ws;              // fold_ws_floats(C, L, nq, nkv, num_sms) piece records
+  unsigned* err;
+  int nreq, b0, replace, L, nq, nkv, W, R, H;
 };
-constexpr int kPrefillMaxSeg = 64;   // prefix segments (CTAs per tapped layer x KV head)
-size_t prefill_ws_floats(int L, int nq);
-int launch_prefill(const PrefillParams& p, int dtype, cudaStream_t s);
+bool fold_supported(int dtype, int d, int R, int nq, int nkv);
+size_t fold_ws_floats(int C, int L, int nq, int nkv, int num_sms);
+int launch_fold(const FoldParams& p, int num_sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ verification
 struct VerifyParams {
