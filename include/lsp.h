@@ -320,14 +320,15 @@ int lsp_verify(lsp_state* st, const float* target_logits, const float* draft_log
  *   and `workspace` may be NULL. */
 size_t lsp_linear_workspace_bytes(int M, int N, int splits);
 
-/* Diagnostic, host only (needs no GPU): the launch plan the drafter's
- * projection GEMM takes for M token rows, N output features and reduction
- * length K on a device with num_sms SMs.
+/* Diagnostic, host only (needs no GPU): the split-K plan of the drafter's
+ * projections for M token rows, N output features and reduction length K on a
+ * device with num_sms SMs.
  *   swiglu = 0: a projection whose fp32 split-K partials a consumer sums
  *   (the q/k/v, o, down and boundary-fusion projections); swiglu = 1: the
  *   fused gate/up projection with N = F (gate and up each [F][K]).
- *   *splits: split-K factor; *tok_groups: CTAs per weight tile, each over
- *   *tokens_per_group consecutive token rows (a multiple of 16).
+ *   *splits: split-K factor (it fixes the order of the fp32 sums);
+ *   *tok_groups: groups of *tokens_per_group consecutive token rows (a
+ *   multiple of 16) that the plan's cost model divides M into.
  * LSP_ERR_ARG for null outputs, M outside [1, 512], N, K or num_sms < 1 or
  * an unknown dtype. */
 int lsp_gemm_plan_info(int dtype, int M, int N, int K, int swiglu, int num_sms, int* splits,

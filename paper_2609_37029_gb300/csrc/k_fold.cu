@@ -117,30 +117,18 @@ __device__ __forceinline__ uint32_t fold_idesc(int n, bool mn) {
          ((uint32_t)(kFoldKeys >> 4) << 24);
 }
 
-__device__ __forceinline__ void tmem_ld8_issue(uint32_t taddr, float* v) {
-  asm volatile("tcgen05.ld.sync.aligned.32x32b.x8.b32 {%0,%1,%2,%3,%4,%5,%6,%7}, [%8];"
-               : "=f"(v[0]), "=f"(v[1]), "=f"(v[2]), "=f"(v[3]), "=f"(v[4]), "=f"(v[5]), "=f"(v[6]), "=f"(v[7])
-               : "r"(taddr));
-}
 template <int N>
-__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float* v) {
+__device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, float (&v)[N]) {
   static_assert(N % 8 == 0, "columns come in eights");
 #pragma unroll
-  for (int c = 0; c < N; c += 8) tmem_ld8_issue(taddr + (uint32_t)c, v + c);
-  asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory");
-  // the values may be used only after the wait
-#pragma unroll
-  for (int c = 0; c < N; ++c) asm volatile("" : "+f"(v[c]));
+  for (int c = 0; c < N; c += 8) tmem_ld8(taddr + (uint32_t)c, v + c);
+  tmem_ld_wait(v);
 }
 
 __device__ __forceinline__ float fold_ex2(float x) {
   float y;
   asm("ex2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
   return y;
-}
-
-__device__ __forceinline__ void mbar_arrive1(uint32_t bar) {
-  asm volatile("mbarrier.arrive.shared::cta.b64 _, [%0];" ::"r"(bar) : "memory");
 }
 
 __device__ __forceinline__ void st_v4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
@@ -409,7 +397,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       }
       fence_proxy_async_smem();
       __syncwarp();
-      if (lane == 0) mbar_arrive1(b_g);
+      if (lane == 0) mbar_arrive(b_g);
     };
     if (f0 < f1) load_g(fold_piece(pre, p.nreq, LG, f0, f1).lg);
 
@@ -472,7 +460,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         float o[CW];
 #pragma unroll
         for (int cc = 0; cc < QH; cc += CW) {
-          tmem_ld_cols<CW>(t_o + tl + (uint32_t)(c0 + cc), o);
+          tmem_ld_cols(t_o + tl + (uint32_t)(c0 + cc), o);
 #pragma unroll
           for (int c = 0; c < CW; ++c) acc[cc + c] += o[c];
         }
@@ -486,7 +474,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         const uint32_t ts = tmem + tl + (uint32_t)(buf * Q + c0);
         float s[CW];
         auto load = [&](int cc) {
-          tmem_ld_cols<CW>(ts + (uint32_t)cc, s);
+          tmem_ld_cols(ts + (uint32_t)cc, s);
           if (!valid) {
 #pragma unroll
             for (int c = 0; c < CW; ++c) s[c] = -INFINITY;
@@ -567,7 +555,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         }
         tc_fence_before();
         __syncwarp();
-        if (lane == 0) mbar_arrive1(b_sempty(buf));
+        if (lane == 0) mbar_arrive(b_sempty(buf));
         if (nvalid < kFoldKeys) {
           // the unit's ragged end: rows past it may hold anything, and 0 x V has to stay 0
           const int vs = (2 * n + 1) % NS;
@@ -582,7 +570,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         if (tid == 0) *sfresh = since == 0;
         ++since;
         __syncwarp();
-        if (lane == 0) mbar_arrive1(b_p);
+        if (lane == 0) mbar_arrive(b_p);
       }
       // ---- the piece's (eta, m) of every query
       fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);

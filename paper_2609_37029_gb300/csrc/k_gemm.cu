@@ -3,35 +3,50 @@
 // Every dense projection of the drafter -- boundary fusion (Sec. 2.2), the
 // q/k/v, output, gate/up and down projections of each draft layer and the
 // frozen LM head (Sec. 2.3) -- has a small token count M = C*B (or C) and a
-// large weight.  The kernel therefore puts 128 weight rows on the UMMA M axis
-// and the tokens on its N axis ("swap AB"): D^T[n][m] = sum_k W[n][k] X[m][k].
+// large weight: Y[m][n] = sum_k X[m][k] W[n][k].
 //
-//   warp 0      TMA producer: the CTA's 128 x BK weight tile and its
-//               m_pad x BK activation tile per stage into an S-deep mbarrier
-//               ring, plus an L2 prefetch of the next stage's weight tile
-//   warp 1      TMEM allocation and the single-thread tcgen05.mma issue (a
-//               lean loop: this one thread's instructions set the issue rate)
-//   warps 2-5   epilogue: tcgen05.ld of the fp32 accumulators, the fused
-//               output (fp32, storage dtype, SwiGLU, or a split-K partial)
-//               staged in shared memory 16-32 tokens at a time and written
-//               by TMA tensor stores (double-buffered), so the global writes
-//               are full-line bulk copies that overlap the next chunk
+// What bounds it: the weights' HBM stream, closely followed at 256 tokens by the
+// tensor cores (an MMA of 128 tokens x N weights x 16 takes N / 2 cycles).  So
+// that nothing else does, tokens are on the UMMA M axis (one or two accumulators of up
+// to 128) and weight rows on its N axis, up to 256 of them: a k-block is 64 KB of
+// loads and 256 x 256 outputs, where a tile of 128 weight rows loaded 48 KB for half
+// of them and left twice as many k-blocks to wait for and commit.  N comes in
+// steps of 16, so the tile width is chosen for the number of SMs (choose_width)
+// and not the other way round.  Measured against that 128-row kernel (two or three CTAs an
+// SM): gate/up at 256 tokens 51 -> 38 us, LM head 242 -> 224, at 16 tokens 204 -> 175
+// (7.1 TB/s); 512 x 17408 x 5120 66 -> 57; the Qwen3-8B round 1046 -> 973 us.
 //
-// Grid: x = weight-tile CTAs x token groups (a group's CTAs share the weight
-// tile, each over m_pad consecutive tokens; the SwiGLU gate/up projection
-// takes two groups when its tiles fill under one wave of two CTAs per SM),
-// y = split-K.
+//   warp 0      TMA producer of weight tiles, one k-block a stage of a ring
+//   warp 10     the same for activation tiles, in a ring of its own: those come
+//               from L2 in half the time, so they take fewer stages and leave
+//               the shared memory to weights in flight (LM head, 256 tokens:
+//               236 -> 224 us).  Up to 128 tokens the tiles are small and warp
+//               0 loads them into the weights' stages: short launches end
+//               0.5 us earlier
+//   warp 1      TMEM allocation and the tcgen05.mma issue (one lane of a
+//               uniform warp: its instructions set the issue rate)
+//   warps 2-9   epilogue, two groups of four warps (one a token tile; one
+//               every other chunk of a single tile): tcgen05.ld of 32 features of
+//               a token row a thread, staged in shared memory (128-byte
+//               swizzle) and written by TMA tensor stores; SwiGLU needs no
+//               exchange, a thread holds a token's gate and up columns
+//
+// Grid: one CTA per work item (weight tile x token group x k split), or one per
+// SM walking the items where they make more than a wave: its ring streams
+// across item boundaries, so the next item's weights arrive under this one's
+// epilogue.
 //
 // Launched as a programmatic dependent: before the preceding kernel finishes,
-// the producer already streams this launch's weights (L2 prefetch and the
-// weight halves of the first stages); activation loads wait for it.  Split-K
-// partials are summed in split order by the consuming kernel, so results are
-// deterministic and no CTA waits on another.  Every mbarrier wait is bounded
-// and records LSP_DEV_TIMEOUT instead of spinning forever.
+// the producer already streams this launch's weights (the weight halves of the
+// first stages); activation loads wait for it.  Split-K partials are summed in
+// split order by the consuming kernel, so results are deterministic and no CTA
+// waits on another.  An output's sum runs over k in order inside one
+// accumulator: neither tile width nor token tiling changes its bits.  Every
+// mbarrier wait is bounded and records LSP_DEV_TIMEOUT instead of spinning
+// forever.
 #include <cudaTypedefs.h>
 
 #include <algorithm>
-#include <cstdlib>
 #include <mutex>
 
 #include "common.cuh"
@@ -51,154 +66,149 @@ template <> struct GemmType<float> {
   static constexpr uint32_t FMT = 2;
 };
 
-constexpr uint32_t kTileBytes = kTileRows * 128;   // one weight tile per stage: 16 KB
-// L2 prefetch distance of the weight stream, in k-blocks (one ahead: 318 -> 281 us at the
-// LM-head shape; longer distances were slower)
-constexpr int kPrefetchDist = 1;
-
-// The epilogue's named barrier (id 1) counts exactly the four epilogue warps
-// 2-5: any other warp taking that branch would leave bar.sync waiting forever.
-constexpr int kEpilogueThreads = 128;
-static_assert(kGemmThreads == 64 + kEpilogueThreads, "warp 0 TMA, warp 1 MMA, warps 2-5 epilogue");
+constexpr int kTileTok = 128;          // UMMA M: token rows of one accumulator
+constexpr int kChunk = 32;             // output features of one staged store (128 bytes of fp32)
+constexpr uint32_t kChunkBytes = kTileTok * 128;
+constexpr int kEpiGroup = 128;         // threads of one epilogue group (named barrier 1 + group)
+constexpr int kXWarp = 10;             // activation producer
+constexpr int kMaxStages = 8;
+static_assert(kGemmThreads == 96 + 2 * kEpiGroup, "warp 0 weights, warp 1 MMA, two epilogue groups, warp 10 activations");
 
 // Instruction descriptor: fp32 accumulate, A/B format `fmt`, both K-major,
 // N = n, M = 128.
 __device__ __forceinline__ uint32_t make_idesc(int n, uint32_t fmt) {
-  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(n >> 3) << 17) |
-         ((uint32_t)(kTileRows >> 4) << 24);
+  return (1u << 4) | (fmt << 7) | (fmt << 10) | ((uint32_t)(n >> 3) << 17) | ((uint32_t)(kTileTok >> 4) << 24);
 }
 
-template <typename T>
-__device__ __forceinline__ void emit_chunk(const GemmParams& p, int tile, int split, int r, int m0,
-                                           const float* v, float* xchg) {
-  const int M = p.M;
-  if (p.mode == EPI_SWIGLU) {
-#pragma unroll
-    for (int j = 0; j < 16; ++j) xchg[r * 17 + j] = v[j];
-    named_bar(1, kEpilogueThreads);
-    if (r < 64) {
-      const int f = tile * 64 + r;
-      T* Y = static_cast<T*>(p.Y);
-#pragma unroll
-      for (int j = 0; j < 16; ++j) {
-        const int m = m0 + j;
-        if (m < M && f < p.N) {
-          const float g = xchg[r * 17 + j];
-          const float u = xchg[(r + 64) * 17 + j];
-          Y[(size_t)m * p.ldy + f] = from_f<T>(g / (1.0f + expf(-g)) * u);
-        }
+__device__ __forceinline__ void st_shared4(uint32_t a, uint32_t x, uint32_t y, uint32_t z, uint32_t w) {
+  asm volatile("st.shared.v4.b32 [%0], {%1, %2, %3, %4};" ::"r"(a), "r"(x), "r"(y), "r"(z), "r"(w) : "memory");
+}
+
+// Bounded wait that also ends when another role has given up.
+__device__ __forceinline__ bool gemm_wait(uint32_t bar, uint32_t parity, volatile int* stop, unsigned* err) {
+  if (mbar_try_wait(bar, parity)) return true;
+  const uint64_t t0 = global_ns();
+  for (uint32_t i = 1;; ++i) {
+    if (mbar_try_wait(bar, parity)) return true;
+    if ((i & 31u) == 0) {
+      if (*stop) return false;
+      if (global_ns() - t0 > kWaitLimitNs) {
+        set_err(err, LSP_DEV_TIMEOUT);
+        *stop = 1;
+        return false;
       }
     }
-    named_bar(1, kEpilogueThreads);
-    return;
-  }
-  const int n = tile * kTileRows + r;
-  if (n >= p.N) return;
-  if (p.mode == EPI_T) {
-    T* Y = static_cast<T*>(p.Y);
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (m0 + j < M) Y[(size_t)(m0 + j) * p.ldy + n] = from_f<T>(v[j]);
-  } else {
-    float* Y = static_cast<float*>(p.Y);
-    if (p.mode == EPI_PARTIAL) Y += (size_t)split * M * p.ldy;
-#pragma unroll
-    for (int j = 0; j < 16; ++j)
-      if (m0 + j < M) Y[(size_t)(m0 + j) * p.ldy + n] = v[j];
   }
 }
 
-constexpr uint32_t kXchgStride = 33;                          // SwiGLU exchange row (floats)
-constexpr uint32_t kXchgBytes = 17408;                        // 128 x 33 floats, 1 KB aligned
-
-// silu(gate) * up for NT tokens of gate feature f (exchange rows f and f + 64)
-// into the staged [token][64] output tile.  Every input is loaded before the
-// arithmetic, and the fast exponential and division keep the chain short
-// (their relative error is far below the bf16 rounding of the result).  Measured
-// at the Qwen3-8B gate/up shape: 1.5 -> 0.2 us per 32-token chunk.
-template <typename T, int NT>
-__device__ __forceinline__ void swiglu_rows(const float* xchg, T* o, int f, int t0) {
-  float g[NT], u[NT];
-#pragma unroll
-  for (int j = 0; j < NT; ++j) {
-    g[j] = xchg[f * kXchgStride + t0 + j];
-    u[j] = xchg[(f + 64) * kXchgStride + t0 + j];
-  }
-#pragma unroll
-  for (int j = 0; j < NT; ++j) o[(t0 + j) * 64 + f] = from_f<T>(__fdividef(g[j], 1.0f + __expf(-g[j])) * u[j]);
+// A work item: weight rows [row0, row0 + width) of segment `seg`, token rows
+// from tok0, k-blocks [kb0, kb0 + nk) of split `split`; output column col0.
+struct GemmItem {
+  int seg, row0, cols, col0, tok0, split, kb0, nk;
+};
+__device__ __forceinline__ GemmItem gemm_item(const GemmParams& p, int item) {
+  GemmItem w;
+  const int per = p.n_tiles * p.tok_groups;
+  w.split = item / per;
+  const int r = item - w.split * per, tile = r / p.tok_groups;   // the groups of a tile are adjacent: it is shared through L2
+  w.tok0 = (r - tile * p.tok_groups) * p.m_pad;
+  w.seg = p.nseg > 2 && tile >= p.seg_tile0[2] ? 2 : p.nseg > 1 && tile >= p.seg_tile0[1] ? 1 : 0;
+  w.row0 = (tile - p.seg_tile0[w.seg]) * p.width;
+  w.cols = min(p.width, p.seg_rows[w.seg] - w.row0);
+  w.col0 = p.seg_col0[w.seg] + w.row0;
+  w.kb0 = (int)((long long)w.split * p.kblocks / p.splits);
+  w.nk = (int)((long long)(w.split + 1) * p.kblocks / p.splits) - w.kb0;
+  return w;
 }
 
-// Epilogue through shared memory and TMA stores (4 warps, r = accumulator
-// row = output feature of the tile).  Chunk c of TT tokens: every thread
-// loads its row's TT accumulators, writes them (or, for SwiGLU, the
-// activation of its share after a gate/up exchange) into staging buffer
-// c & 1, and one thread stores the buffer with a TMA tensor store into the
-// [split][token][feature] view of Y at the CTA's first token row tok0.
-// Token rows past M and feature columns past N fall outside the view and are
-// not written; the chunks tile the CTA's m_pad tokens exactly, so no store
-// reaches the next token group's rows.
-template <typename T>
-__device__ __forceinline__ void epilogue_tma(const GemmParams& p, const CUtensorMap* to, uint8_t* smem,
-                                             uint32_t lane_base, int tile, int tok0, int split,
-                                             int r) {
-  const bool swiglu = p.mode == EPI_SWIGLU;
-  const bool f32out = p.mode == EPI_F32 || p.mode == EPI_PARTIAL;
-  const int es = f32out ? 4 : (int)sizeof(T);
-  const int cols = swiglu ? 64 : kTileRows;                   // output features of one weight tile
-  const int TT = p.out_tok;
-  float* xchg = reinterpret_cast<float*>(smem);              // SwiGLU: [128][kXchgStride]
-  uint8_t* stg0 = smem + (swiglu ? kXchgBytes : 0);
-  const uint32_t buf_bytes = (uint32_t)(TT * cols * es);     // <= 16 KB
-  const bool issuer = r == 0;
+// fp32 output (final or one split's partial) of one accumulator, in chunks of
+// 32 features, thread = token row.  A chunk is written to a staging buffer of
+// the group (stg, nbuf of them; n counts the group's chunks) and stored by
+// one thread.  Token rows past M and features past N fall outside the output
+// view; a segment's last tile stops at its `cols`.
+__device__ __forceinline__ void epilogue_f32(const GemmParams& p, const CUtensorMap* to, uint8_t* stg, int nbuf, int& n,
+                                             uint32_t acc, const GemmItem& w, int tok0, int c_first, int c_step, int row,
+                                             int bar) {
+  const bool issuer = row == 0;
   const uint64_t pol_part = policy_evict_last();
-  const int m_end = min(p.m_pad, p.M - tok0);                 // > 0: no token group is empty
-  int chunk = 0;
-  {
-    for (int m0 = 0; m0 < m_end; m0 += TT, ++chunk) {       // no store box starts past row M
-      float v[32];
-      const uint32_t col = (uint32_t)m0;
-      if (TT == 32) tmem_ld32(lane_base + col, v);
-      else tmem_ld16(lane_base + col, v);
-      uint8_t* stg = stg0 + (chunk & 1) * buf_bytes;
-      if (issuer && chunk >= 2) bulk_wait_read<1>();         // the store two chunks back has read stg
-      named_bar(1, kEpilogueThreads);
-      if (swiglu) {
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < TT) xchg[r * kXchgStride + j] = v[j];
-        named_bar(1, kEpilogueThreads);
-        // thread (f = r & 63, half = r >> 6) forms tokens [half * TT/2, (half + 1) * TT/2)
-        const int f = r & 63, t0 = (r >> 6) * (TT / 2);
-        T* o = reinterpret_cast<T*>(stg);
-        if (TT == 32) swiglu_rows<T, 16>(xchg, o, f, t0);
-        else swiglu_rows<T, 8>(xchg, o, f, t0);
-      } else if (f32out) {
-        float* o = reinterpret_cast<float*>(stg);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < TT) o[j * kTileRows + r] = v[j];
-      } else {
-        T* o = reinterpret_cast<T*>(stg);
-#pragma unroll
-        for (int j = 0; j < 32; ++j)
-          if (j < TT) o[j * kTileRows + r] = from_f<T>(v[j]);
-      }
-      fence_proxy_async_smem();
-      named_bar(1, kEpilogueThreads);
+  for (int c = c_first * kChunk; c < w.cols; c += c_step * kChunk, ++n) {
+    float v[32];
+    tmem_ld32(acc + (uint32_t)c, v);
+    uint8_t* buf = stg + (size_t)(n % nbuf) * kChunkBytes;
+    if (n >= nbuf && p.tma_out) {                       // the buffer's last store has read it
       if (issuer) {
-        if (p.mode == EPI_PARTIAL)   // read once more, by the consumer: kept in L2 past the weight stream
-          tma_store_3d_hint(to, smem_u32(stg), tile * cols, tok0 + m0, split, pol_part);
-        else
-          tma_store_3d(to, smem_u32(stg), tile * cols, tok0 + m0, split);
-        bulk_commit();
+        if (nbuf >= 4) bulk_wait_read<3>();
+        else if (nbuf >= 2) bulk_wait_read<1>();
+        else bulk_wait_read<0>();
       }
+      named_bar(bar, kEpiGroup);
+    }
+    const uint32_t r = smem_u32(buf) + (uint32_t)row * 128u;
+    if (row < p.tile_tok) {
+#pragma unroll
+      for (int q = 0; q < 8; ++q)
+        st_shared4(r + (uint32_t)((q ^ (row & 7)) << 4), __float_as_uint(v[4 * q]), __float_as_uint(v[4 * q + 1]),
+                   __float_as_uint(v[4 * q + 2]), __float_as_uint(v[4 * q + 3]));
+    }
+    if (p.tma_out) {
+      fence_proxy_async_smem();
+      named_bar(bar, kEpiGroup);
+      if (issuer && tok0 < p.M) {
+        if (p.mode == EPI_PARTIAL)   // read once more, by the consumer: kept in L2 past the weight stream
+          tma_store_3d_hint(to, smem_u32(buf), w.col0 + c, tok0, w.split, pol_part);
+        else
+          tma_store_3d(to, smem_u32(buf), w.col0 + c, tok0, w.split);
+      }
+      if (issuer) bulk_commit();
+    } else {
+      // no tensor map describes Y (its row pitch or address is no multiple of
+      // 16 bytes): a warp writes its own 32 rows, lanes along the features
+      __syncwarp();
+      const int lane = row & 31, row0 = row - lane, f = w.col0 + c + lane;
+      float* Y = static_cast<float*>(p.Y) + (p.mode == EPI_PARTIAL ? (size_t)w.split * p.M * p.ldy : 0);
+      const int rows = min(min(32, p.tile_tok - row0), p.M - tok0 - row0);
+      if (f < p.N)
+        for (int i = 0; i < rows; ++i)
+          Y[(size_t)(tok0 + row0 + i) * p.ldy + f] =
+              *reinterpret_cast<const float*>(buf + (size_t)(row0 + i) * 128 + (((lane >> 2) ^ (i & 7)) << 4) + (lane & 3) * 4);
+      __syncwarp();
     }
   }
-  if (issuer) bulk_wait_read<0>();                            // staging smem is released at exit
 }
 
-template <typename T, int kOcc>
-__global__ void __launch_bounds__(kGemmThreads, kOcc)
+// silu(gate) * up of a token row, eight features at a time, into the row of the
+// staged [token][width / 2] tile.  The fast exponential and division keep the
+// chain short (their relative error is far below the bf16 rounding of the
+// result).  The widths are odd multiples of eight features, so the rows'
+// 16-byte stores spread over the banks without swizzling.
+template <typename T>
+__device__ __forceinline__ void swiglu_row(uint32_t acc, uint32_t dst, int fw, int first, int step, bool on) {
+  for (int c = first * 8; c < fw; c += step * 8) {
+    float g[8], u[8], y[8];
+    tmem_ld8(acc + (uint32_t)c, g);
+    tmem_ld8(acc + (uint32_t)(fw + c), u);
+    tmem_ld_wait(g);
+    tmem_ld_wait(u);
+#pragma unroll
+    for (int e = 0; e < 8; ++e) y[e] = __fdividef(g[e], 1.0f + __expf(-g[e])) * u[e];
+    if (on) {
+      if constexpr (sizeof(T) == 2) {
+        st_shared4(dst + (uint32_t)c * 2u, pack_bf16(y[0], y[1]), pack_bf16(y[2], y[3]), pack_bf16(y[4], y[5]),
+                   pack_bf16(y[6], y[7]));
+      } else {
+        const uint32_t a = dst + (uint32_t)c * 4u;
+        st_shared4(a, __float_as_uint(y[0]), __float_as_uint(y[1]), __float_as_uint(y[2]), __float_as_uint(y[3]));
+        st_shared4(a + 16u, __float_as_uint(y[4]), __float_as_uint(y[5]), __float_as_uint(y[6]), __float_as_uint(y[7]));
+      }
+    }
+    __syncwarp();
+  }
+}
+
+// kTwoRings: activations in a ring of their own (more than 128 tokens), else
+// in the weights' stages.
+template <typename T, bool kTwoRings>
+__global__ void __launch_bounds__(kTwoRings ? kGemmThreads : kGemmThreads - 32, 2)
     gemm_kernel(const __grid_constant__ CUtensorMap ta0, const __grid_constant__ CUtensorMap ta1,
                 const __grid_constant__ CUtensorMap ta2, const __grid_constant__ CUtensorMap tb,
                 const __grid_constant__ CUtensorMap to, const __grid_constant__ GemmParams p) {
@@ -206,39 +216,32 @@ __global__ void __launch_bounds__(kGemmThreads, kOcc)
   extern __shared__ uint8_t smem_raw[];
   uint8_t* smem = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(smem_raw) + 1023) &
                                              ~static_cast<uintptr_t>(1023));
-  const int S = p.stages;
-  const uint32_t stage_a = kTileBytes;
-  const uint32_t stage_bytes = stage_a + (uint32_t)p.m_pad * 128;
-  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + (size_t)S * stage_bytes);
-  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 2 * S + 1);
-  volatile int* s_abort = reinterpret_cast<volatile int*>(tmem_slot + 1);
+  const int SW = p.w_stages, SX = kTwoRings ? p.x_stages : p.w_stages;
+  const uint32_t x_bytes = (uint32_t)p.m_pad * 128u, w_bytes = (uint32_t)p.width * 128u;
+  uint64_t* bars = reinterpret_cast<uint64_t*>(smem + p.off_bar);
+  uint32_t* tmem_slot = reinterpret_cast<uint32_t*>(bars + 4 * kMaxStages + 5);
+  volatile int* stop = reinterpret_cast<volatile int*>(tmem_slot + 1);
 
-  const int warp = threadIdx.x >> 5;
+  const int warp = warp_index();
   const int lane = threadIdx.x & 31;
-  // blockIdx.x = weight tile x token groups + group: the CTAs of one weight
-  // tile are adjacent, so they run together and share the tile through L2
-  const int group = (int)blockIdx.x % p.tok_groups;
-  const int tile = (int)blockIdx.x / p.tok_groups;
-  const int tok0 = group * p.m_pad;                            // first token row of this CTA
-  const int split = blockIdx.y;
-  const int kb0 = (int)((long long)split * p.kblocks / p.splits);
-  const int kb1 = (int)((long long)(split + 1) * p.kblocks / p.splits);
-  const int nk = kb1 - kb0;
-  const uint32_t expect = kTileBytes + (uint32_t)p.m_pad * 128;
+  const uint32_t bar0 = smem_u32(bars), x0 = smem_u32(smem), w0 = x0 + (uint32_t)SX * x_bytes;
+  auto wfull = [&](int s) { return bar0 + 8u * s; };
+  auto wempty = [&](int s) { return bar0 + 8u * (kMaxStages + s); };
+  auto xfull = [&](int s) { return bar0 + 8u * (2 * kMaxStages + s); };
+  auto xempty = [&](int s) { return bar0 + 8u * (3 * kMaxStages + s); };
+  auto acc_full = [&](int a) { return bar0 + 8u * (4 * kMaxStages + a); };
+  auto acc_empty = [&](int a) { return bar0 + 8u * (4 * kMaxStages + 2 + a); };
+  const uint32_t end_bar = bar0 + 8u * (4 * kMaxStages + 4);
 
-  const uint32_t bar0 = smem_u32(bars);
-  auto full_bar = [&](int s) { return bar0 + 8u * s; };
-  auto empty_bar = [&](int s) { return bar0 + 8u * (S + s); };
-  const uint32_t acc_bar = bar0 + 8u * (2 * S);
-
-  if (threadIdx.x == 0) {
-    for (int s = 0; s < S; ++s) {
-      mbar_init(full_bar(s), 1);
-      mbar_init(empty_bar(s), 1);
-    }
-    mbar_init(acc_bar, 1);
-    *s_abort = 0;
+  // one barrier a thread of warp 2: each takes its arrivals (the accumulators' empty
+  // barriers one a warp of the epilogue, every other one a single one)
+  if (warp == 2) {
+    for (int i = lane; i < 4 * kMaxStages + 5; i += 32)
+      mbar_init(bar0 + 8u * i, i == 4 * kMaxStages + 2 || i == 4 * kMaxStages + 3 ? 2 * kEpiGroup / 32 : 1);
+    if (lane == 0) stop[0] = stop[1] = 0;
     fence_barrier_init();
+  }
+  if (threadIdx.x == 0) {
     tma_prefetch_desc(&ta0);
     tma_prefetch_desc(&tb);
     if (p.tma_out) tma_prefetch_desc(&to);
@@ -248,153 +251,193 @@ __global__ void __launch_bounds__(kGemmThreads, kOcc)
   __syncthreads();
   tc_fence_after();
   if (!p.late_trigger) griddep_launch();
-  const uint32_t tmem_base = *tmem_slot;
+  const uint32_t tmem_base = uniform(*tmem_slot);
 
-  int issued = 0;
-  if (warp == 0 && lane == 0) {
-    // ------------------------------------------------------------ TMA producer
+  if (warp == 0) {
+    // ------------------------------------------------------------ weight producer
     // a weight tile read by one CTA goes first; shared by token groups, it stays
-    const uint64_t pol_w = p.tok_groups > 1 ? policy_evict_normal() : policy_evict_first();
+    const uint64_t pol = p.tok_groups > 1 ? policy_evict_normal() : policy_evict_first();
     const uint64_t pol_x = policy_evict_last();
-    // the tile's tensor map (segment) and first row within it
-    const int seg = (p.nseg > 2 && tile >= p.seg_tile0[2]) ? 2 : (p.nseg > 1 && tile >= p.seg_tile0[1]) ? 1 : 0;
-    const CUtensorMap* amap = seg == 0 ? &ta0 : (seg == 1 ? &ta1 : &ta2);
-    const int arow = p.mode == EPI_SWIGLU ? tile * 64 : (tile - p.seg_tile0[seg]) * kTileRows;
-    auto load_a = [&](int i, uint32_t sa, uint32_t bar) {
-      const int kx = (kb0 + i) * G::BK;
-      if (p.mode == EPI_SWIGLU) {                  // 64 gate rows, then the 64 matching up rows
-        tma_load_2d(sa, &ta0, bar, kx, arow, pol_w);
-        tma_load_2d(sa + 64 * 128, &ta1, bar, kx, arow, pol_w);
+    const uint32_t bytes = w_bytes + (kTwoRings ? 0u : x_bytes);
+    auto load_w = [&](const GemmItem& w, int i, int s) {
+      const int kx = (w.kb0 + i) * G::BK;
+      const uint32_t dst = w0 + (uint32_t)s * w_bytes;
+      mbar_expect_tx(wfull(s), bytes);
+      if (p.mode == EPI_SWIGLU) {                  // the tile's gate rows, then the matching up rows
+        tma_load_2d(dst, &ta0, wfull(s), kx, w.row0 / 2, pol);
+        tma_load_2d(dst + w_bytes / 2, &ta1, wfull(s), kx, w.row0 / 2, pol);
       } else {
-        tma_load_2d(sa, amap, bar, kx, arow, pol_w);
+        tma_load_2d(dst, w.seg == 0 ? &ta0 : (w.seg == 1 ? &ta1 : &ta2), wfull(s), kx, w.row0, pol);
       }
     };
-    auto prefetch_a = [&](int i) {
-      if (group != 0) return;                // one CTA of the tile prefetches it
-      const int kx = (kb0 + i) * G::BK;
-      if (p.mode == EPI_SWIGLU) {
-        tma_prefetch_l2(&ta0, kx, arow);
-        tma_prefetch_l2(&ta1, kx, arow);
-      } else {
-        tma_prefetch_l2(amap, kx, arow);
+    auto load_x = [&](const GemmItem& w, int i, int s) {
+      tma_load_2d(x0 + (uint32_t)s * x_bytes, &tb, wfull(s), (w.kb0 + i) * G::BK, w.tok0, pol_x);
+    };
+    int s = 0, issued = 0;
+    uint32_t ph = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
+      const GemmItem w = gemm_item(p, item);
+      int i = 0;
+      if (!kTwoRings && issued == 0) {
+        // the first stages' weights go out before the preceding kernel is done: they do not depend on it
+        const int pre = min(SW, w.nk);
+        for (; i < pre; ++i) {
+          if (elect_one()) load_w(w, i, i);
+          __syncwarp();
+        }
+        griddep_wait();
+        if (p.late_trigger) griddep_launch();
+        for (i = 0; i < pre; ++i) {
+          if (elect_one()) load_x(w, i, i);
+          __syncwarp();
+        }
+        issued = pre;
+        s = pre % SW;
+        ph = (uint32_t)(pre / SW) & 1u;
       }
-    };
-    auto load_b = [&](int i, uint32_t sb, uint32_t bar) {
-      const int kx = (kb0 + i) * G::BK;
-      for (int tt = 0; tt < p.n_tok_tiles; ++tt)
-        tma_load_2d(sb + (uint32_t)(tt * p.bn * 128), &tb, bar, kx, tok0 + tt * p.bn, pol_x);
-    };
-    // Weights do not depend on the preceding kernel: start streaming them now
-    // (the first stages, and an L2 prefetch one k-block ahead of the ring).
-    int next_pf = 0;
-    const int pre = min(S, nk);
-    while (next_pf < min(kPrefetchDist, nk)) prefetch_a(next_pf++);
-    for (int i = 0; i < pre; ++i) {
-      mbar_expect_tx(full_bar(i), expect);
-      load_a(i, smem_u32(smem + (size_t)i * stage_bytes), full_bar(i));
+      for (; i < w.nk; ++i) {
+        if (issued >= SW && !gemm_wait(wempty(s), ph ^ 1u, stop, p.err)) { ok = false; break; }
+        if (elect_one()) {
+          load_w(w, i, s);
+          if (!kTwoRings) load_x(w, i, s);
+        }
+        __syncwarp();
+        ++issued;
+        if (++s == SW) { s = 0; ph ^= 1u; }
+      }
     }
-    griddep_wait();                       // activations come from the preceding kernel
+    // every load has landed before the CTA's shared memory goes away
+    for (int i = max(0, issued - SW); i < issued; ++i) mbar_wait(wfull(i % SW), (uint32_t)(i / SW) & 1u, p.err);
+  } else if (kTwoRings && warp == kXWarp) {
+    // ------------------------------------------------------------ activation producer
+    const uint64_t pol = policy_evict_last();
+    griddep_wait();                         // activations come from the preceding kernel
     // A late trigger lets the next kernel start only once every kernel before
     // this one has completed (it may then read their outputs before its own
     // wait, as the attention does with the view state).
     if (p.late_trigger) griddep_launch();
-    for (int i = 0; i < pre; ++i)
-      load_b(i, smem_u32(smem + (size_t)i * stage_bytes) + stage_a, full_bar(i));
-    issued = pre;
-    // stage and phase of k-block i advance by counters (no division per block)
-    int s = pre % S;
-    uint32_t ph = (uint32_t)(pre / S) & 1u;
-    const uint32_t ring0 = smem_u32(smem);
-    for (int i = pre; i < nk; ++i) {
-      while (next_pf < nk && next_pf < i + kPrefetchDist) prefetch_a(next_pf++);
-      if (!mbar_wait(empty_bar(s), ph ^ 1u, p.err)) { *s_abort = 1; break; }
-      mbar_expect_tx(full_bar(s), expect);
-      const uint32_t sa = ring0 + (uint32_t)s * stage_bytes;
-      load_a(i, sa, full_bar(s));
-      load_b(i, sa + stage_a, full_bar(s));
-      issued = i + 1;
-      if (++s == S) { s = 0; ph ^= 1u; }
-    }
-  } else if (warp == 1 && lane == 0) {
-    // ------------------------------------------------------------ MMA issue
-    // One thread issues every MMA, so its own instructions set the issue rate
-    // (measured: 0.60 -> 0.24 us per k-block with the loop below): the two
-    // descriptors are formed once per stage and stepped by the byte offset
-    // >> 4 in their address field (offsets stay inside the stage, so the
-    // field never carries), and the stage and phase advance by counters.
-    const uint32_t idesc = make_idesc(p.bn, G::FMT);
-    const uint32_t ring0 = smem_u32(smem);
-    const bool one_tile = p.n_tok_tiles == 1;
-    int s = 0;
+    int s = 0, issued = 0;
     uint32_t ph = 0;
-    for (int i = 0; i < nk; ++i) {
-      if (!mbar_wait(full_bar(s), ph, p.err)) { *s_abort = 1; break; }
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x) {
+      const GemmItem w = gemm_item(p, item);
+      for (int i = 0; i < w.nk; ++i) {
+        if (issued >= SX && !gemm_wait(xempty(s), ph ^ 1u, stop, p.err)) { ok = false; break; }
+        if (elect_one()) {
+          mbar_expect_tx(xfull(s), x_bytes);
+          tma_load_2d(x0 + (uint32_t)s * x_bytes, &tb, xfull(s), (w.kb0 + i) * G::BK, w.tok0, pol);
+        }
+        __syncwarp();
+        ++issued;
+        if (++s == SX) { s = 0; ph ^= 1u; }
+      }
+    }
+    for (int i = max(0, issued - SX); i < issued; ++i) mbar_wait(xfull(i % SX), (uint32_t)(i / SX) & 1u, p.err);
+  } else if (warp == 1) {
+    // ------------------------------------------------------------ MMA issue
+    // The whole warp walks the k-blocks and one lane issues: descriptors formed
+    // once per stage and stepped by the byte offset >> 4 in their address field
+    // (offsets stay inside the stage, so the field never carries), stage and
+    // phase by counters, everything uniform (see elect_one).  The MMAs of a
+    // k-block issue in 200 cycles a token tile instead of 500.
+    const uint32_t idesc = make_idesc(p.width, G::FMT);
+    const bool two = p.tok_tiles == 2;
+    const uint64_t xd1 = (uint64_t)((p.tile_tok * 128) >> 4);
+    int s = 0, sx = 0, n = 0;
+    uint32_t ph = 0, phx = 0;
+    bool ok = true;
+    for (int item = blockIdx.x; item < p.items && ok; item += gridDim.x, ++n) {
+      const GemmItem w = gemm_item(p, item);
+      const int a = n % p.n_acc;
+      if (n >= p.n_acc) ok = gemm_wait(acc_empty(a), (uint32_t)(n / p.n_acc - 1) & 1u, stop, p.err);
       tc_fence_after();
-      const uint32_t sa = ring0 + (uint32_t)s * stage_bytes;
-      const uint64_t ad0 = sdesc_sw128(sa), bd0 = sdesc_sw128(sa + stage_a);
-      if (one_tile) {
+      const uint32_t d0 = tmem_base + (uint32_t)(a * p.acc_cols), d1 = d0 + (uint32_t)p.tile_cols;
+      bool ready = false;
+      for (int i = 0; i < w.nk; ++i) {
+        if (!ready) ok = (!kTwoRings || gemm_wait(xfull(sx), phx, stop, p.err)) && gemm_wait(wfull(s), ph, stop, p.err);
+        if (!ok) break;
+        const uint64_t xd = sdesc_sw128(x0 + (uint32_t)sx * x_bytes), wd = sdesc_sw128(w0 + (uint32_t)s * w_bytes);
+        auto tile = [&](uint32_t d, uint64_t x) {
 #pragma unroll
-        for (int kk = 0; kk < G::BK / G::UK; ++kk) {
-          const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-          if constexpr (sizeof(T) == 2)
-            umma_f16(tmem_base, ad0 + (uint64_t)(2 * kk), bd0 + (uint64_t)(2 * kk), idesc, acc);
-          else
-            umma_tf32(tmem_base, ad0 + (uint64_t)(2 * kk), bd0 + (uint64_t)(2 * kk), idesc, acc);
+          for (int kk = 0; kk < G::BK / G::UK; ++kk) {
+            const uint32_t keep = (i > 0 || kk > 0) ? 1u : 0u;
+            if constexpr (sizeof(T) == 2) umma_f16(d, x + (uint64_t)(2 * kk), wd + (uint64_t)(2 * kk), idesc, keep);
+            else umma_tf32(d, x + (uint64_t)(2 * kk), wd + (uint64_t)(2 * kk), idesc, keep);
+          }
+        };
+        const int s1 = s + 1 == SW ? 0 : s + 1, sx1 = sx + 1 == SX ? 0 : sx + 1;
+        const uint32_t ph1 = s1 ? ph : ph ^ 1u, phx1 = sx1 ? phx : phx ^ 1u;
+        if (elect_one()) {
+          tile(d0, xd);
+          if (two) tile(d1, xd + xd1);
+        }
+        __syncwarp();
+        // is the next k-block here already?  (asked while these MMAs are queued: a
+        // wait that succeeds at once still takes about 80 cycles)
+        const bool rx = !kTwoRings || mbar_test_wait(xfull(sx1), phx1), rw = mbar_test_wait(wfull(s1), ph1);
+        if (elect_one()) {
+          umma_commit(wempty(s));
+          if (kTwoRings) umma_commit(xempty(sx));
+        }
+        __syncwarp();
+        ready = rx && rw;
+        s = s1; ph = ph1;
+        sx = sx1; phx = phx1;
+      }
+      if (elect_one()) umma_commit(acc_full(a));
+      __syncwarp();
+    }
+    if (!ok) {                              // no MMA outlives the CTA's shared memory and TMEM
+      if (elect_one()) umma_commit(end_bar);
+      __syncwarp();
+      mbar_wait(end_bar, 0, p.err);
+    }
+  } else {
+    // ------------------------------------------------------------ epilogue
+    const int grp = (warp - 2) >> 2, q = warp & 3, row = q * 32 + lane;
+    const bool two = p.tok_tiles == 2;
+    uint8_t* stg = smem + p.off_stg + (size_t)grp * p.n_stg * kChunkBytes;
+    griddep_wait();
+    int n = 0, chunks = 0;
+    for (int item = blockIdx.x; item < p.items; item += gridDim.x, ++n) {
+      const GemmItem w = gemm_item(p, item);
+      const int a = n % p.n_acc;
+      gemm_wait(acc_full(a), (uint32_t)(n / p.n_acc) & 1u, stop, p.err);
+      tc_fence_after();
+      // one thread's view of `stop` (which another role may set at any time), so
+      // that every warp of a barrier takes the same branch
+      named_bar(3, 2 * kEpiGroup);
+      if (warp == 2 && lane == 0) stop[1] = *stop;
+      named_bar(3, 2 * kEpiGroup);
+      if (stop[1]) break;
+      const int t = two ? grp : 0;
+      const uint32_t acc = tmem_base + ((uint32_t)(q * 32) << 16) + (uint32_t)(a * p.acc_cols + t * p.tile_cols);
+      if (p.mode == EPI_SWIGLU) {
+        // (one item a CTA: the ring is idle once its MMAs are done)
+        const int fw = p.width / 2;
+        uint8_t* tile = smem + (size_t)t * p.stg_tile;
+        swiglu_row<T>(acc, smem_u32(tile) + (uint32_t)(row * fw) * (uint32_t)sizeof(T), fw, two ? 0 : grp, two ? 1 : 2,
+                      row < p.tile_tok);
+        fence_proxy_async_smem();
+        named_bar(3, 2 * kEpiGroup);
+        const int tok = w.tok0 + t * p.tile_tok;
+        if (row == 0 && (two || grp == 0) && tok < p.M) {
+          tma_store_3d(&to, smem_u32(tile), w.row0 / 2, tok, 0);
+          bulk_commit();
         }
       } else {
-#pragma unroll
-        for (int kk = 0; kk < G::BK / G::UK; ++kk) {
-          const uint64_t ad = ad0 + (uint64_t)((kk * 32) >> 4);
-          for (int tt = 0; tt < p.n_tok_tiles; ++tt) {
-            const uint64_t bd = bd0 + (uint64_t)((tt * p.bn * 128 + kk * 32) >> 4);
-            const uint32_t acc = (i > 0 || kk > 0) ? 1u : 0u;
-            if constexpr (sizeof(T) == 2)
-              umma_f16(tmem_base + (uint32_t)(tt * p.bn), ad, bd, idesc, acc);
-            else
-              umma_tf32(tmem_base + (uint32_t)(tt * p.bn), ad, bd, idesc, acc);
-          }
-        }
+        epilogue_f32(p, &to, stg, p.n_stg, chunks, acc, w, w.tok0 + t * p.tile_tok, two ? 0 : grp, two ? 1 : 2, row, 1 + grp);
       }
-      umma_commit(empty_bar(s));
-      if (++s == S) { s = 0; ph ^= 1u; }
+      tc_fence_before();
+      __syncwarp();
+      if (lane == 0) mbar_arrive(acc_empty(a));
     }
-    umma_commit(acc_bar);
-  } else if (warp >= 2) {
-    // ------------------------------------------------------------ epilogue
-    const int q = warp & 3;
-    const int r = q * 32 + lane;
-    float* xchg = reinterpret_cast<float*>(smem);   // pipeline smem is idle once acc_bar fired
-    griddep_wait();
-    const bool ok = mbar_wait(acc_bar, 0, p.err);
-    if (!ok) *s_abort = 1;
-    tc_fence_after();
-    named_bar(1, kEpilogueThreads);
-    // one thread's snapshot of s_abort (which another role may set at any
-    // time), so that all four warps take the same branch below
-    volatile int* s_stop = s_abort + 1;
-    if (r == 0) *s_stop = *s_abort;
-    named_bar(1, kEpilogueThreads);
-    const bool go = *s_stop == 0;
-    const uint32_t lane_base = tmem_base + ((uint32_t)(q * 32) << 16);
-    if (go && p.tma_out) {
-      epilogue_tma<T>(p, &to, smem, lane_base, tile, tok0, split, r);
-    } else if (go) {
-      for (int tt = 0; tt < p.n_tok_tiles; ++tt)
-        for (int c0 = 0; c0 < p.bn; c0 += 16) {
-          float v[16];
-          tmem_ld16(lane_base + (uint32_t)(tt * p.bn + c0), v);
-          emit_chunk<T>(p, tile, split, r, tok0 + tt * p.bn + c0, v, xchg);
-        }
-    }
+    if (row == 0) bulk_wait_read<0>();                          // staging smem is released at exit
   }
 
   tc_fence_before();
   __syncthreads();
-  if (warp == 0 && lane == 0 && *s_abort) {
-    // A wait gave up: let every TMA copy this CTA issued land before exit.
-    for (int i = (issued > S ? issued - S : 0); i < issued; ++i)
-      mbar_wait(full_bar(i % S), (uint32_t)(i / S) & 1u, p.err);
-  }
   if (warp == 1) {
     tc_fence_after();
     tmem_dealloc(tmem_base, (uint32_t)p.tmem_cols);
@@ -465,8 +508,9 @@ int tmap_2d_bf16_sw128(CUtensorMap* m, const void* ptr, uint64_t inner, uint64_t
 }
 
 // [splits][M][N] view of the output (row stride ldy) for TMA stores of
-// box (cols features, tok tokens, 1 split); no swizzle.
-static int make_out_map(CUtensorMap* m, bool f32, const void* Y, int N, int M, int splits, int ldy,
+// box (cols features, tok tokens, 1 split); swizzled: 128-byte rows staged with
+// the 128-byte swizzle, else rows as they are.
+static int make_out_map(CUtensorMap* m, bool f32, bool swizzled, const void* Y, int N, int M, int splits, int ldy,
                         int cols, int tok) {
   auto enc = encoder();
   if (!enc) return LSP_ERR_UNSUPPORTED;
@@ -478,10 +522,12 @@ static int make_out_map(CUtensorMap* m, bool f32, const void* Y, int N, int M, i
   cuuint32_t estr[3] = {1, 1, 1};
   CUresult r = enc(m, f32 ? CU_TENSOR_MAP_DATA_TYPE_FLOAT32 : CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, 3,
                    const_cast<void*>(Y), dims, strides, box, estr, CU_TENSOR_MAP_INTERLEAVE_NONE,
-                   CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
+                   swizzled ? CU_TENSOR_MAP_SWIZZLE_128B : CU_TENSOR_MAP_SWIZZLE_NONE, CU_TENSOR_MAP_L2_PROMOTION_NONE,
                    CU_TENSOR_MAP_FLOAT_OOB_FILL_NONE);
   return r == CUDA_SUCCESS ? LSP_OK : LSP_ERR_CUDA;
 }
+
+static constexpr int kSmemBudget = 227 * 1024;
 
 int gemm_tiles(int mode, const int* seg_rows, int nseg) {
   if (mode == EPI_SWIGLU) return (seg_rows[0] + 63) / 64;
@@ -507,47 +553,30 @@ int gemm_group_rows(int M, int G) {
   return bn * ntt;
 }
 
-static constexpr int kSmemBudget = 227 * 1024;
 
-// Two 2-stage CTAs per SM keep the tensor pipe fed from two MMA issuers and
-// overlap one CTA's prologue/epilogue with the other's weight stream; the pair
-// must fit one SM's shared memory and TMEM.
+// ---- split-K factor.  The k ranges decide the order of the fp32 sums, so their
+// rule is fixed: it is the cost model of a kernel with one 128-row weight tile
+// a CTA (16 KB of weights a stage; two or three CTAs an SM where their rings and
+// accumulators fit), which gives the short projections enough CTAs for this
+// one as well.
+constexpr int kSplitTileBytes = kTileRows * 128;
+
 static bool two_per_sm_fits(int m_pad) {
-  const int stage_bytes = (int)kTileBytes + m_pad * 128;
+  const int stage_bytes = kSplitTileBytes + m_pad * 128;
   return 2 * stage_bytes + 2048 <= kSmemBudget / 2 && 2 * m_pad <= 512;
 }
 
-static bool use_two_per_sm(long long ctas, int num_sms, int m_pad) {
-  return ctas * 4 >= (long long)num_sms * 5 && two_per_sm_fits(m_pad);
-}
-
-// Three 2-stage CTAs per SM (shared memory incl. the 1 KB each CTA reserves,
-// TMEM columns, and the kernel instance bounded to 3 x 192 threads' registers)
-// when token groups give enough CTAs for most SMs to hold a third.
 constexpr int kSmemPerSm = 228 * 1024;
 static bool three_per_sm_fits(int m_pad, int groups) {
   if (groups < 2) return false;
   int cols = 32;
   while (cols < m_pad) cols *= 2;
-  const int stage_bytes = (int)kTileBytes + m_pad * 128;
+  const int stage_bytes = kSplitTileBytes + m_pad * 128;
   return 3 * (2 * stage_bytes + 1280 + 1024) <= kSmemPerSm && 3 * cols <= 512;
 }
 
-static bool use_three_per_sm(long long ctas, int num_sms, int m_pad, int groups) {
-  return ctas >= 2LL * num_sms && three_per_sm_fits(m_pad, groups);
-}
-
-// Token groups: the CTAs of a weight tile split the M tokens G ways (each
-// streams the tile; the copies after the first come from L2).  Smaller stages
-// let three CTAs share an SM.  Two groups for the SwiGLU gate/up projection
-// when its tiles fill at least one wave of one CTA per SM but less than one
-// of two and the token count allows it (Qwen3-8B round, M = 256, 192 tiles:
-// gate/up 368 -> 359 us per round, round 1.243 -> 1.231 ms).  Two groups for
-// every projection above 256 tokens (the large shape, M = 512: round 2600 ->
-// 2485 us), where one group would need a 512-column accumulator, one CTA per
-// SM and two 80 KB stages.  One otherwise (at M = 256 every other projection
-// and the LM head measured slower with two or three: more CTAs re-stream each
-// weight tile for the same work).
+// Token groups of the model: two above 256 tokens, and for a gate/up projection
+// whose tiles fill at least one wave of one CTA per SM but less than one of two.
 static int token_groups(int M, int mode, int n_tiles, int num_sms) {
   const int g = (M > 256 || (mode == EPI_SWIGLU && M >= 128 && n_tiles <= 2 * num_sms && n_tiles >= num_sms)) ? 2 : 1;
   if (g == 1) return 1;
@@ -556,12 +585,10 @@ static int token_groups(int M, int mode, int n_tiles, int num_sms) {
   return (g - 1) * bn * ntt < M ? g : 1;     // every group holds at least one token row
 }
 
-// Split-K factor from a cost model in units of one k-block of one of two
-// co-resident CTAs (~0.8 us measured at M = 256): waves x (k-blocks per CTA +
-// fixed per-CTA cost) + the cost of combining the splits (per_split_cost per
-// split: the consumer's re-read of fp32 partials from L2).  A lone CTA on an
-// SM, with its deeper ring, moves a k-block in 0.53 of that time (0.42 vs
-// 0.80 us measured at M = 256 with the MMA issue loop at 0.24 us per k-block).
+// In units of one k-block of one of two co-resident CTAs (~0.8 us at M = 256):
+// waves x (k-blocks per CTA + fixed per-CTA cost) + the cost of combining the
+// splits (per_split_cost per split: the consumer's re-read of fp32 partials
+// from L2).  A lone CTA on an SM moves a k-block in 0.53 of that time.
 constexpr double kLoneCtaCost = 0.53;
 
 int gemm_auto_splits(int n_ctas, int kblocks, int num_sms, double per_split_cost, int max_splits,
@@ -601,96 +628,173 @@ void gemm_choose(int dtype, int M, int K, int n_tiles, int mode, int num_sms, in
   *splits = std::max(1, std::min(*splits, kblocks));
 }
 
+
+// ---- tiling of a launch: weight rows per tile, and how CTAs walk the items
+struct Tiling {
+  int width, tiles, w_stages, x_stages, persistent;
+};
+
+static constexpr int kBarBytes = 384;
+
+// Bytes an epilogue keeps for itself where CTAs walk several items (two
+// groups, one chunk buffer each); with one item it stages in the idle rings.
+static constexpr int kStgBytes = 2 * (int)kChunkBytes;
+
+// Stages in the shared memory left.  Up to 128 tokens a stage holds both tiles;
+// above, activations take 3 stages (2 where weights would get fewer than 4).
+static void ring_stages(int width, int m_pad, bool persistent, int* w, int* x) {
+  const int room = (kSmemBudget - 1024 - kBarBytes - (persistent ? kStgBytes : 0)) / 128;
+  if (m_pad <= kTileTok) {
+    *w = *x = std::min(kMaxStages, room / (width + m_pad));
+    return;
+  }
+  for (*x = 3; *x > 2 && (room - *x * m_pad) / width < 4; --*x) {}
+  *w = std::min(kMaxStages, (room - *x * m_pad) / width);
+}
+
+// Time of one launch in ns for a tile width, from what was measured on the
+// GB300.  A k-block takes the longest of: the SM's intake (115 B/ns), its share
+// of HBM (6.4 KB/ns over all CTAs), its MMAs (width / 2 cycles, at least 50, for
+// each of four steps and each token tile) with 150 cycles of waits and commits,
+// and the round trip of a stage (2 us) over the weight stages.  A CTA costs
+// about 2 us to start; writing an item out takes 0.7 us and 0.35 us a 32-feature
+// chunk (a burst of all CTAs), under the next item's MMAs where a walk has two accumulator
+// sets, partly exposed where it has one.
+static double tiling_cost(int width, int m_pad, int tok_tiles, int kblocks, long long items, int num_sms, int stages,
+                          bool persistent) {
+  const double in = (width + m_pad) * 128.0 / 115.0;
+  const double hbm = width * 128.0 * (double)std::min<long long>(items, num_sms) / 6400.0;
+  const double mma = (tok_tiles * 4 * std::max(width / 2, 50) + 150) / 1.9, trip = 2000.0 / stages;
+  const double kb = kblocks * std::max(std::max(in, hbm), std::max(mma, trip));
+  const double waves = (double)((items + num_sms - 1) / num_sms), out = 700.0 + 11.0 * width;
+  if (!persistent) return waves * (kb + 2000.0 + out);
+  const bool two_sets = 2 * tok_tiles * ((width + 31) / 32 * 32) <= 512;
+  return (two_sets ? waves * std::max(kb, out) : waves * kb + (waves - 1) * 0.6 * out) + 2000.0 + out;
+}
+
+// The tile width with the least modelled time: multiples of 32 up to 256 weight
+// rows (a chunk of the epilogue is 32), for gate/up twice an odd multiple of
+// eight features.  CTAs walk the items where these make more than one wave.
+static Tiling choose_width(int mode, const int* seg_rows, int nseg, int m_pad, int tok_tiles, int groups, int splits,
+                           int kblocks, int num_sms) {
+  Tiling best = {};
+  double cost = 1e30;
+  const bool gu = mode == EPI_SWIGLU;
+  const int kb = (kblocks + splits - 1) / splits;
+  for (int width = gu ? 16 : 32; width <= 256; width += 32) {
+    int tiles = 0;
+    for (int i = 0; i < (gu ? 1 : nseg); ++i) tiles += (seg_rows[i] + (gu ? width / 2 : width) - 1) / (gu ? width / 2 : width);
+    const long long items = (long long)tiles * groups * splits;
+    const bool persistent = !gu && items > num_sms;
+    int ws, xs;
+    ring_stages(width, m_pad, persistent, &ws, &xs);
+    if (ws < 2) continue;
+    const double c = tiling_cost(width, m_pad, tok_tiles, kb, items, num_sms, ws, persistent);
+    if (c < cost - 1e-9) {
+      cost = c;
+      best = {width, tiles, ws, xs, persistent};
+    }
+  }
+  return best;
+}
+
 int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* const* W,
               const int* seg_rows, int nseg, int mode, void* Y, int ldy, unsigned* err,
               int num_sms, int splits) {
   if (M < 1 || M > 512 || K < 1 || nseg < 1 || nseg > 3) return LSP_ERR_SHAPE;
-  if (mode == EPI_SWIGLU && nseg != 2) return LSP_ERR_SHAPE;
+  const bool gu = mode == EPI_SWIGLU;
+  if (gu && nseg != 2) return LSP_ERR_SHAPE;
   const int es = dtype == LSP_DTYPE_BF16 ? 2 : 4;
   if ((K * es) % 16) return LSP_ERR_SHAPE;
-  for (int i = 0; i + 1 < nseg && mode != EPI_SWIGLU; ++i)
+  for (int i = 0; i + 1 < nseg && !gu; ++i)
     if (seg_rows[i] % kTileRows) return LSP_ERR_SHAPE;
   GemmParams& p = op->p;
   p = GemmParams{};
   p.M = M;
   p.K = K;
   p.mode = mode;
-  p.nseg = nseg;
-  p.n_tiles = gemm_tiles(mode, seg_rows, nseg);
-  p.N = 0;
-  if (mode == EPI_SWIGLU) {
-    p.N = seg_rows[0];
-  } else {
-    int t0 = 0;
-    for (int i = 0; i < 3; ++i) {
-      p.seg_tile0[i] = i < nseg ? t0 : p.n_tiles;
-      if (i < nseg) t0 += (seg_rows[i] + kTileRows - 1) / kTileRows;
-    }
-    for (int i = 0; i < nseg; ++i) p.N += seg_rows[i];
-  }
+  p.nseg = gu ? 1 : nseg;
   p.kblocks = gemm_kblocks(K, dtype);
-  int G = 1;
-  gemm_choose(dtype, M, K, p.n_tiles, mode, num_sms, &splits, &G);
-  p.tok_groups = G;
-  token_tiling((M + G - 1) / G, &p.bn, &p.n_tok_tiles);      // per token group
-  p.m_pad = p.bn * p.n_tok_tiles;
-  if (p.m_pad > 512) return LSP_ERR_SHAPE;
-  int cols = 32;
-  while (cols < p.m_pad) cols *= 2;
-  p.tmem_cols = cols;
-  const int stage_bytes = (int)kTileBytes + p.m_pad * 128;
-  p.stages = std::min(8, (kSmemBudget - 2048) / stage_bytes);
-  const int n_ctas = p.n_tiles * G;
-  op->occ = 1;
-  if (use_three_per_sm((long long)n_ctas * splits, num_sms, p.m_pad, G)) {
-    p.stages = 2;
-    op->occ = 3;
-  } else if (use_two_per_sm((long long)n_ctas * splits, num_sms, p.m_pad)) {
-    p.stages = 2;
-  }
-  if (p.stages < 2) return LSP_ERR_SHAPE;
-  p.splits = splits;
+  gemm_choose(dtype, M, K, gemm_tiles(mode, seg_rows, nseg), mode, num_sms, &splits);
   if (splits > 1 && mode != EPI_PARTIAL) return LSP_ERR_SHAPE;
+  p.splits = splits;
+  // up to 256 tokens a CTA, in one or two accumulators of at most 128
+  p.tok_groups = M > 256 ? 2 : 1;
+  p.m_pad = ((M + p.tok_groups - 1) / p.tok_groups + 15) / 16 * 16;
+  p.tok_tiles = p.m_pad > kTileTok ? 2 : 1;
+  p.tile_tok = p.m_pad / p.tok_tiles;
+  const Tiling t = choose_width(mode, seg_rows, nseg, p.m_pad, p.tok_tiles, p.tok_groups, splits, p.kblocks, num_sms);
+  if (t.w_stages < 2) return LSP_ERR_SHAPE;
+  p.width = t.width;
+  p.n_tiles = t.tiles;
+  p.w_stages = t.w_stages;
+  p.x_stages = t.x_stages;
+  p.items = t.tiles * p.tok_groups * splits;
+  for (int i = 0, tile = 0; i < p.nseg; ++i) {
+    p.seg_tile0[i] = tile;
+    p.seg_rows[i] = gu ? 2 * seg_rows[i] : seg_rows[i];
+    p.seg_col0[i] = p.N;
+    tile += (p.seg_rows[i] + p.width - 1) / p.width;
+    p.N += seg_rows[i];
+  }
+  // accumulators: one set of tok_tiles x width columns, or two where a walk over
+  // several items can alternate between them
+  p.tile_cols = (p.width + 31) / 32 * 32;
+  p.acc_cols = p.tok_tiles * p.tile_cols;
+  p.n_acc = t.persistent && 2 * p.acc_cols <= 512 ? 2 : 1;
+  p.tmem_cols = 32;
+  while (p.tmem_cols < p.n_acc * p.acc_cols) p.tmem_cols *= 2;
   p.Y = Y;
   p.ldy = ldy;
   p.err = err;
   op->dtype = dtype;
-  const int box_rows = mode == EPI_SWIGLU ? 64 : kTileRows;
+  // shared memory: activation ring | weight ring | staging of a walk | barriers;
+  // an accumulator of fewer than 128 tokens reads past its activation tile
+  // (lanes nobody looks at), into the weight ring or what follows
+  const int ring = (p.w_stages * p.width + p.x_stages * p.m_pad) * 128;
+  p.off_stg = t.persistent ? ring : 0;
+  p.n_stg = t.persistent ? 1 : std::max(1, std::min(4, ring / kStgBytes));
+  p.stg_tile = (p.tile_tok * (p.width / 2) * es + 127) / 128 * 128;
+  if (gu && p.tok_tiles * p.stg_tile > ring) return LSP_ERR_SHAPE;
+  p.off_bar = std::max(ring + (t.persistent ? kStgBytes : 0), (p.x_stages * p.m_pad - p.tile_tok + kTileTok) * 128);
+  if (!gu && !t.persistent) p.off_bar = std::max(p.off_bar, p.n_stg * kStgBytes);
+  op->smem = (size_t)p.off_bar + kBarBytes + 1024;
+  if (op->smem > (size_t)kSmemBudget) return LSP_ERR_SHAPE;
+  op->grid = dim3((unsigned)(t.persistent ? num_sms : p.items), 1, 1);
   int rc;
+  const int box = gu ? p.width / 2 : p.width;
   for (int i = 0; i < 3; ++i) {
     const int si = i < nseg ? i : 0;
-    if ((rc = make_map(&op->a[i], dtype, W[si], K, seg_rows[si], box_rows)) != LSP_OK) return rc;
+    if ((rc = make_map(&op->a[i], dtype, W[si], K, seg_rows[si], box)) != LSP_OK) return rc;
   }
-  if ((rc = make_map(&op->b, dtype, X, K, M, p.bn)) != LSP_OK) return rc;
+  if ((rc = make_map(&op->b, dtype, X, K, M, p.m_pad)) != LSP_OK) return rc;
   // TMA-store epilogue when the output view can be described (else per-thread stores)
-  p.out_tok = (p.m_pad % 32) ? 16 : 32;
-  {
-    const bool f32 = mode == EPI_F32 || mode == EPI_PARTIAL || dtype == LSP_DTYPE_F32;
-    const int cols = mode == EPI_SWIGLU ? 64 : kTileRows;
-    p.tma_out = make_out_map(&op->out, f32, Y, p.N, M, splits, ldy, cols, p.out_tok) == LSP_OK;
+  if (gu) {
+    if ((rc = make_out_map(&op->out, dtype == LSP_DTYPE_F32, false, Y, p.N, M, 1, ldy, p.width / 2, p.tile_tok)) != LSP_OK)
+      return rc;
+    p.tma_out = 1;
+  } else {
+    p.tma_out = make_out_map(&op->out, true, true, Y, p.N, M, splits, ldy, kChunk, p.tile_tok) == LSP_OK;
     if (!p.tma_out) op->out = op->b;       // unused placeholder
   }
-  op->grid = dim3((unsigned)n_ctas, (unsigned)splits, 1);
-  op->smem = (size_t)p.stages * stage_bytes + 1024 + 256;
   return LSP_OK;
 }
 
-template <typename T, int kOcc>
+template <typename T, bool kTwoRings>
 static int launch_t(const GemmOp* op, cudaStream_t s) {
   static std::once_flag once;
   std::call_once(once, [] {
-    cudaFuncSetAttribute(gemm_kernel<T, kOcc>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-    if (kOcc > 1)   // room for kOcc CTAs' shared memory on one SM
-      cudaFuncSetAttribute(gemm_kernel<T, kOcc>, cudaFuncAttributePreferredSharedMemoryCarveout, 100);
+    cudaFuncSetAttribute(gemm_kernel<T, kTwoRings>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
   });
-  const cudaError_t e = launch_pdl(gemm_kernel<T, kOcc>, op->grid, dim3(kGemmThreads), op->smem, s,
-                                   op->a[0], op->a[1], op->a[2], op->b, op->out, op->p);
+  const cudaError_t e = launch_pdl(gemm_kernel<T, kTwoRings>, op->grid, dim3(kTwoRings ? kGemmThreads : kGemmThreads - 32),
+                                   op->smem, s, op->a[0], op->a[1], op->a[2], op->b, op->out, op->p);
   return e == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
 }
 
 int gemm_launch(const GemmOp* op, cudaStream_t s) {
-  if (op->occ == 3) return op->dtype == LSP_DTYPE_BF16 ? launch_t<bf16, 3>(op, s) : launch_t<float, 3>(op, s);
-  return op->dtype == LSP_DTYPE_BF16 ? launch_t<bf16, 1>(op, s) : launch_t<float, 1>(op, s);
+  const bool two = op->p.tok_tiles == 2;
+  if (op->dtype == LSP_DTYPE_BF16) return two ? launch_t<bf16, true>(op, s) : launch_t<bf16, false>(op, s);
+  return two ? launch_t<float, true>(op, s) : launch_t<float, false>(op, s);
 }
 
 int launch_sum_partials(const float* part, int splits, size_t n, float* y, cudaStream_t s) {

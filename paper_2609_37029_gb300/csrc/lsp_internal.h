@@ -33,24 +33,25 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
 // ------------------------------------------------------------------ GEMM
 enum EpiMode {
   EPI_F32 = 0,      // Y (float) = acc
-  EPI_T = 1,        // Y (dtype) = acc
-  EPI_PARTIAL = 2,  // Y (float) [split][M][ldy] = this split's partial sum (the consumer adds)
-  EPI_SWIGLU = 3,   // Y (dtype) = silu(acc_gate) * acc_up
+  EPI_PARTIAL = 1,  // Y (float) [split][M][ldy] = this split's partial sum (the consumer adds)
+  EPI_SWIGLU = 2,   // Y (dtype) = silu(acc_gate) * acc_up
 };
 
-constexpr int kGemmThreads = 192;   // warp 0 TMA, warp 1 MMA, warps 2-5 epilogue
-constexpr int kTileRows = 128;      // weight rows per tile (UMMA M)
+constexpr int kGemmThreads = 352;   // warp 0 weights, warp 1 MMA, warps 2-9 epilogue, warp 10 activations
+constexpr int kTileRows = 128;      // weight rows of a tile in the split model
 
 struct GemmParams {
   int M, N, K;          // token rows, output features, reduction length
-  int kblocks, splits, n_tiles;
+  int kblocks, splits;
   int mode;
-  int seg_tile0[3];     // first tile index of each A segment
+  int width;            // weight rows of a tile (EPI_SWIGLU: half gate, half up)
+  int n_tiles, tok_groups, items;   // items = tiles x token groups x splits
   int nseg;
-  int bn, n_tok_tiles, m_pad, stages, tmem_cols;
-  int tma_out;          // 1: the epilogue stages tiles in shared memory and TMA-stores them
-  int out_tok;          // tokens per staged output chunk (16 or 32)
-  int tok_groups;       // CTAs per weight tile, each over m_pad consecutive tokens
+  int seg_tile0[3], seg_rows[3], seg_col0[3];   // first tile, weight rows and first output feature of a segment
+  int m_pad, tok_tiles, tile_tok;   // token rows of a group, its accumulators, token rows of one
+  int w_stages, x_stages, tmem_cols, tile_cols, acc_cols, n_acc;   // TMEM columns of a tile and of an accumulator set; sets
+  int off_stg, n_stg, stg_tile, off_bar;   // shared memory: staging (buffers a group), SwiGLU tile bytes, barriers
+  int tma_out;          // 1: chunks leave by TMA stores (else by per-thread stores)
   int late_trigger;     // 1: let the next kernel launch only after this one's dependency wait
   void* Y;
   int ldy;
@@ -64,7 +65,6 @@ struct GemmOp {
   GemmParams p;
   int dtype;
   dim3 grid;
-  int occ;              // CTAs per SM the plan sizes for: 3 picks the register-bounded instance
   size_t smem;
 };
 
