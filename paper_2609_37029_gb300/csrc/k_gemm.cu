@@ -444,14 +444,34 @@ __global__ void __launch_bounds__(kTwoRings ? kGemmThreads : kGemmThreads - 32, 
   }
 }
 
-__global__ void sum_partials_kernel(const float* __restrict__ part, int splits, size_t n,
-                                    float* __restrict__ y) {
+// y[i] = part[0][i] + part[1][i] + ... in split order.  Every split's load of a
+// thread is in flight at once (a loop of dependent loads paid the L2 latency for
+// each split: 3.5 us more at 7 x 4096 outputs and 9 splits), four outputs a thread where
+// the split stride keeps float4 alignment.
+template <typename V>
+__device__ __forceinline__ V add_vec(const V& a, const V& b);
+template <>
+__device__ __forceinline__ float add_vec(const float& a, const float& b) { return a + b; }
+template <>
+__device__ __forceinline__ float4 add_vec(const float4& a, const float4& b) {
+  return make_float4(a.x + b.x, a.y + b.y, a.z + b.z, a.w + b.w);
+}
+
+template <typename V>
+__global__ void __launch_bounds__(256) sum_partials_kernel(const V* __restrict__ part, int splits, size_t n, V* __restrict__ y) {
   griddep_launch();
   griddep_wait();
-  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n;
-       i += (size_t)gridDim.x * blockDim.x) {
-    float acc = part[i];
-    for (int s = 1; s < splits; ++s) acc += part[(size_t)s * n + i];
+  for (size_t i = blockIdx.x * (size_t)blockDim.x + threadIdx.x; i < n; i += (size_t)gridDim.x * blockDim.x) {
+    V acc = part[i];
+    for (int s0 = 1; s0 < splits; s0 += 8) {
+      V v[8];
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s0 + u < splits) v[u] = __ldcs(part + (size_t)(s0 + u) * n + i);
+#pragma unroll
+      for (int u = 0; u < 8; ++u)
+        if (s0 + u < splits) acc = add_vec(acc, v[u]);
+    }
     y[i] = acc;
   }
 }
@@ -798,11 +818,13 @@ int gemm_launch(const GemmOp* op, cudaStream_t s) {
 }
 
 int launch_sum_partials(const float* part, int splits, size_t n, float* y, cudaStream_t s) {
-  const unsigned blocks = (unsigned)std::min<size_t>((n + 255) / 256, 4096);
-  return launch_pdl(sum_partials_kernel, dim3(blocks), dim3(256), 0, s, part, splits, n, y) ==
-                 cudaSuccess
-             ? LSP_OK
-             : LSP_ERR_CUDA;
+  const bool vec = n % 4 == 0 && (((uintptr_t)part | (uintptr_t)y) & 15) == 0;
+  const size_t m = vec ? n / 4 : n;
+  const dim3 blocks((unsigned)std::min<size_t>((m + 255) / 256, 4096));
+  const cudaError_t e = vec ? launch_pdl(sum_partials_kernel<float4>, blocks, dim3(256), 0, s,
+                                         reinterpret_cast<const float4*>(part), splits, m, reinterpret_cast<float4*>(y))
+                            : launch_pdl(sum_partials_kernel<float>, blocks, dim3(256), 0, s, part, splits, m, y);
+  return e == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
 }
 
 }  // namespace lsp
