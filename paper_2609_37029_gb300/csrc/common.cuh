@@ -325,13 +325,22 @@ __device__ __forceinline__ uint4 philox4x32_10(uint4 c, uint2 k) {
 // fast log's absolute error (~2^-21) is a relative error below 2^-16; the
 // outer log only needs absolute accuracy.  The drafted tokens are compared
 // with the fp64 definition wherever the top-2 gap exceeds 1e-2.
+//
+// The noise is the arithmetic of sampling, so the instructions are counted: with
+// k = x >> 9 < 2^23, the bits 0x3f800000 | k are 1 + k 2^-23, one funnel shift;
+// subtracting 1 - 2^-24 leaves u exactly, and 1 - u is exact again (integer to
+// float conversions would share the slow pipe of the logarithms).  Neither
+// logarithm's argument is subnormal.
+__device__ __forceinline__ float neg_ln(float x) {
+  float y;
+  asm("lg2.approx.ftz.f32 %0, %1;" : "=f"(y) : "f"(x));
+  return -(y * 0.693147180559945f);
+}
 __device__ __forceinline__ float gumbel_of(uint32_t x) {
-  const uint32_t k = x >> 9;
-  const float u = ((float)k + 0.5f) * 1.1920928955078125e-07f;          // 2^-23
-  const float w = ((float)(8388607u - k) + 0.5f) * 1.1920928955078125e-07f;   // 1 - u, exact
+  const float u = __uint_as_float(__funnelshift_r(x, 0x7fu, 9)) - 0.999999940395355224609375f;
+  const float w = 1.0f - u;
   const float series = w * fmaf(w, fmaf(w, 0.333333343f, 0.5f), 1.0f);
-  const float l = w < 0.03125f ? series : -__logf(u);
-  return -__logf(l);
+  return neg_ln(w < 0.03125f ? series : neg_ln(u));
 }
 
 // ---------------------------------------------------------------- warp-level mma.sync helpers

@@ -9,19 +9,19 @@
 //
 // sample_persistent_kernel (bf16, C <= 16, rc in {32, 64}, vocabulary slice
 // fits shared memory): one cooperative launch for all B steps, one CTA per SM.
-// Each CTA owns a contiguous slice of 16-row vocabulary tiles and keeps its
-// W_c rows resident in shared memory for the whole launch.  Sixteen compute
-// warps form the correction as mma.sync tiles with the requests on M (16) and
-// the vocabulary on N, add the base logits (staged one step ahead by
-// cp.async), add the noise and keep a running argmax.  A control warp
-// publishes the CTA's best (value, index) of every request as one 64-bit
-// atomicMax key, arrives on the step's counter, waits (bounded) for every CTA,
-// reads y_i and gathers E_c(y_i) for the next step, while the compute warps
-// draw the next step's noise.  The k index of the contraction is permuted
+// Each CTA owns a contiguous slice of 32-row vocabulary tiles and keeps its
+// W_c rows resident in shared memory for the whole launch.  The requests form one
+// or two groups of eight, which sixteen compute warps take in turn: the
+// correction as mma.sync tiles with the vocabulary on M and the group's requests on N, base
+// logits, noise, a running argmax.  A control warp of each group exchanges the
+// CTA's best (value, index) with the other CTAs, learns y_i and gathers
+// E_c(y_i) for the next step, and an I/O warp moves the corrected logits out and
+// the next ones in, while the compute warps draw the next step's noise and score
+// the other group.  The k index of the contraction is permuted
 // identically in both operands so that each lane's operand words are
-// contiguous in shared memory, and the vocabulary columns are permuted so that
-// each lane's accumulators are four consecutive vocabulary entries (one
-// Philox call, one float4 of logits).
+// contiguous in shared memory, and the vocabulary rows are permuted so that
+// each lane's accumulators are four consecutive vocabulary entries of two requests (one
+// Philox call, one float4 of logits each).
 //
 // sample_step_kernel (every other shape): one launch per step i: every CTA
 // first finishes step i-1's argmax from the per-CTA partials (so y_{i-1} is
@@ -280,15 +280,21 @@ __global__ void __launch_bounds__(kSampThreads, 2) sample_step_kernel(const Samp
 
 // ------------------------------------------------------------------ persistent kernel
 constexpr int kPWarps = 16;                          // compute warps
-constexpr int kPThreads = (kPWarps + 1) * 32;        // + the control warp
-constexpr int kPTilesPerWarp = 4;
-constexpr int kPMaxTiles = kPWarps * kPTilesPerWarp; // 64 tiles = 1024 vocabulary rows per CTA
-constexpr int kPMaxC = 16;
-constexpr int kSlotStride = 16;                      // u64 words between step keys: one 128-byte line
-                                                     // per (step, request) spreads the atomics over L2
-constexpr int kBarKeys = 1;                          // compute warps -> control warp: keys ready
-constexpr int kBarNext = 2;                          // control warp -> compute warps: E_c(y_i) ready
-constexpr int kBarPub = 3;                           // control warp -> compute warps: keys published (T = 0)
+constexpr int kPMaxGroups = 2;                       // request groups of eight
+constexpr int kPPairsPerWarp = 2;
+constexpr int kPMaxPairs = kPWarps * kPPairsPerWarp; // 32-row vocabulary tiles a CTA: 1024 rows
+constexpr int kPGroup = 8;                           // requests of a group (mma N)
+constexpr int kPMaxC = kPGroup * kPMaxGroups;
+constexpr int kSlotStride = 16;                      // (fp32 kernel) u64 words between step keys
+constexpr int kIdxBits = 18, kTagBits = 14;          // low half of an exchanged key: ~index, step tag
+constexpr int kAnsCopies = 8;                        // copies of the answers
+constexpr int kLeadBatch = 5;                        // slots a leader's lane has in flight (152 CTAs in one go)
+// named barriers of the compute warps with one more warp: 1 + group, a step's keys (-> control); 3 + group,
+// E_c(y) (control ->); 5 + group, a step's corrected rows (-> I/O)
+constexpr int kPBar = (kPWarps + 1) * 32;
+// Floats between two requests' logits rows in shared memory: 16 bytes of padding
+// put the four requests that lanes read together on different banks.
+__host__ __device__ inline int z_pitch(int tpc) { return tpc * 32 + 4; }
 
 // Order-preserving 64-bit key of (value, index): a larger value wins, equal
 // values go to the lower index; -0 ranks as +0.
@@ -303,10 +309,12 @@ __device__ __forceinline__ unsigned long long max_u64(unsigned long long a, unsi
   return a > b ? a : b;
 }
 
-__device__ __forceinline__ void cp_async16(void* dst, const void* src, uint32_t src_bytes) {
-  asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(smem_u32(dst)), "l"(src),
-               "r"(src_bytes)
-               : "memory");
+// The warp's largest key, in every lane: the value half, then the index half of
+// the lanes that hold it.
+__device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k) {
+  const unsigned hi = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32));
+  const unsigned lo = __reduce_max_sync(0xffffffffu, (unsigned)(k >> 32) == hi ? (unsigned)k : 0u);
+  return ((unsigned long long)hi << 32) | lo;
 }
 
 __device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
@@ -319,6 +327,10 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
+}
+
+__device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
+  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
 __device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
@@ -339,43 +351,51 @@ __device__ __forceinline__ bool wait_count(const unsigned* c, unsigned target) {
   }
 }
 
-// Control warp: E_c rows of the current tokens (lane r < C holds y_r) into Es,
-// 16-byte chunk c of row r stored at chunk c ^ (r & 1).
+// Control warp: E_c rows of the group's current tokens (lane r < C holds y_r)
+// into Es, 16-byte chunk c of row r stored at chunk c ^ (r & 1).
 template <int CH>
 __device__ __forceinline__ void gather_e(const bf16* Ec, int y, int C, int rc, uint8_t* Es, int lane) {
+  uint4 v[(kPGroup * CH + 31) / 32];
 #pragma unroll
-  for (int i0 = 0; i0 < kPMaxC * CH; i0 += 32) {
+  for (int i0 = 0; i0 < kPGroup * CH; i0 += 32) {
     const int i = i0 + lane, r = i / CH, c = i % CH;
-    const int yr = __shfl_sync(0xffffffffu, y, r);
-    if (r < C) {
-      const uint4 v = *reinterpret_cast<const uint4*>(Ec + (size_t)yr * rc + c * 8);
-      *reinterpret_cast<uint4*>(Es + r * (CH * 16) + ((c ^ (r & 1)) * 16)) = v;
-    }
+    const int yr = __shfl_sync(0xffffffffu, y, r & 31);
+    if (r < C) v[i0 / 32] = *reinterpret_cast<const uint4*>(Ec + (size_t)yr * rc + c * 8);
+  }
+#pragma unroll
+  for (int i0 = 0; i0 < kPGroup * CH; i0 += 32) {
+    const int i = i0 + lane, r = i / CH, c = i % CH;
+    if (r < C) *reinterpret_cast<uint4*>(Es + r * (CH * 16) + ((c ^ (r & 1)) * 16)) = v[i0 / 32];
   }
 }
 
-// KS = rc / 16 k-steps of the m16n8k16 contraction.
-// (17 warps of 32 threads: at 120 registers a thread the occupancy query
-// reports no resident CTA, so the bound stays at 96 registers)
-template <int KS>
-__global__ void __launch_bounds__(kPThreads, 1)
-    sample_persistent_kernel(const SampleParams p, const int ntiles) {
+// Where row r of the W_c slice sits: rows r and r + 4, which neighbouring lane
+// groups read together, are adjacent (and swizzled against each other).
+__device__ __forceinline__ int wc_pos(int r) { return (r & ~7) + 2 * (r & 3) + ((r >> 2) & 1); }
+
+// KS = rc / 16 k-steps of the m16n8k16 contraction; NG groups of up to eight
+// requests: 16 compute warps, then a control warp and an I/O warp a group (20 warps:
+// 96 registers a thread).
+template <int KS, int NG>
+__global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
+    sample_persistent_kernel(const SampleParams p, const int npairs) {
   constexpr int RB = KS * 32;        // bytes of one W_c / E_c row
   constexpr int CH = RB / 16;        // 16-byte chunks per row
   constexpr int TCH = KS / 2;        // chunks of one lane's k range
+  constexpr int kThreads = (kPWarps + 2 * NG) * 32;
   extern __shared__ __align__(128) uint8_t psm[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int nblk = gridDim.x;
-  const int t_begin = (int)(((long long)blockIdx.x * ntiles) / nblk);
-  const int cnt = (int)(((long long)(blockIdx.x + 1) * ntiles) / nblk) - t_begin;
-  const int tpc = (ntiles + nblk - 1) / nblk;
-  uint8_t* Ws = psm;                                                    // [tpc*16][RB]
-  float4* Zs = reinterpret_cast<float4*>(psm + (size_t)tpc * 16 * RB);  // [tpc][2][32]
-  uint8_t* Es = reinterpret_cast<uint8_t*>(Zs + (size_t)tpc * 64);      // [16][RB]
-  unsigned long long* red = reinterpret_cast<unsigned long long*>(Es + kPMaxC * RB);   // [warps][16]
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(red + kPWarps * kPMaxC);
-  unsigned long long* slots = p.sync;                                   // [B][16][kSlotStride]
-  unsigned* counts = reinterpret_cast<unsigned*>(p.sync + (size_t)p.B * kPMaxC * kSlotStride);   // [B]
+  const int t_begin = (int)(((long long)blockIdx.x * npairs) / nblk);
+  const int cnt = (int)(((long long)(blockIdx.x + 1) * npairs) / nblk) - t_begin;
+  const int tpc = (npairs + nblk - 1) / nblk;
+  const int zpitch = z_pitch(tpc);                                      // floats
+  uint8_t* Ws = psm;                                                    // [tpc*32][RB]
+  float* Zs = reinterpret_cast<float*>(psm + (size_t)tpc * 32 * RB);    // [NG][8][zpitch]
+  uint8_t* Es = reinterpret_cast<uint8_t*>(Zs + (size_t)NG * kPGroup * zpitch);              // [NG][8][RB]
+  unsigned long long* red = reinterpret_cast<unsigned long long*>(Es + NG * kPGroup * RB);   // [NG][warps][8]
+  unsigned long long* zbar = red + NG * kPWarps * kPGroup;                        // [NG] the group's logits have landed
+  volatile int* abort_flag = reinterpret_cast<volatile int*>(zbar + NG);
   const bf16* Wc = static_cast<const bf16*>(p.Wc);
   const bf16* Ec = static_cast<const bf16*>(p.Ec);
   const int C = p.C, B = p.B, V = p.V, rc = p.rc;
@@ -384,14 +404,18 @@ __global__ void __launch_bounds__(kPThreads, 1)
   const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
   const int g = lane >> 2, q = lane & 3;                               // mma group / thread in group
 
-  // ---- prologue: W_c slice, zero E rows, step-0 logits, y_0, E_c(y_0)
-  for (int i = tid; i < cnt * 16 * CH; i += kPThreads) {
-    const int r = i / CH, c = i % CH;
-    cp_async16(Ws + r * RB + ((c ^ (r & 1)) * 16), Wc + (size_t)(t_begin * 16 + r) * rc + c * 8, 16);
+  // ---- prologue: W_c slice, zero E rows, y_0, E_c(y_0)
+  for (int i = tid; i < cnt * 32 * CH; i += kThreads) {
+    const int r = i / CH, c = i % CH, pos = wc_pos(r);
+    if (t_begin * 32 + r < V) cp_async16(Ws + pos * RB + ((c ^ (pos & 1)) * 16), Wc + (size_t)(t_begin * 32 + r) * rc + c * 8);
   }
-  for (int i = tid; i < kPMaxC * RB / 16; i += kPThreads)
+  for (int i = tid; i < NG * kPGroup * RB / 16; i += kThreads)
     reinterpret_cast<uint4*>(Es)[i] = make_uint4(0u, 0u, 0u, 0u);
-  if (tid == 0) *abort_flag = 0;
+  if (tid == 0) {
+    *abort_flag = 0;
+    for (int h = 0; h < NG; ++h) mbar_init(smem_u32(zbar + h), 1);
+    fence_barrier_init();
+  }
   // E_c rows are gathered at random every step: keep the table in L2 (this CTA's share)
   if (tid == kPWarps * 32) {
     const size_t bytes = (size_t)V * rc * 2;
@@ -407,217 +431,275 @@ __global__ void __launch_bounds__(kPThreads, 1)
     }
   }
 
-  // this lane's own logits of step s for local tile lt (the same lane reads them)
-  auto issue_z_tile = [&](int s, int lt) {
-    const int v = (t_begin + lt) * 16 + 4 * q;
+  // A lane's four vocabulary entries of local tile lt start at v_of(lt); its
+  // requests of group h are 8 h + 2 q + e, e = 0, 1.
+  auto v_of = [&](int lt) { return (t_begin + lt) * 32 + 4 * g; };
+  float gn[kPPairsPerWarp][NG][2][4];      // noise of the step about to be scored
+  auto draw_noise_tile = [&](int s, int j, int lt, int h) {
+    const int v = v_of(lt);
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const int r = g + 8 * h;
-      const bool ok = r < C;
-      cp_async16(&Zs[(lt * 2 + h) * 32 + lane], p.src + (ok ? ((size_t)r * B + s) * V + v : 0), ok ? 16u : 0u);
+    for (int e = 0; e < 2; ++e) {
+      if (e == 1 && h * kPGroup + 1 >= C) break;                        // one request in the group
+      const uint4 x = philox4x32_10(make_uint4((uint32_t)(v >> 2), (uint32_t)s, (uint32_t)(p.b0 + h * kPGroup + 2 * q + e), p.round), key);
+      gn[j][h][e][0] = gumbel_of(x.x);
+      gn[j][h][e][1] = gumbel_of(x.y);
+      gn[j][h][e][2] = gumbel_of(x.z);
+      gn[j][h][e][3] = gumbel_of(x.w);
     }
   };
-  float gn[kPTilesPerWarp][2][4];      // noise of the step about to be scored
-  auto draw_noise_tile = [&](int s, int j, int lt) {
-    const int v = (t_begin + lt) * 16 + 4 * q;
 #pragma unroll
-    for (int h = 0; h < 2; ++h) {
-      const uint4 x = philox4x32_10(make_uint4((uint32_t)(v >> 2), (uint32_t)s, (uint32_t)(p.b0 + g + 8 * h), p.round), key);
-      gn[j][h][0] = gumbel_of(x.x);
-      gn[j][h][1] = gumbel_of(x.y);
-      gn[j][h][2] = gumbel_of(x.z);
-      gn[j][h][3] = gumbel_of(x.w);
-    }
-  };
+  for (int j = 0; j < kPPairsPerWarp; ++j)
+#pragma unroll
+    for (int h = 0; h < NG; ++h)
+#pragma unroll
+      for (int e = 0; e < 2; ++e) gn[j][h][e][0] = gn[j][h][e][1] = gn[j][h][e][2] = gn[j][h][e][3] = 0.f;
 
-  int y = 0;                                                            // control warp: y of lane < C
-  if (warp < kPWarps) {
-#pragma unroll
-    for (int j = 0; j < kPTilesPerWarp; ++j)
-      if (warp + kPWarps * j < cnt) issue_z_tile(0, warp + kPWarps * j);
-  } else {
-    __syncwarp();
-    if (lane < C) {
-      y = p.prev[(size_t)lane * p.prev_stride];
+  const bool control = warp >= kPWarps && warp < kPWarps + NG;
+  const int grp = warp < kPWarps ? 0 : (warp - kPWarps) % NG;           // control and I/O warps: their group
+  const int Cg = min(kPGroup, C - grp * kPGroup);
+  int y = 0;                                                            // control warps: y of request `lane`
+  unsigned epoch = 0;
+  if (control) {
+    epoch = *reinterpret_cast<volatile unsigned*>(p.sync);              // before any CTA can end
+    if (lane < Cg) {
+      y = p.prev[(size_t)(grp * kPGroup + lane) * p.prev_stride];
       if (y < 0 || y >= V) {
         if (blockIdx.x == 0) set_err(p.err, LSP_DEV_BAD_TOKEN);
         y = 0;
       }
     }
   }
-  asm volatile("cp.async.commit_group;" ::: "memory");
-  __syncthreads();                                                      // E rows zeroed
-  if (warp == kPWarps) gather_e<CH>(Ec, y, C, rc, Es, lane);
+  __syncthreads();                                                      // E rows zeroed, barriers ready
+  if (control) gather_e<CH>(Ec, y, Cg, rc, Es + grp * kPGroup * RB, lane);
+  // this CTA's slice of a logits row
+  const size_t first = (size_t)t_begin * 32;
+  const uint32_t zrow = (uint32_t)(min((size_t)cnt * 32, (size_t)V - first) * sizeof(float));
+  // I/O warp: rows of step s into the group's buffer (lane r: its request's row)
+  auto load_rows = [&](int s) {
+    const uint32_t bar = smem_u32(zbar + grp);
+    if (lane == 0) mbar_expect_tx(bar, zrow * (uint32_t)Cg);
+    __syncwarp();
+    if (lane < Cg)
+      asm volatile("cp.async.bulk.shared::cluster.global.mbarrier::complete_tx::bytes [%0], [%1], %2, [%3];" ::"r"(
+                       smem_u32(Zs + (size_t)(grp * kPGroup + lane) * zpitch)),
+                   "l"(p.src + ((size_t)(grp * kPGroup + lane) * B + s) * V + first), "r"(zrow), "r"(bar)
+                   : "memory");
+  };
+  if (warp >= kPWarps + NG) load_rows(0);
   if (warp < kPWarps && sample) {
 #pragma unroll
-    for (int j = 0; j < kPTilesPerWarp; ++j)
-      if (warp + kPWarps * j < cnt) draw_noise_tile(0, j, warp + kPWarps * j);
+    for (int j = 0; j < kPPairsPerWarp; ++j)
+#pragma unroll
+      for (int h = 0; h < NG; ++h)
+        if (warp + kPWarps * j < cnt) draw_noise_tile(0, j, warp + kPWarps * j, h);
   }
   asm volatile("cp.async.wait_all;" ::: "memory");
   __syncthreads();                                                      // W_c slice and E_c(y_0) visible
 
   if (warp < kPWarps) {
-    // ================= compute warps
+    // ================= compute warps: the groups in turn, so that one group's
+    // exchange and logits traffic run under the other's scoring and noise
     for (int s = 0; s < B; ++s) {
-      // A operand: E_c(y) rows g and g + 8 over this lane's k range
-      uint32_t a[KS][4];
-      {
-        uint32_t e0[2 * KS], e1[2 * KS];
-#pragma unroll
-        for (int c = 0; c < TCH; ++c) {
-          const int pc = (TCH * q + c) ^ (g & 1);
-          const uint4 u0 = *reinterpret_cast<const uint4*>(Es + g * RB + pc * 16);
-          const uint4 u1 = *reinterpret_cast<const uint4*>(Es + (g + 8) * RB + pc * 16);
-          e0[4 * c] = u0.x; e0[4 * c + 1] = u0.y; e0[4 * c + 2] = u0.z; e0[4 * c + 3] = u0.w;
-          e1[4 * c] = u1.x; e1[4 * c + 1] = u1.y; e1[4 * c + 2] = u1.z; e1[4 * c + 3] = u1.w;
-        }
-#pragma unroll
-        for (int ks = 0; ks < KS; ++ks) {
-          a[ks][0] = e0[2 * ks];
-          a[ks][1] = e1[2 * ks];
-          a[ks][2] = e0[2 * ks + 1];
-          a[ks][3] = e1[2 * ks + 1];
-        }
-      }
-      asm volatile("cp.async.wait_all;" ::: "memory");                  // this lane's z_s landed
-      const int v_first = (t_begin + warp) * 16 + 4 * q;
-      float bv[2] = {-INFINITY, -INFINITY};
-      int bi[2] = {v_first, v_first};
-#pragma unroll
-      for (int j = 0; j < kPTilesPerWarp; ++j) {
-        const int lt = warp + kPWarps * j;
-        if (lt >= cnt) break;                                           // warp-uniform
-        const int v = (t_begin + lt) * 16 + 4 * q;
-        float acc[2][4];
-#pragma unroll
-        for (int t = 0; t < 2; ++t) {
-          // column n = g of n-tile t is vocabulary row 4 (g >> 1) + 2 t + (g & 1) of the tile
-          const int row = lt * 16 + 4 * (g >> 1) + 2 * t + (g & 1);
-          uint32_t bw[2 * KS];
-#pragma unroll
-          for (int c = 0; c < TCH; ++c) {
-            const uint4 u = *reinterpret_cast<const uint4*>(Ws + row * RB + (((TCH * q + c) ^ (g & 1)) * 16));
-            bw[4 * c] = u.x; bw[4 * c + 1] = u.y; bw[4 * c + 2] = u.z; bw[4 * c + 3] = u.w;
-          }
-          acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
-#pragma unroll
-          for (int ks = 0; ks < KS; ++ks) mma_bf16_s(acc[t], a[ks], bw[2 * ks], bw[2 * ks + 1]);
-        }
-#pragma unroll
-        for (int h = 0; h < 2; ++h) {
-          const float4 z = Zs[(lt * 2 + h) * 32 + lane];
-          float zc[4] = {z.x + acc[0][2 * h], z.y + acc[0][2 * h + 1], z.z + acc[1][2 * h],
-                         z.w + acc[1][2 * h + 1]};
-          // corrected logits go out after the keys are published (below)
-          if (p.dst) Zs[(lt * 2 + h) * 32 + lane] = make_float4(zc[0], zc[1], zc[2], zc[3]);
-          if (sample) {
-#pragma unroll
-            for (int e = 0; e < 4; ++e) zc[e] = zc[e] * inv_temp + gn[j][h][e];
-          }
-#pragma unroll
-          for (int e = 0; e < 4; ++e)
-            if (zc[e] > bv[h]) { bv[h] = zc[e]; bi[h] = v + e; }
-        }
-      }
-#pragma unroll
-      for (int h = 0; h < 2; ++h) {
-        unsigned long long k = warp < cnt ? arg_key(bv[h], bi[h]) : 0ull;
-        k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, 1));
-        k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, 2));
-        if (q == 0) red[warp * kPMaxC + g + 8 * h] = k;
-      }
-      named_arrive(kBarKeys, kPThreads);
-      // HBM traffic of this lane (corrected logits out, next logits in) and the
-      // next step's noise overlap the grid-wide wait; tile by tile, so that the
-      // noise arithmetic of a tile runs while its memory operations drain
-      // instead of the warp stalling on a full store queue.  Greedy (no noise):
-      // the traffic waits until the control warp has published the step's keys,
-      // so that the key atomics and their release do not queue behind it
-      // (measured at the Qwen3-8B shape: 6.0 -> 5.3 us per step at T = 0; at
-      // T = 1 the same wait, filled with noise, made the round 8 us slower).
-      if (!sample) named_bar(kBarPub, kPThreads);
       const bool more = s + 1 < B;
 #pragma unroll
-      for (int j = 0; j < kPTilesPerWarp; ++j) {
-        const int lt = warp + kPWarps * j;
-        if (lt < cnt) {
-          if (p.dst) {
-            const int v = (t_begin + lt) * 16 + 4 * q;
+      for (int h = 0; h < NG; ++h) {
+        if (s > 0) {
+          named_bar(3 + h, kPBar);
+          if (*abort_flag) {                                            // the others wait for keys, and see the flag
 #pragma unroll
-            for (int h = 0; h < 2; ++h)
-              if (g + 8 * h < C)
-                *reinterpret_cast<float4*>(p.dst + ((size_t)(g + 8 * h) * B + s) * V + v) =
-                    Zs[(lt * 2 + h) * 32 + lane];
-          }
-          if (more) {
-            issue_z_tile(s + 1, lt);                                    // slot already consumed
-            if (sample) draw_noise_tile(s + 1, j, lt);
+            for (int u = 0; u < NG; ++u) {
+              named_arrive(1 + u, kPBar);
+              named_arrive(5 + u, kPBar);
+            }
+            return;
           }
         }
+        // B operand: E_c(y) row g of the group over this lane's k range
+        uint32_t eb[2 * KS];
+#pragma unroll
+        for (int c = 0; c < TCH; ++c) {
+          const uint4 u = *reinterpret_cast<const uint4*>(Es + (h * kPGroup + g) * RB + (((TCH * q + c) ^ (g & 1)) * 16));
+          eb[4 * c] = u.x; eb[4 * c + 1] = u.y; eb[4 * c + 2] = u.z; eb[4 * c + 3] = u.w;
+        }
+        mbar_wait(smem_u32(zbar + h), (uint32_t)s & 1u, p.err);         // z_s landed
+        float bv[2] = {-INFINITY, -INFINITY};
+        int bi[2] = {v_of(warp), v_of(warp)};
+#pragma unroll
+        for (int j = 0; j < kPPairsPerWarp; ++j) {
+          const int lt = warp + kPWarps * j;
+          if (lt >= cnt) break;                                         // warp-uniform
+          const int v = v_of(lt);
+          // row g (+ 8) of m-tile t is vocabulary row 4 g + 2 t (+ 1): a lane's
+          // accumulators are four consecutive entries of two requests
+          float acc[2][4];
+#pragma unroll
+          for (int t = 0; t < 2; ++t) {
+            uint32_t w0[2 * KS], w1[2 * KS];
+            const int pos = lt * 32 + (g >> 1) * 8 + 4 * t + (g & 1);
+#pragma unroll
+            for (int c = 0; c < TCH; ++c) {
+              const int pc = ((TCH * q + c) ^ (g & 1)) * 16;
+              const uint4 u0 = *reinterpret_cast<const uint4*>(Ws + pos * RB + pc);
+              const uint4 u1 = *reinterpret_cast<const uint4*>(Ws + (pos + 2) * RB + pc);
+              w0[4 * c] = u0.x; w0[4 * c + 1] = u0.y; w0[4 * c + 2] = u0.z; w0[4 * c + 3] = u0.w;
+              w1[4 * c] = u1.x; w1[4 * c + 1] = u1.y; w1[4 * c + 2] = u1.z; w1[4 * c + 3] = u1.w;
+            }
+            acc[t][0] = acc[t][1] = acc[t][2] = acc[t][3] = 0.f;
+#pragma unroll
+            for (int ks = 0; ks < KS; ++ks) {
+              const uint32_t a[4] = {w0[2 * ks], w1[2 * ks], w0[2 * ks + 1], w1[2 * ks + 1]};
+              mma_bf16_s(acc[t], a, eb[2 * ks], eb[2 * ks + 1]);
+            }
+          }
+#pragma unroll
+          for (int e = 0; e < 2; ++e) {
+            float4* zp = reinterpret_cast<float4*>(Zs + (size_t)(h * kPGroup + 2 * q + e) * zpitch + lt * 32 + 4 * g);
+            const float4 z = *zp;
+            float zc[4] = {z.x + acc[0][e], z.y + acc[0][2 + e], z.z + acc[1][e], z.w + acc[1][2 + e]};
+            if (p.dst) *zp = make_float4(zc[0], zc[1], zc[2], zc[3]);   // the I/O warp stores the row
+            if (sample) {
+#pragma unroll
+              for (int i = 0; i < 4; ++i) zc[i] = zc[i] * inv_temp + gn[j][h][e][i];
+            }
+#pragma unroll
+            for (int i = 0; i < 4; ++i)
+              if (zc[i] > bv[e] && v < V) { bv[e] = zc[i]; bi[e] = v + i; }
+          }
+        }
+#pragma unroll
+        for (int e = 0; e < 2; ++e) {
+          unsigned long long k = warp < cnt && bi[e] < V ? arg_key(bv[e], bi[e]) : 0ull;
+          k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, 4));
+          k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, 8));
+          k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, 16));
+          if (g == 0) red[(h * kPWarps + warp) * kPGroup + 2 * q + e] = k;
+        }
+        named_arrive(1 + h, kPBar);
+        fence_proxy_async_smem();                                       // the row buffers go to the async proxy
+        named_arrive(5 + h, kPBar);
+        if (more && sample) {
+#pragma unroll
+          for (int j = 0; j < kPPairsPerWarp; ++j)
+            if (warp + kPWarps * j < cnt) draw_noise_tile(s + 1, j, warp + kPWarps * j, h);
+        }
       }
-      if (!more) break;
-      asm volatile("cp.async.commit_group;" ::: "memory");
-      named_bar(kBarNext, kPThreads);
-      if (*abort_flag) break;
     }
-    asm volatile("cp.async.wait_all;" ::: "memory");
     return;
   }
 
-  // ================= control warp
-  const size_t zrow = (size_t)cnt * 16 * sizeof(float);                  // this CTA's slice of one logits row
+  if (warp >= kPWarps + NG) {
+    // ================= I/O warp of group grp: the corrected rows out and the next
+    // ones in by bulk copies, a row a lane, so that no compute warp waits on
+    // the memory system (their vector stores and loads took 2.6 us a step at
+    // 16 requests, the bandwidth's time, with nothing under them)
+    for (int s = 0; s < B; ++s) {
+      named_bar(5 + grp, kPBar);
+      if (*abort_flag) {
+        mbar_wait(smem_u32(zbar + grp), (uint32_t)s & 1u, p.err);       // the load of step s may be in flight
+        return;
+      }
+      if (lane < Cg && p.dst) {
+        asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
+                         p.dst + ((size_t)(grp * kPGroup + lane) * B + s) * V + first),
+                     "r"(smem_u32(Zs + (size_t)(grp * kPGroup + lane) * zpitch)), "r"(zrow)
+                     : "memory");
+        bulk_commit();
+        bulk_wait_read<0>();
+      }
+      __syncwarp();
+      if (s + 1 < B) load_rows(s + 1);
+    }
+    return;
+  }
+
+  // ================= control warp of group grp
+  // The exchange carries its own evidence: a CTA's best (value, index) of a
+  // request is one 64-bit word with the step's tag in its low bits, written with a
+  // plain store into the CTA's slot.  The request's leader (CTA r leads request r,
+  // round robin where there are fewer CTAs) reads its slots until all tags are the step's,
+  // and answers with a tagged word that every CTA reads: no counter, no
+  // fence and no atomic, so the words do not queue behind the step's logits
+  // traffic (the atomic key, release add and count of before: 3.6 + 1.3 us a step at
+  // T = 1).  The answers go out in 8 copies, a 128-byte line each, that 19 CTAs read:
+  // polls of one line by every CTA hold up the store they wait for (C = 8:
+  // 84 us with one copy, 78 with 8, 80 with 32).  Slots alternate between two sets: a CTA writes step s + 2 only after
+  // the answer of step s + 1, which its leader gives after reading step s.
+  // Tags go on from launch to launch (the epoch word), so nothing is cleared.
+  unsigned long long* answers = p.slots;                                // [2][kAnsCopies][kPMaxC]
+  constexpr unsigned long long kTagMask = (1ull << kTagBits) - 1;
+  const int r0 = grp * kPGroup;
   for (int s = 0; s < B; ++s) {
-    // pull the next step's logits slice into L2 while the compute warps score this one
-    if (s + 1 < B && lane < C && zrow > 0)
-      asm volatile("cp.async.bulk.prefetch.L2.global [%0], %1;" ::"l"(
-                       p.src + ((size_t)lane * B + s + 1) * V + (size_t)t_begin * 16),
-                   "r"((uint32_t)zrow)
-                   : "memory");
-    named_bar(kBarKeys, kPThreads);
-    if (lane < C) {
+    const unsigned long long tag = (unsigned long long)(epoch + s + 1) & kTagMask;
+    unsigned long long* slots = p.slots + 2 * kAnsCopies * kPMaxC + (size_t)(s & 1) * C * nblk;   // [request][CTA]
+    unsigned long long* ans = answers + (s & 1) * kAnsCopies * kPMaxC;
+    named_bar(1 + grp, kPBar);
+    if (*abort_flag) return;                                            // the other group has given up
+    if (lane < Cg) {
       unsigned long long k = 0ull;
 #pragma unroll
-      for (int w = 0; w < kPWarps; ++w) k = max_u64(k, red[w * kPMaxC + lane]);
-      atomicMax(&slots[(s * kPMaxC + lane) * kSlotStride], k);
+      for (int w = 0; w < kPWarps; ++w) k = max_u64(k, red[(grp * kPWarps + w) * kPGroup + lane]);
+      st_relaxed_u64(slots + (size_t)(r0 + lane) * nblk + blockIdx.x,
+                     (k & 0xffffffff00000000ull) | ((k & ((1ull << kIdxBits) - 1)) << kTagBits) | tag);
     }
     __syncwarp();
-    if (lane == 0) red_release_add(&counts[s], 1u);                     // orders the warp's key atomics
-    if (!sample) {
-      __syncwarp();
-      named_arrive(kBarPub, kPThreads);                                 // compute warps may store now
+    bool ok = true;
+    // ---- leader: the best of all CTAs
+    for (int r = r0 + ((int)blockIdx.x - r0 % nblk + nblk) % nblk; r < r0 + Cg && ok; r += nblk) {
+      unsigned long long best = 0ull;
+      for (int c0 = 0; c0 < nblk && ok; c0 += 32 * kLeadBatch) {
+        unsigned long long k[kLeadBatch];
+        const uint64_t t0 = global_ns();
+        for (uint32_t it = 1;; ++it) {
+          bool all = true;
+#pragma unroll
+          for (int u = 0; u < kLeadBatch; ++u) {
+            const int c = c0 + u * 32 + lane;
+            k[u] = c < nblk ? ld_relaxed_u64(slots + (size_t)r * nblk + c) : tag;
+          }
+#pragma unroll
+          for (int u = 0; u < kLeadBatch; ++u) all = all && (k[u] & kTagMask) == tag;
+          if (__all_sync(0xffffffffu, all)) break;
+          if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
+        }
+#pragma unroll
+        for (int u = 0; u < kLeadBatch; ++u) best = max_u64(best, k[u]);
+      }
+      best = warp_max_key(best);
+      if (ok && lane < kAnsCopies) st_relaxed_u64(ans + lane * kPMaxC + r, best);
+      if (ok && lane == 0) {
+        const int t = (int)(~(uint32_t)(best >> kTagBits) & ((1u << kIdxBits) - 1));
+        p.out_tokens[(size_t)r * B + s] = t < V ? t : 0;
+      }
     }
     const bool last = s + 1 == B;
-    if (last && blockIdx.x != 0) return;                                // only CTA 0 needs y_B
-    const bool ok = __all_sync(0xffffffffu, wait_count(&counts[s], (unsigned)nblk));
+    if (last && ok) break;
+    // ---- everyone: the answers
+    if (ok) {
+      const uint64_t t0 = global_ns();
+      unsigned long long k = tag;
+      for (uint32_t it = 1;; ++it) {
+        if (lane < Cg) k = ld_relaxed_u64(ans + ((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane);
+        if (__all_sync(0xffffffffu, (k & kTagMask) == tag)) break;
+        if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
+      }
+      y = (int)(~(uint32_t)(k >> kTagBits) & ((1u << kIdxBits) - 1));
+      if (y >= V) y = 0;                                                // (no entry of the row compared)
+    }
     if (!ok) {
-      if (lane == 0) set_err(p.err, LSP_DEV_TIMEOUT);
-      if (!last) {
-        if (lane == 0) *abort_flag = 1;
-        __syncwarp();
-        named_arrive(kBarNext, kPThreads);
-      }
-      return;
-    }
-    if (lane < C) {
-      y = (int)~(uint32_t)ld_relaxed_u64(&slots[(s * kPMaxC + lane) * kSlotStride]);
-      if (y < 0 || y >= V) {                                            // no key arrived: corrupt sync words
+      if (lane == 0) {
         set_err(p.err, LSP_DEV_TIMEOUT);
-        y = 0;
+        *abort_flag = 1;
       }
-      if (blockIdx.x == 0) p.out_tokens[(size_t)lane * B + s] = y;
-    }
-    if (last) {
-      // every CTA has arrived on every counter, so no one reads the sync words
-      // again: leave them zero for the next launch
       __syncwarp();
-      for (int i = lane; i < B * kPMaxC; i += 32) slots[i * kSlotStride] = 0ull;
-      for (int i = lane; i < B; i += 32) counts[i] = 0u;
+      if (!last) named_arrive(3 + grp, kPBar);                          // releases the compute warps, and they the others
       return;
     }
-    gather_e<CH>(Ec, y, C, rc, Es, lane);
+    gather_e<CH>(Ec, y, Cg, rc, Es + grp * kPGroup * RB, lane);
     __syncwarp();
-    named_arrive(kBarNext, kPThreads);
+    named_arrive(3 + grp, kPBar);
   }
+  // every CTA has read the epoch before its first keys, and those have arrived here
+  if (blockIdx.x == 0 && grp == 0 && lane == 0) *reinterpret_cast<volatile unsigned*>(p.sync) = epoch + (unsigned)B;
 }
 
 // ------------------------------------------------------------------ persistent kernel, fp32 storage
@@ -764,49 +846,65 @@ static cudaError_t launch_step(const SampleParams& p, int step, size_t smem, cud
   return launch_pdl(sample_step_kernel<T, KG>, dim3(p.nblk), dim3(kSampThreads), smem, s, p, step);
 }
 
+// The bf16 loop's exchange: two sets of answers (copies x requests) and of (request, CTA) key slots.
+size_t sample_slot_bytes(int C, int num_sms) {
+  return (size_t)2 * (kAnsCopies * kPMaxC + std::min(C, kPMaxC) * num_sms) * sizeof(unsigned long long);
+}
+
 size_t sample_sync_bytes(int B) {
   return ((size_t)B * kPMaxC * kSlotStride * sizeof(unsigned long long) + (size_t)B * sizeof(unsigned) +
           255) / 256 * 256;
 }
 
-static size_t persistent_smem(int tpc, int rc) {
-  const size_t rb = (size_t)rc * 2;
-  return (size_t)tpc * 16 * rb + (size_t)tpc * 64 * 16 + kPMaxC * rb +
-         (size_t)kPWarps * kPMaxC * sizeof(unsigned long long) + 16;
+// The bf16 loop's vocabulary tiles, CTAs and shared memory.
+struct PersistentPlan {
+  int npairs, nblk, tpc, groups;
+  size_t smem;
+};
+static PersistentPlan persistent_plan(const SampleParams& p) {
+  PersistentPlan q;
+  q.npairs = (p.V + 31) / 32;
+  q.nblk = std::min(p.num_sms, q.npairs);
+  q.tpc = (q.npairs + q.nblk - 1) / q.nblk;
+  q.groups = p.C > kPGroup ? 2 : 1;
+  const size_t rb = (size_t)p.rc * 2;
+  q.smem = (size_t)q.tpc * 32 * rb + (size_t)q.groups * kPGroup * (z_pitch(q.tpc) * sizeof(float) + rb) +
+           (size_t)q.groups * (kPWarps * kPGroup + 1) * sizeof(unsigned long long) + 16;
+  return q;
 }
 
-template <int KS>
+template <int KS, int NG>
 static int launch_persistent(const SampleParams& p, cudaStream_t s) {
-  const int ntiles = p.V / 16;
-  const int nblk = std::min(p.num_sms, ntiles);
-  const int tpc = (ntiles + nblk - 1) / nblk;
-  if (tpc > kPMaxTiles) return LSP_ERR_SHAPE;
-  const size_t smem = persistent_smem(tpc, p.rc);
-  if (smem > 227 * 1024) return LSP_ERR_SHAPE;
+  const PersistentPlan q = persistent_plan(p);
+  const int threads = (kPWarps + 2 * NG) * 32;
   static size_t attr = 0;
-  if (smem > attr) {
-    if (cudaFuncSetAttribute(sample_persistent_kernel<KS>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
+  if (q.smem > attr) {
+    if (cudaFuncSetAttribute(sample_persistent_kernel<KS, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
+                             (int)q.smem) != cudaSuccess)
       return LSP_ERR_CUDA;
-    attr = smem;
+    attr = q.smem;
   }
   int per_sm = 0;
-  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample_persistent_kernel<KS>, kPThreads,
-                                                    smem) != cudaSuccess)
+  if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample_persistent_kernel<KS, NG>, threads, q.smem) !=
+      cudaSuccess)
     return LSP_ERR_CUDA;
   if (per_sm < 1) return LSP_ERR_SHAPE;
   cudaLaunchConfig_t cfg = {};
-  cfg.gridDim = dim3(nblk);
-  cfg.blockDim = dim3(kPThreads);
-  cfg.dynamicSmemBytes = smem;
+  cfg.gridDim = dim3(q.nblk);
+  cfg.blockDim = dim3(threads);
+  cfg.dynamicSmemBytes = q.smem;
   cfg.stream = s;
   cudaLaunchAttribute attr_c[1];
   attr_c[0].id = cudaLaunchAttributeCooperative;       // every CTA resident: the step waits are safe
   attr_c[0].val.cooperative = 1;
   cfg.attrs = attr_c;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, sample_persistent_kernel<KS>, p, ntiles) == cudaSuccess ? LSP_OK
-                                                                                          : LSP_ERR_CUDA;
+  return cudaLaunchKernelEx(&cfg, sample_persistent_kernel<KS, NG>, p, q.npairs) == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
+}
+
+static int launch_persistent_any(const SampleParams& p, cudaStream_t s) {
+  if (p.C > kPGroup) return p.rc == 32 ? launch_persistent<2, 2>(p, s) : launch_persistent<4, 2>(p, s);
+  return p.rc == 32 ? launch_persistent<2, 1>(p, s) : launch_persistent<4, 1>(p, s);
 }
 
 // The persistent kernel's shape limits (anything else takes the per-step kernel).
@@ -860,12 +958,10 @@ static int launch_persistent_f32(const SampleParams& p, cudaStream_t s) {
 }
 
 static bool persistent_ok(const SampleParams& p, int dtype) {
-  if (dtype != LSP_DTYPE_BF16 || p.C > kPMaxC || (p.rc != 32 && p.rc != 64) || !p.sync || p.num_sms < 1)
+  if (dtype != LSP_DTYPE_BF16 || p.C > kPMaxC || (p.rc != 32 && p.rc != 64) || !p.sync || !p.slots || p.num_sms < 1)
     return false;
-  const int ntiles = p.V / 16;
-  const int nblk = std::min(p.num_sms, ntiles);
-  const int tpc = (ntiles + nblk - 1) / nblk;
-  if (tpc > kPMaxTiles || persistent_smem(tpc, p.rc) > 227 * 1024) return false;
+  const PersistentPlan q = persistent_plan(p);
+  if (q.tpc > kPMaxPairs || q.smem > 227 * 1024 || p.V > (1 << kIdxBits) || 2 * p.B + 2 > (1 << kTagBits)) return false;
   return coop_ok();
 }
 
@@ -908,8 +1004,7 @@ int launch_sample(const SampleParams& p, int dtype, cudaStream_t s) {
   if (persistent_groups(p, dtype) > 0) {
     for (int g0 = 0; g0 < p.C; g0 += kPMaxC) {
       const SampleParams q = request_group(p, g0);
-      const int rc = persistent_ok(q, dtype) ? (q.rc == 32 ? launch_persistent<2>(q, s) : launch_persistent<4>(q, s))
-                                             : launch_persistent_f32(q, s);
+      const int rc = persistent_ok(q, dtype) ? launch_persistent_any(q, s) : launch_persistent_f32(q, s);
       if (rc != LSP_OK) return rc;
     }
     return LSP_OK;

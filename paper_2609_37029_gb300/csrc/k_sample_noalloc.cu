@@ -13,6 +13,7 @@
 // are cleared on the caller's stream before every launch, so a launch that
 // gave up waiting cannot affect the next one.
 #include <cmath>
+#include <algorithm>
 #include <mutex>
 
 #include "lsp_internal.h"
@@ -81,7 +82,12 @@ extern "C" int lsp_sample_noalloc(const float* base_logits, const int32_t* prev_
   const size_t sync_bytes = lsp::sample_sync_bytes(B);
   if (sync_off + sync_bytes > kStaticScratchBytes) return LSP_ERR_SHAPE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  if (cudaMemsetAsync(scratch + sync_off, 0, sync_bytes, s) != cudaSuccess) return LSP_ERR_CUDA;
+  // The bf16 loop's key slots take the room of the partials, or what is left
+  // behind the sync words (the per-step kernel runs where neither holds them).
+  const size_t slot_bytes = lsp::sample_slot_bytes(C, num_sms), slot_off = slot_bytes <= sync_off ? 0 : sync_off + sync_bytes;
+  const bool slots = slot_off + slot_bytes <= kStaticScratchBytes;
+  const size_t clear = std::max(sync_off + sync_bytes, slots ? slot_off + slot_bytes : 0);
+  if (cudaMemsetAsync(scratch, 0, clear, s) != cudaSuccess) return LSP_ERR_CUDA;
   lsp::SampleParams p = {};
   p.src = base_logits;
   p.dst = out_logits;
@@ -93,6 +99,7 @@ extern "C" int lsp_sample_noalloc(const float* base_logits, const int32_t* prev_
   p.part_val = reinterpret_cast<float*>(scratch);
   p.part_idx = reinterpret_cast<int*>(scratch + part * sizeof(float));
   p.sync = reinterpret_cast<unsigned long long*>(scratch + sync_off);
+  p.slots = slots ? reinterpret_cast<unsigned long long*>(scratch + slot_off) : nullptr;
   p.err = reinterpret_cast<unsigned*>(dev_error);
   p.C = C;
   p.B = B;

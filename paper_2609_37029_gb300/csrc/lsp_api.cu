@@ -79,7 +79,7 @@ struct lsp_state {
   int* ver_pi = nullptr;
   unsigned* ver_ctr = nullptr;
   unsigned long long* sample_sync = nullptr;
-  size_t sample_sync_bytes = 0;
+  size_t sample_sync_bytes = 0, sample_part_bytes = 0;
   int nblk = 0;
   // cached projection plans
   AttnTcPlan attn_tc = {};
@@ -231,8 +231,9 @@ int lsp_state_create(const lsp_config* cfg, lsp_state** out) {
   const size_t w_log = off; off = align256(off + (size_t)M * c.V * 4);
   const size_t w_rope = off; off = align256(off + (size_t)M * (c.d / 2) * 2 * 4);
   const size_t w_part = off; off = align256(off + pbytes);
-  const size_t w_pv = off; off = align256(off + (size_t)2 * st->nblk * c.C * 4);
-  const size_t w_pi = off; off = align256(off + (size_t)2 * st->nblk * c.C * 4);
+  // argmax partials (values, indices) of the per-step sampler, or the key slots of the bf16 loop
+  st->sample_part_bytes = std::max((size_t)16 * st->nblk * c.C, sample_slot_bytes(c.C, st->num_sms));
+  const size_t w_pv = off; off = align256(off + st->sample_part_bytes);
   const size_t w_sync = off; off = align256(off + sample_sync_bytes(c.B));
   const bool fold_ok = fold_supported(c.dtype, c.d, c.R, c.nq, c.nkv);
   const size_t w_pf = off;
@@ -256,7 +257,7 @@ int lsp_state_create(const lsp_config* cfg, lsp_state** out) {
   st->part = reinterpret_cast<float*>(w + w_part);
   st->part_bytes = pbytes;
   st->part_val = reinterpret_cast<float*>(w + w_pv);
-  st->part_idx = reinterpret_cast<int*>(w + w_pi);
+  st->part_idx = reinterpret_cast<int*>(st->part_val + (size_t)2 * st->nblk * c.C);
   st->sample_sync = reinterpret_cast<unsigned long long*>(w + w_sync);
   st->fold_ws = fold_ok ? reinterpret_cast<float*>(w + w_pf) : nullptr;
   st->ver_sa = reinterpret_cast<float*>(w + w_vsa);
@@ -466,7 +467,7 @@ static int run_sampler(lsp_state* st, const float* src, float* dst, const int32_
   SampleParams p = {};
   p.src = src; p.dst = dst; p.prev = prev; p.prev_stride = prev_stride; p.Ec = Ec; p.Wc = Wc;
   p.out_tokens = out_tokens; p.part_val = st->part_val; p.part_idx = st->part_idx;
-  p.sync = st->sample_sync; p.err = st->err;
+  p.sync = st->sample_sync; p.slots = reinterpret_cast<unsigned long long*>(st->part_val); p.err = st->err;
   p.C = c.C; p.B = c.B; p.V = c.V; p.rc = c.rc; p.nblk = st->nblk; p.num_sms = st->num_sms;
   p.temperature = sp->temperature; p.round = sp->round; p.seed = sp->seed;
   return launch_sample(p, c.dtype, s);
@@ -612,6 +613,7 @@ int lsp_round_launches(lsp_state* st) {
   const lsp_config& c = st->cfg;
   SampleParams p = {};
   p.C = c.C; p.B = c.B; p.V = c.V; p.rc = c.rc; p.num_sms = st->num_sms; p.sync = st->sample_sync;
+  p.slots = reinterpret_cast<unsigned long long*>(st->part_val);
   // view update, fuse, combine; per layer q/k/v GEMM, finalize (not with the
   // tcgen05 attention, which finalises q/k/v itself), attention, o, norm,
   // gate/up, down, norm; LM head; the sampler
@@ -651,9 +653,10 @@ int lsp_get_error(lsp_state* st, uint32_t* dev_error, int clear, lsp_stream_t st
       cudaStreamSynchronize(s) != cudaSuccess)
     return LSP_ERR_CUDA;
   if (clear && v && cudaMemsetAsync(st->err, 0, sizeof(unsigned), s) != cudaSuccess) return LSP_ERR_CUDA;
-  // a sampler launch that gave up waiting leaves its step counters behind
+  // a sampler launch that gave up waiting leaves its step counters and tagged keys behind
   if (clear && (v & LSP_DEV_TIMEOUT) &&
-      cudaMemsetAsync(st->sample_sync, 0, st->sample_sync_bytes, s) != cudaSuccess)
+      (cudaMemsetAsync(st->sample_sync, 0, st->sample_sync_bytes, s) != cudaSuccess ||
+       cudaMemsetAsync(st->part_val, 0, st->sample_part_bytes, s) != cudaSuccess))
     return LSP_ERR_CUDA;
   *dev_error = v;
   if (v & LSP_DEV_TIMEOUT) return LSP_ERR_TIMEOUT;

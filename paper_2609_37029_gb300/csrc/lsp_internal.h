@@ -252,8 +252,9 @@ struct SampleParams {
   int32_t* out_tokens;    // [C][B]
   float* part_val;        // [2][nblk][C]   (per-step kernel)
   int* part_idx;          // [2][nblk][C]
-  unsigned long long* sync;   // sample_sync_bytes(B): step keys + arrival counts (persistent
-                              // kernel); all zero between launches
+  unsigned long long* sync;   // sample_sync_bytes(B), zero at first: the fp32 loop's step keys and
+                              // arrival counts (zero between launches), or the bf16 loop's epoch and answers
+  unsigned long long* slots;  // sample_slot_bytes(C, num_sms), zero at first: the bf16 loop's key slots
   unsigned* err;
   int C, B, V, rc, nblk;
   int num_sms;
@@ -264,6 +265,7 @@ struct SampleParams {
 };
 int sample_blocks(int num_sms);
 size_t sample_sync_bytes(int B);
+size_t sample_slot_bytes(int C, int num_sms);
 int launch_sample(const SampleParams& p, int dtype, cudaStream_t s);
 // Kernel launches one launch_sample call issues for these shapes on this device.
 int sample_launches(const SampleParams& p, int dtype);
