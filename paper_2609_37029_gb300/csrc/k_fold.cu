@@ -32,6 +32,8 @@
 //               queries, P = 2^((s - ref) log2(e) / sqrt(d)) is written as a
 //               bf16 high part and a bf16 remainder (two MMAs, ~16
 //               significant bits), and the sums stay in registers.
+//   warps 10-11 the window ring and the boundary rows; the softmax warps join
+//               them when their blocks are done
 //
 // The reference ref of each query is not the running maximum: bf16 and fp32
 // share their exponent range, so P keeps its precision under any reference
@@ -47,9 +49,9 @@
 // it) and the stored state, in share order: deterministic.
 //
 // Measured (GB300, Qwen3-8B heads, 5 layers): lsp_prefill of 131072 rows
-// (2.68 GB) 745 us with the mma.sync kernel, 411 + 7 us now (6.5 TB/s, the copy
-// bandwidth); lsp_view_update of 2048 rows 232 -> 24 us for one request, 423 ->
-// 183 us for 16.  Relative error of m against 64 bits at 131072 rows: 4.6e-6 ->
+// (2.68 GB) 745 us with the mma.sync kernel, 397 + 7 us now (6.8 TB/s, the copy
+// bandwidth); lsp_view_update of 2048 rows 232 -> 22 us for one request, 423 ->
+// 162 us for 16.  Relative error of m against 64 bits at 131072 rows: 4.6e-6 ->
 // 2.8e-6.
 #include <algorithm>
 #include <type_traits>
@@ -63,13 +65,14 @@ namespace {
 constexpr int kFoldD = 128;                  // head dim
 constexpr int kFoldKeys = 128;               // keys per block (UMMA M)
 constexpr int kFoldSoftmax = 256;            // softmax threads (8 warps)
-constexpr int kFoldThreads = kFoldSoftmax + 64;
+constexpr int kFoldCopy = 64;                // threads that copy the window (2 warps)
+constexpr int kFoldThreads = kFoldSoftmax + 64 + kFoldCopy;
 constexpr int kFoldSlot = kFoldKeys * 256;   // bytes of one K or V block
 constexpr int kFoldRec = 16 + 16 * kFoldD;   // floats per (piece, query head): eta[16], m[16][d]
 constexpr int kFlushBlocks = 8;
 constexpr float kRefSlack = 24.f;            // log2 units a score may pass its reference by
 constexpr int kFoldMaxC = 64;
-constexpr int kCopyBatch = 4;                // window vectors a thread has in flight (K and V each)
+constexpr int kCopyBatch = 4;                // window vectors a copying lane has in flight (K and V each)
 constexpr int kFoldMaxSlots = 5;
 
 struct FoldLayout {
@@ -78,13 +81,13 @@ struct FoldLayout {
 };
 
 // bytes: G [2][16 REP][128 B], P high and remainder [64-query blocks][128][128 B],
-// the ring, then references, scales and 1 / sums, block counts and barriers
+// the ring, then references, scales, block counts, rows and slots, barriers
 __host__ __device__ constexpr FoldLayout fold_layout(int rep) {
   FoldLayout L{};
   const int nb = (16 * rep + 63) / 64;
   L.off_p = (uint32_t)rep * 4096u;
   L.off_ring = L.off_p + 2u * (uint32_t)nb * 16384u;
-  const uint32_t misc = 3u * 128u * 4u + 272u + 160u;
+  const uint32_t misc = 2u * 128u * 4u + 272u + 2u * kFoldMaxC * 4u + 160u;
   const int fit = (int)((227u * 1024u - 1024u - misc - L.off_ring) / (uint32_t)kFoldSlot);
   L.slots = fit < kFoldMaxSlots ? fit : kFoldMaxSlots;
   L.off_misc = L.off_ring + (uint32_t)L.slots * kFoldSlot;
@@ -240,18 +243,17 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(fsm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const uint32_t s_g = smem_u32(sm), s_p = s_g + L.off_p, s_ring = s_g + L.off_ring;
   float* sref = reinterpret_cast<float*>(sm + L.off_misc);   // reference of each query
-  float* sscale = sref + 128;                                // factor of a reference that moved
-  float* sinv = sscale + 128;                                // 1 / sum
-  int* pre = reinterpret_cast<int*>(sinv + 128);             // [65]
-  uint64_t* bars = reinterpret_cast<uint64_t*>(pre + 68);
+  float* sscale = sref + 128;                                // factor of a reference that moved; at a piece's end 1 / sum
+  float* sinv = sscale;
+  int* pre = reinterpret_cast<int*>(sscale + 128);           // [65]
+  int* srows = pre + 68;                                     // new rows of each request
+  int* sslot = srows + kFoldMaxC;                            // and its first window slot
+  uint64_t* bars = reinterpret_cast<uint64_t*>(sslot + kFoldMaxC);
   uint32_t* tslot = reinterpret_cast<uint32_t*>(bars + 2 * kFoldMaxSlots + 8);
   volatile int* stop = reinterpret_cast<volatile int*>(tslot + 1);
   volatile int* sfresh = stop + 1;
+  int* scopy = reinterpret_cast<int*>(tslot + 3);            // next chunk of the window copy
   float* exch = reinterpret_cast<float*>(sm + L.off_p);      // [4][Q] between warps, while P is idle
-  // new rows and first window slot of each request, in the remainder half of P
-  // until the first block's barriers (every window copy is done by then)
-  int* srows = reinterpret_cast<int*>(sm + L.off_p + NB * 16384);
-  int* sslot = srows + kFoldMaxC;
   const uint32_t bar0 = smem_u32(bars);
   auto b_full = [&](int s) { return bar0 + 8u * (uint32_t)s; };
   auto b_empty = [&](int s) { return bar0 + 8u * (uint32_t)(kFoldMaxSlots + s); };
@@ -259,7 +261,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   auto b_sempty = [&](int s) { return bar0 + 8u * (uint32_t)(2 * kFoldMaxSlots + 2 + s); };
   const uint32_t b_p = bar0 + 8u * (2 * kFoldMaxSlots + 4), b_pv = b_p + 8, b_g = b_p + 16, b_end = b_p + 24;
 
-  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31;
   if (tid == 0) {
     for (int s = 0; s < NS; ++s) {
       mbar_init(b_full(s), 1);
@@ -274,6 +276,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     mbar_init(b_g, kFoldSoftmax / 32);
     mbar_init(b_end, 1);
     *stop = 0;
+    *scopy = 0;
     fence_barrier_init();
     tma_prefetch_desc(&mk);
     tma_prefetch_desc(&mv);
@@ -291,13 +294,13 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
   tc_fence_before();
   __syncthreads();
   tc_fence_after();
-  const uint32_t tmem = *tslot, t_o = tmem + 2u * Q;
+  const uint32_t tmem = uniform(*tslot), t_o = tmem + 2u * Q;
   const int LG = p.L * p.nkv;
   const long long total = (long long)pre[kFoldMaxC] * LG;
   const long long nshare = fold_shares(total, gridDim.x);
   const int f0 = (int)min(total, total * blockIdx.x / nshare), f1 = (int)min(total, total * (blockIdx.x + 1) / nshare);
 
-  if (warp == 8 && lane == 0) {
+  if (warp == 8) {
     // ------------------------------------------------------------ TMA producer
     const uint64_t pol = policy_evict_first();
     int q = 0;                                            // ring position: K and V of a block in turn
@@ -310,17 +313,20 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         for (int kv = 0; kv < 2; ++kv, ++q) {
           const int s = q % NS;
           if (q >= NS && !fold_wait(b_empty(s), (uint32_t)(q / NS - 1) & 1u, stop, p.err)) { ok = false; break; }
-          mbar_expect_tx(b_full(s), kFoldSlot);
-          const uint32_t dst = s_ring + (uint32_t)s * kFoldSlot;
-          const CUtensorMap* mp = kv ? &mv : &mk;
-          tma_load_2d(dst, mp, b_full(s), x, y0 + i * kFoldKeys, pol);
-          tma_load_2d(dst + kFoldSlot / 2, mp, b_full(s), x + 64, y0 + i * kFoldKeys, pol);
+          if (elect_one()) {
+            mbar_expect_tx(b_full(s), kFoldSlot);
+            const uint32_t dst = s_ring + (uint32_t)s * kFoldSlot;
+            const CUtensorMap* mp = kv ? &mv : &mk;
+            tma_load_2d(dst, mp, b_full(s), x, y0 + i * kFoldKeys, pol);
+            tma_load_2d(dst + kFoldSlot / 2, mp, b_full(s), x + 64, y0 + i * kFoldKeys, pol);
+          }
+          __syncwarp();
         }
       f += pc.n;
     }
     // every load has landed before the CTA's shared memory goes away
     for (int i = max(0, q - NS); i < q; ++i) mbar_wait(b_full(i % NS), (uint32_t)(i / NS) & 1u, p.err);
-  } else if (warp == 9 && lane == 0) {
+  } else if (warp == 9) {
     // ------------------------------------------------------------ MMA issue
     const uint32_t id_s = fold_idesc(Q, false), id_o = fold_idesc(Q, true);
     int n = 0, piece = 0;                                 // block and piece of this CTA
@@ -332,14 +338,17 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       if (!ok) return;
       tc_fence_after();
       const uint32_t sk = s_ring + (uint32_t)s * kFoldSlot;
+      if (elect_one()) {
 #pragma unroll
-      for (int ks = 0; ks < kFoldD / 16; ++ks) {
-        const uint32_t kb = (uint32_t)(ks >> 2), in = (uint32_t)(ks & 3) * 32u;
-        umma_f16(tmem + (uint32_t)(buf * Q), sdesc_sw128(sk + kb * (kFoldSlot / 2) + in),
-                 sdesc_sw128(s_g + kb * (uint32_t)(Q * 128) + in), id_s, ks > 0 ? 1u : 0u);
+        for (int ks = 0; ks < kFoldD / 16; ++ks) {
+          const uint32_t kb = (uint32_t)(ks >> 2), in = (uint32_t)(ks & 3) * 32u;
+          umma_f16(tmem + (uint32_t)(buf * Q), sdesc_sw128(sk + kb * (kFoldSlot / 2) + in),
+                   sdesc_sw128(s_g + kb * (uint32_t)(Q * 128) + in), id_s, ks > 0 ? 1u : 0u);
+        }
+        umma_commit(b_empty(s));
+        umma_commit(b_sfull(buf));
       }
-      umma_commit(b_empty(s));
-      umma_commit(b_sfull(buf));
+      __syncwarp();
     };
     for (int f = f0; f < f1; ++piece) {
       const FoldPiece pc = fold_piece(pre, p.nreq, LG, f, f1);
@@ -353,19 +362,23 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         if (!ok) continue;
         tc_fence_after();
         const uint32_t sv = s_ring + (uint32_t)s * kFoldSlot;
-        const uint32_t keep = *sfresh ? 0u : 1u;          // fresh: the accumulator was drained
+        const uint32_t keep = uniform(*sfresh ? 0u : 1u);   // fresh: the accumulator was drained
+        if (elect_one()) {
 #pragma unroll
-        for (int ks = 0; ks < kFoldKeys / 16; ++ks) {
-          const uint64_t ad = fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2);
-          umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)ks * 2048u, 16384u), id_o, ks > 0 ? 1u : keep);
-          umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)(NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o, 1u);
+          for (int ks = 0; ks < kFoldKeys / 16; ++ks) {
+            const uint64_t ad = fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2);
+            umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)ks * 2048u, 16384u), id_o, ks > 0 ? 1u : keep);
+            umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)(NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o, 1u);
+          }
+          umma_commit(b_empty(s));
+          umma_commit(b_pv);
         }
-        umma_commit(b_empty(s));
-        umma_commit(b_pv);
+        __syncwarp();
       }
       f += pc.n;
     }
-    umma_commit(b_end);                                   // no MMA outlives the CTA's TMEM
+    if (elect_one()) umma_commit(b_end);                  // no MMA outlives the CTA's TMEM
+    __syncwarp();
     mbar_wait(b_end, 0, p.err);
   } else if (warp < 8) {
     // ------------------------------------------------------------ softmax
@@ -388,61 +401,24 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     auto load_g = [&](int lg) {
       const int l = lg / p.nkv, g = lg % p.nkv;
       const bf16* G = static_cast<const bf16*>(p.G) + ((size_t)l * p.nq + (size_t)g * REP) * p.R * kFoldD;
-      for (int i = tid; i < Q * 16; i += kFoldSoftmax) {
-        const int row = i >> 4, c8 = i & 15, hh = row >> 4, r = row & 15;
-        uint4 v = make_uint4(0u, 0u, 0u, 0u);
-        if (r < p.R) v = *reinterpret_cast<const uint4*>(G + ((size_t)hh * p.R + r) * kFoldD + c8 * 8);
+      uint4 v[REP];                                       // every load before the first store
+#pragma unroll
+      for (int u = 0; u < REP; ++u) {
+        const int i = tid + u * kFoldSoftmax, row = i >> 4, c8 = i & 15, hh = row >> 4, r = row & 15;
+        v[u] = make_uint4(0u, 0u, 0u, 0u);
+        if (r < p.R) v[u] = *reinterpret_cast<const uint4*>(G + ((size_t)hh * p.R + r) * kFoldD + c8 * 8);
+      }
+#pragma unroll
+      for (int u = 0; u < REP; ++u) {
+        const int i = tid + u * kFoldSoftmax, row = i >> 4, c8 = i & 15;
         st_v4(s_g + (uint32_t)((c8 >> 3) * (Q * 128) + (row >> 3) * 1024 + (row & 7) * 128 + (((c8 & 7) ^ (row & 7)) << 4)),
-              v.x, v.y, v.z, v.w);
+              v[u].x, v[u].y, v[u].z, v[u].w);
       }
       fence_proxy_async_smem();
       __syncwarp();
       if (lane == 0) mbar_arrive(b_g);
     };
     if (f0 < f1) load_g(fold_piece(pre, p.nreq, LG, f0, f1).lg);
-
-    // ---- while the first rows land: the window ring (row q of the prefix in
-    // slot q mod W), the boundary rows, counts out of range
-    if (p.acc && blockIdx.x == 0 && tid < p.nreq && (p.acc[tid] < 0 || p.acc[tid] > p.rows)) set_err(p.err, LSP_DEV_BAD_DELTA);
-    {
-      const int vpr = p.nkv * (kFoldD / 8), span = p.W * vpr;   // 16-byte vectors of a row (all KV heads), of a window
-      const int items = p.nreq * p.L * span;
-      for (int k0 = (int)blockIdx.x * (kCopyBatch * kFoldSoftmax) + tid; k0 < items; k0 += (int)gridDim.x * (kCopyBatch * kFoldSoftmax)) {
-        uint4 xk[kCopyBatch], xv[kCopyBatch];
-        size_t dst[kCopyBatch];
-        bool on[kCopyBatch];
-#pragma unroll
-        for (int u = 0; u < kCopyBatch; ++u) {
-          const int k = k0 + u * kFoldSoftmax, ul = k / span, w = k - ul * span, r = w / vpr, c = w - r * vpr;
-          const int i = ul / p.L, l = ul - i * p.L;
-          on[u] = k < items && r < min(srows[i], p.W);
-          if (on[u]) {
-            const int n = srows[i];
-            int slot = sslot[i] + r;
-            if (slot >= p.W) slot -= p.W;
-            dst[u] = ((((size_t)(p.b0 + i) * p.L + l) * p.nkv + (c >> 4)) * p.W + slot) * kFoldD + (size_t)(c & 15) * 8;
-            const size_t src = (((size_t)ul * p.rows + (n - min(n, p.W)) + r) * vpr + c) * 8;
-            xk[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.k) + src);
-            xv[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.v) + src);
-          }
-        }
-#pragma unroll
-        for (int u = 0; u < kCopyBatch; ++u)
-          if (on[u]) {
-            *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_k) + dst[u]) = xk[u];
-            *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_v) + dst[u]) = xv[u];
-          }
-      }
-      if (p.h)
-        for (int ul = (int)blockIdx.x; ul < p.nreq * p.L; ul += (int)gridDim.x) {
-          const int i = ul / p.L, n = srows[i];
-          if (n == 0) continue;
-          const bf16* hin = static_cast<const bf16*>(p.hid) + ((size_t)ul * p.h_rows + (p.h_rows == 1 ? 0 : n - 1)) * p.H;
-          bf16* hout = static_cast<bf16*>(p.h) + ((size_t)p.b0 * p.L + ul) * p.H;
-          for (int k = tid * 8; k < p.H; k += kFoldSoftmax * 8)
-            *reinterpret_cast<uint4*>(hout + k) = *reinterpret_cast<const uint4*>(hin + k);
-        }
-    }
 
     int n = 0;
     bool first_piece = true;
@@ -497,7 +473,7 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
           }
           move = softmax_any(mx * sl2 > kRefSlack);
           // P and the accumulator are free once the previous block's MMAs are done
-          fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
+          if (CW != QH || move || since == kFlushBlocks) fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
           if (move || since == kFlushBlocks) {
             drain();
             since = 0;
@@ -528,29 +504,45 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
             }
           }
         }
-        // P = high + remainder (bf16 each), eight queries a 16-byte store
+        // P = high + remainder (bf16 each), eight queries a 16-byte store; where a
+        // thread holds all its scores, P is formed under the previous block's
+        // MMAs and waits for them only here
+        auto weights = [&](int cc, int c, uint32_t* hi, uint32_t* lo) {
+          const float4 ra = *reinterpret_cast<const float4*>(sref + c0 + cc + c);
+          const float4 rb = *reinterpret_cast<const float4*>(sref + c0 + cc + c + 4);
+          const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
 #pragma unroll
-        for (int cc = 0; cc < QH; cc += CW) {
-          if (CW != QH) load(cc);
+          for (int e = 0; e < 8; e += 2) {
+            const float x0 = fold_ex2((s[c + e] - r[e]) * sl2), x1 = fold_ex2((s[c + e + 1] - r[e + 1]) * sl2);
+            sum[cc + c + e] += x0;
+            sum[cc + c + e + 1] += x1;
+            const uint32_t h = pack_bf16(x0, x1);
+            hi[e >> 1] = h;
+            lo[e >> 1] = pack_bf16(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u));
+          }
+        };
+        auto store_p = [&](int col, const uint32_t* hi, const uint32_t* lo) {
+          const uint32_t a = prow + (uint32_t)(col >> 6) * 16384u + (uint32_t)((((col & 63) >> 3) ^ (j & 7)) << 4);
+          st_v4(a, hi[0], hi[1], hi[2], hi[3]);
+          st_v4(a + (uint32_t)(NB * 16384), lo[0], lo[1], lo[2], lo[3]);
+        };
+        if constexpr (CW == QH) {
+          uint32_t hi[QH / 2], lo[QH / 2];
 #pragma unroll
-          for (int c = 0; c < CW; c += 8) {
-            const float4 ra = *reinterpret_cast<const float4*>(sref + c0 + cc + c);
-            const float4 rb = *reinterpret_cast<const float4*>(sref + c0 + cc + c + 4);
-            const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
-            uint32_t hi[4], lo[4];
+          for (int c = 0; c < QH; c += 8) weights(0, c, hi + c / 2, lo + c / 2);
+          if (i > 0) fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
 #pragma unroll
-            for (int e = 0; e < 8; e += 2) {
-              const float x0 = fold_ex2((s[c + e] - r[e]) * sl2), x1 = fold_ex2((s[c + e + 1] - r[e + 1]) * sl2);
-              sum[cc + c + e] += x0;
-              sum[cc + c + e + 1] += x1;
-              const uint32_t h = pack_bf16(x0, x1);
-              hi[e >> 1] = h;
-              lo[e >> 1] = pack_bf16(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u));
+          for (int c = 0; c < QH; c += 8) store_p(c0 + c, hi + c / 2, lo + c / 2);
+        } else {
+#pragma unroll
+          for (int cc = 0; cc < QH; cc += CW) {
+            load(cc);
+#pragma unroll
+            for (int c = 0; c < CW; c += 8) {
+              uint32_t hi[4], lo[4];
+              weights(cc, c, hi, lo);
+              store_p(c0 + cc + c, hi, lo);
             }
-            const int col = c0 + cc + c;
-            const uint32_t a = prow + (uint32_t)(col >> 6) * 16384u + (uint32_t)((((col & 63) >> 3) ^ (j & 7)) << 4);
-            st_v4(a, hi[0], hi[1], hi[2], hi[3]);
-            st_v4(a + (uint32_t)(NB * 16384), lo[0], lo[1], lo[2], lo[3]);
           }
         }
         tc_fence_before();
@@ -592,6 +584,58 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
       }
       f += pc.n;
     }
+  }
+
+  // ---- window ring (row q of the prefix in slot q mod W) and boundary rows: warps
+  // 10 and 11 from the start, and the softmax warps once their blocks are done
+  // (a long fold hides the copy under its blocks, in a short one it is most of the
+  // work).  A warp takes kCopyBatch x 32 vectors of the CTA's share at a time.
+  if (warp < 8 || warp >= 10) {
+    if (p.acc && blockIdx.x == 0 && warp == 10)
+      for (int i = lane; i < p.nreq; i += 32)
+        if (p.acc[i] < 0 || p.acc[i] > p.rows) set_err(p.err, LSP_DEV_BAD_DELTA);
+    const int vpr = p.nkv * (kFoldD / 8), span = p.W * vpr;     // 16-byte vectors of a row (all KV heads), of a window
+    const int items = p.nreq * p.L * span;
+    for (;;) {
+      int c = lane == 0 ? atomicAdd(scopy, 1) : 0;
+      c = __shfl_sync(0xffffffffu, c, 0);
+      const long long first = ((long long)c * gridDim.x + blockIdx.x) * (kCopyBatch * 32);
+      if (first >= items) break;
+      const int k0 = (int)first + lane;
+      uint4 xk[kCopyBatch], xv[kCopyBatch];
+      size_t dst[kCopyBatch];
+      bool on[kCopyBatch];
+#pragma unroll
+      for (int u = 0; u < kCopyBatch; ++u) {
+        const int k = k0 + u * 32, ul = k / span, w = k - ul * span, r = w / vpr, v = w - r * vpr;
+        const int i = ul / p.L, l = ul - i * p.L;
+        on[u] = k < items && r < min(srows[i], p.W);
+        if (on[u]) {
+          const int n = srows[i];
+          int slot = sslot[i] + r;
+          if (slot >= p.W) slot -= p.W;
+          dst[u] = ((((size_t)(p.b0 + i) * p.L + l) * p.nkv + (v >> 4)) * p.W + slot) * kFoldD + (size_t)(v & 15) * 8;
+          const size_t src = (((size_t)ul * p.rows + (n - min(n, p.W)) + r) * vpr + v) * 8;
+          xk[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.k) + src);
+          xv[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.v) + src);
+        }
+      }
+#pragma unroll
+      for (int u = 0; u < kCopyBatch; ++u)
+        if (on[u]) {
+          *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_k) + dst[u]) = xk[u];
+          *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_v) + dst[u]) = xv[u];
+        }
+    }
+    if (p.h && warp >= 10)
+      for (int ul = (int)blockIdx.x; ul < p.nreq * p.L; ul += (int)gridDim.x) {
+        const int i = ul / p.L, n = srows[i];
+        if (n == 0) continue;
+        const bf16* hin = static_cast<const bf16*>(p.hid) + ((size_t)ul * p.h_rows + (p.h_rows == 1 ? 0 : n - 1)) * p.H;
+        bf16* hout = static_cast<bf16*>(p.h) + ((size_t)p.b0 * p.L + ul) * p.H;
+        for (int k = (tid - (kFoldSoftmax + 64)) * 8; k < p.H; k += kFoldCopy * 8)
+          *reinterpret_cast<uint4*>(hout + k) = *reinterpret_cast<const uint4*>(hin + k);
+      }
   }
 
   tc_fence_before();
