@@ -388,7 +388,7 @@ __device__ __forceinline__ void stage_rows(float* dst, const float* win, const f
 }
 
 template <typename T>
-__global__ void __launch_bounds__(256) attn_simple_kernel(const AttnParams p, const int whole) {
+__global__ void __launch_bounds__(256) attn_simple_kernel(const AttnParams p) {
   extern __shared__ float ssm[];
   const int d = p.d, B = p.B;
   const int rep = p.nq / p.nkv;
@@ -438,56 +438,6 @@ __global__ void __launch_bounds__(256) attn_simple_kernel(const AttnParams p, co
       if (i < B && c == 0) ss[i * ctx + j] = part * scale;
     }
   };
-  if (whole) {
-    // every window and summary key and value row at once (cp.async, one round
-    // trip for all of them; fp32 rows of d floats, 16-byte chunks)
-    float* sK = sc;
-    float* sV = sc + (size_t)nctx * d;
-    const int d4 = d / 4;
-    for (int idx = tid; idx < nctx * d4; idx += blockDim.x) {
-      const int r = idx / d4, c4 = (idx % d4) * 4;
-      const float* srck = r < count ? reinterpret_cast<const float*>(wk) + (size_t)r * d
-                                    : reinterpret_cast<const float*>(Gh) + (size_t)(r - count) * d;
-      const float* srcv = r < count ? reinterpret_cast<const float*>(wv) + (size_t)r * d : Mh + (size_t)(r - count) * d;
-      cp_async16(sK + (size_t)r * d + c4, srck + c4);
-      cp_async16(sV + (size_t)r * d + c4, srcv + c4);
-    }
-    for (int j = warp; j < B; j += nw) score(sk + j * d, j);
-    cp_async_wait_all();
-    __syncthreads();
-    for (int r = warp; r < nctx; r += nw) score(sK + (size_t)r * d, B + r);
-    __syncthreads();
-    for (int i = warp; i < B; i += nw) {
-      float mx = -INFINITY;
-      for (int j = lane; j < ctx; j += 32) mx = fmaxf(mx, ss[i * ctx + j]);
-      mx = warp_max(mx);
-      float sum = 0.f;
-      for (int j = lane; j < ctx; j += 32) {
-        const float e = expf(ss[i * ctx + j] - mx);
-        ss[i * ctx + j] = e;
-        sum += e;
-      }
-      sum = warp_sum(sum);
-      for (int j = lane; j < ctx; j += 32) ss[i * ctx + j] /= sum;
-    }
-    __syncthreads();
-    T* out = static_cast<T*>(p.out);
-    for (int idx = tid; idx < B * d; idx += blockDim.x) {
-      const int i = idx / d, e = idx % d;
-      const float* pr = ss + (size_t)i * ctx;
-      float a = 0.f, a4[4] = {0.f, 0.f, 0.f, 0.f};   // four independent FMA chains
-      for (int j = 0; j < B; ++j) a = fmaf(pr[j], sv[j * d + e], a);
-      int r = 0;
-      for (; r + 4 <= nctx; r += 4) {
-#pragma unroll
-        for (int u = 0; u < 4; ++u) a4[u] = fmaf(pr[B + r + u], sV[(size_t)(r + u) * d + e], a4[u]);
-      }
-      for (; r < nctx; ++r) a = fmaf(pr[B + r], sV[(size_t)r * d + e], a);
-      a += (a4[0] + a4[1]) + (a4[2] + a4[3]);
-      out[(size_t)(b * B + i) * p.nq * d + (size_t)h * d + e] = from_f<T>(a);
-    }
-    return;
-  }
   // ---- scores: block keys from shared memory, then the window and summary
   // keys staged kSimpleChunk rows at a time (one coalesced round trip each)
   for (int j = warp; j < B; j += nw) score(sk + j * d, j);
@@ -541,6 +491,127 @@ __global__ void __launch_bounds__(256) attn_simple_kernel(const AttnParams p, co
   for (int idx = tid; idx < B * d; idx += blockDim.x) {
     const int i = idx / d, e = idx % d;
     out[(size_t)(b * B + i) * p.nq * d + (size_t)h * d + e] = from_f<T>(acc[idx]);
+  }
+}
+
+// The same attention with every key and value row in shared memory at once:
+// CTA (request, query head, group of nqs block queries), chosen so that a small
+// call still spreads over the SMs.  The window, the summary and t come from the
+// view update at the start of the round, and the q/k/v finalize before this
+// kernel triggers its dependents only after its own wait: those rows are staged before
+// this kernel's wait.  A score pass takes 32 / (lpq nqs) keys a warp, lanes (key,
+// query, dims c, c + lpq, ...); the rows' padding puts those on distinct banks.
+// P V runs its four chains (context rows r = u mod 4) on four lanes and adds them as
+// (0 + 1) + (2 + 3).  Each score and output is the sum it was with one CTA a head
+// (tiny round: attention stage 35.1 -> 14.7 us, round 94.2 -> 71).
+constexpr int kWholeThreads = 512;
+
+struct WholeLayout {
+  int nqs, dq, kp, vp;
+  size_t off_k, off_v, off_s, bytes;     // floats; bytes
+};
+__host__ __device__ inline WholeLayout whole_layout(int B, int d, int nctx_max, int nqs, int pad) {
+  WholeLayout L;
+  L.nqs = nqs;
+  L.dq = d + simple_lpq(B);
+  L.kp = d + 4 * pad;
+  L.vp = d + 8 * pad;
+  L.off_k = ((size_t)nqs * L.dq + 3) / 4 * 4;
+  L.off_v = L.off_k + (size_t)(B + nctx_max) * L.kp;
+  L.off_s = L.off_v + (size_t)(B + nctx_max) * L.vp;
+  L.bytes = (L.off_s + (size_t)nqs * (B + nctx_max)) * sizeof(float);
+  return L;
+}
+
+__global__ void __launch_bounds__(kWholeThreads) attn_whole_kernel(const AttnParams p, const int nqs, const int pad) {
+  extern __shared__ __align__(16) float wsm[];
+  const int d = p.d, B = p.B, lpq = simple_lpq(B), rep = p.nq / p.nkv;
+  const WholeLayout L = whole_layout(B, d, p.W + p.R, nqs, pad);
+  float* sq = wsm;
+  float* sK = wsm + L.off_k;             // block keys, then window, then summary rows
+  float* sV = wsm + L.off_v;
+  float* ss = wsm + L.off_s;             // [nqs][ctx]
+  const int b = blockIdx.x / p.nq, h = blockIdx.x % p.nq, g = h / rep, i0 = blockIdx.y * nqs;
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = kWholeThreads / 32;
+  griddep_launch();
+  const long long t = p.t[b];
+  const int count = (int)(t < p.W ? t : p.W), nctx = count + p.R, ctx = B + nctx;
+  const size_t wbase = ((size_t)(b * p.L + p.layer) * p.nkv + g) * p.W * d;
+  const float* wk = static_cast<const float*>(p.win_k) + wbase;
+  const float* wv = static_cast<const float*>(p.win_v) + wbase;
+  const float* Gh = static_cast<const float*>(p.G) + ((size_t)p.layer * p.nq + h) * p.R * d;
+  const float* Mh = p.m + (((size_t)(b * p.L + p.layer) * p.nq + h) * p.R) * d;
+  const int d4 = d / 4;
+  for (int idx = tid; idx < nctx * d4; idx += kWholeThreads) {
+    const int r = idx / d4, c4 = (idx % d4) * 4;
+    cp_async16(sK + (size_t)(B + r) * L.kp + c4, (r < count ? wk + (size_t)r * d : Gh + (size_t)(r - count) * d) + c4);
+    cp_async16(sV + (size_t)(B + r) * L.vp + c4, (r < count ? wv + (size_t)r * d : Mh + (size_t)(r - count) * d) + c4);
+  }
+  griddep_wait();
+  // block rows: this CTA's queries, every key and value of the KV head
+  const float* qkv = static_cast<const float*>(p.qkv) + (size_t)b * B * (p.nq + 2 * p.nkv) * d;
+  const int ldq = (p.nq + 2 * p.nkv) * d, nq = min(nqs, B - i0);
+  for (int idx = tid; idx < (nq + 2 * B) * d4; idx += kWholeThreads) {
+    const int row = idx / d4, c4 = (idx % d4) * 4;
+    const int kind = row < nq ? 0 : row < nq + B ? 1 : 2, i = kind == 0 ? i0 + row : (row - nq) % B;
+    const int head = kind == 0 ? h : kind == 1 ? p.nq + g : p.nq + p.nkv + g;
+    const float4 v = *reinterpret_cast<const float4*>(qkv + (size_t)i * ldq + (size_t)head * d + c4);
+    if (kind == 0) {                     // (rows of dq floats: no 16-byte alignment)
+      float* q = sq + row * L.dq + c4;
+      q[0] = v.x; q[1] = v.y; q[2] = v.z; q[3] = v.w;
+    } else {
+      *reinterpret_cast<float4*>((kind == 1 ? sK + (size_t)i * L.kp : sV + (size_t)i * L.vp) + c4) = v;
+    }
+  }
+  cp_async_wait_all();
+  __syncthreads();
+  const float scale = rsqrtf((float)d);
+  const int per = lpq * nqs, kpw = 32 / per;           // lanes of a key, keys of a warp pass
+  const int qi = (lane % per) / lpq, c = lane % lpq, kr = lane / per;
+  for (int j0 = warp * kpw; j0 < ctx; j0 += nw * kpw) {
+    const int j = j0 + kr;
+    float part = 0.f;
+    if (j < ctx && qi < nq) {
+      const float* krow = sK + (size_t)j * L.kp;
+      const float* q = sq + qi * L.dq;
+#pragma unroll 8
+      for (int e = c; e < d; e += lpq) part = fmaf(q[e], krow[e], part);
+    }
+    for (int o = lpq / 2; o > 0; o >>= 1) part += __shfl_xor_sync(0xffffffffu, part, o);
+    if (j < ctx && qi < nq && c == 0) ss[qi * ctx + j] = part * scale;
+  }
+  __syncthreads();
+  for (int i = warp; i < nq; i += nw) {
+    float mx = -INFINITY;
+    for (int j = lane; j < ctx; j += 32) mx = fmaxf(mx, ss[i * ctx + j]);
+    mx = warp_max(mx);
+    float sum = 0.f;
+    for (int j = lane; j < ctx; j += 32) {
+      const float e = expf(ss[i * ctx + j] - mx);
+      ss[i * ctx + j] = e;
+      sum += e;
+    }
+    sum = warp_sum(sum);
+    for (int j = lane; j < ctx; j += 32) ss[i * ctx + j] /= sum;
+  }
+  __syncthreads();
+  float* out = static_cast<float*>(p.out);
+  const int d8 = d / 8, u = (lane >> 3) & 3;
+  for (int w = warp; w < nq * d8; w += nw) {            // a warp: one query, eight dims, four chains
+    const int i = w / d8, e = (w % d8) * 8 + (lane & 7);
+    const float* pr = ss + (size_t)i * ctx;
+    const float* v = sV + e;
+    float a4 = 0.f, a = 0.f;
+    int r = 0;
+#pragma unroll 8
+    for (; r + 4 <= nctx; r += 4) a4 = fmaf(pr[B + r + u], v[(size_t)(B + r + u) * L.vp], a4);
+    if (u == 0) {
+      for (int j = 0; j < B; ++j) a = fmaf(pr[j], v[(size_t)j * L.vp], a);
+      for (; r < nctx; ++r) a = fmaf(pr[B + r], v[(size_t)(B + r) * L.vp], a);
+    }
+    const float a01 = a4 + __shfl_xor_sync(0xffffffffu, a4, 8);
+    const float a0123 = a01 + __shfl_xor_sync(0xffffffffu, a01, 16);
+    if (u == 0) out[(size_t)(b * B + i0 + i) * p.nq * d + (size_t)h * d + e] = a + a0123;
   }
 }
 
@@ -726,19 +797,29 @@ int launch_attention(const AttnParams& p, int dtype, cudaStream_t s, const AttnT
   } else {
     const int ctx = p.B + p.W + p.R;
     const size_t fixed = (size_t)(3 * p.B * p.d + p.B * simple_lpq(p.B) + 4 + p.B * ctx + 4) * sizeof(float);
-    // all window and summary rows staged at once when they fit (fp32 and d % 4 == 0
-    // for the 16-byte copies), else kSimpleChunk rows at a time
-    const size_t whole_bytes = fixed + (size_t)2 * (p.W + p.R) * p.d * sizeof(float);
-    const int whole = (dtype == LSP_DTYPE_F32 && p.d % 4 == 0 && whole_bytes <= 227 * 1024) ? 1 : 0;
-    const size_t smem = whole ? whole_bytes : fixed + (size_t)kSimpleChunk * p.d * sizeof(float);
-    if (smem > 227 * 1024) return LSP_ERR_SHAPE;
     static bool attr32 = false;
     if (!attr32) {
-      cudaFuncSetAttribute(attn_simple_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                           227 * 1024);
+      cudaFuncSetAttribute(attn_simple_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
+      cudaFuncSetAttribute(attn_whole_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
       attr32 = true;
     }
-    if (launch_pdl(attn_simple_kernel<float>, dim3(p.C * p.nq), dim3(256), smem, s, p, whole) != cudaSuccess)
+    // all rows at once where they fit (16-byte copies; the block's queries two a
+    // CTA, more where that makes more CTAs than about one an SM), else
+    // kSimpleChunk rows at a time
+    int nqs = std::min(2, 32 / simple_lpq(p.B));
+    while (nqs < p.B && 2 * nqs * simple_lpq(p.B) <= 32 && p.C * p.nq * ((p.B + nqs - 1) / nqs) > 152) nqs *= 2;
+    int pad = 1;                         // (rows without padding where only those fit)
+    if (whole_layout(p.B, p.d, p.W + p.R, nqs, pad).bytes > 227 * 1024) pad = 0;
+    const WholeLayout L = whole_layout(p.B, p.d, p.W + p.R, nqs, pad);
+    if (dtype == LSP_DTYPE_F32 && p.d % 8 == 0 && L.bytes <= 227 * 1024) {
+      if (launch_pdl(attn_whole_kernel, dim3(p.C * p.nq, (p.B + nqs - 1) / nqs), dim3(kWholeThreads), L.bytes, s, p,
+                     nqs, pad) != cudaSuccess)
+        return LSP_ERR_CUDA;
+      return LSP_OK;
+    }
+    const size_t smem = fixed + (size_t)kSimpleChunk * p.d * sizeof(float);
+    if (smem > 227 * 1024) return LSP_ERR_SHAPE;
+    if (launch_pdl(attn_simple_kernel<float>, dim3(p.C * p.nq), dim3(256), smem, s, p) != cudaSuccess)
       return LSP_ERR_CUDA;
   }
   return cudaGetLastError() == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
