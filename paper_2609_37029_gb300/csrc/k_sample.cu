@@ -285,8 +285,7 @@ constexpr int kPPairsPerWarp = 2;
 constexpr int kPMaxPairs = kPWarps * kPPairsPerWarp; // 32-row vocabulary tiles a CTA: 1024 rows
 constexpr int kPGroup = 8;                           // requests of a group (mma N)
 constexpr int kPMaxC = kPGroup * kPMaxGroups;
-constexpr int kSlotStride = 16;                      // (fp32 kernel) u64 words between step keys
-constexpr int kIdxBits = 18, kTagBits = 14;          // low half of an exchanged key: ~index, step tag
+constexpr int kIdxBits = 20, kTagBits = 12;          // low half of an exchanged key: ~index, step tag
 constexpr int kAnsCopies = 8;                        // copies of the answers
 constexpr int kLeadBatch = 5;                        // slots a leader's lane has in flight (152 CTAs in one go)
 // named barriers of the compute warps with one more warp: 1 + group, a step's keys (-> control); 3 + group,
@@ -317,12 +316,6 @@ __device__ __forceinline__ unsigned long long warp_max_key(unsigned long long k)
   return ((unsigned long long)hi << 32) | lo;
 }
 
-__device__ __forceinline__ unsigned ld_acquire_u32(const unsigned* p) {
-  unsigned v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-
 __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long long* p) {
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
@@ -333,22 +326,8 @@ __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned l
   asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
 }
 
-__device__ __forceinline__ void red_release_add(unsigned* p, unsigned v) {
-  asm volatile("red.release.gpu.global.add.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
-}
-
 __device__ __forceinline__ void named_arrive(int id, int count) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "r"(count) : "memory");
-}
-
-// Wait (every lane of a warp, same address) until *c >= target; false after kWaitLimitNs.
-__device__ __forceinline__ bool wait_count(const unsigned* c, unsigned target) {
-  if (ld_acquire_u32(c) >= target) return true;
-  const uint64_t t0 = global_ns();
-  for (uint32_t i = 1;; ++i) {
-    if (ld_acquire_u32(c) >= target) return true;
-    if ((i & 63u) == 0 && global_ns() - t0 > kWaitLimitNs) return false;
-  }
 }
 
 // Control warp: E_c rows of the group's current tokens (lane r < C holds y_r)
@@ -705,14 +684,15 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
 // ------------------------------------------------------------------ persistent kernel, fp32 storage
 // One cooperative launch for all B steps with fp32 W_c / E_c (the fp32
 // reference shape): CTA k owns 16-row vocabulary tiles [t_begin, t_begin +
-// cnt) and keeps their W_c rows resident in shared memory.  Per step, a warp
-// takes one request at a time: its lanes form z = z^(0) + W_c[v] . E_c(y)
-// (fp32 FMA) over the slice, write the corrected logits, add the noise and
-// keep a running argmax, which the warp publishes as one 64-bit atomicMax key.
-// Thread 0 then arrives on the step's counter (release) and waits, bounded,
-// for every CTA; y_i is read back from the keys and E_c(y_i) gathered for the
-// next step.  The synchronisation words are those of the bf16 kernel and are
-// left zero at exit.
+// cnt) and keeps their W_c rows resident in shared memory (a float4 of padding puts
+// the rows that lanes read together on different banks).  A warp takes its
+// requests through all steps on its own: its lanes form z = z^(0) + W_c[v] .
+// E_c(y) (fp32 FMA) over the slice, write the corrected logits, add the noise and
+// keep a running argmax; the CTA's best goes into its slot as one tagged word,
+// the warp reads the slots of all CTAs until they carry the step's tag (as in
+// the bf16 loop), and gathers E_c(y_i) for the next step.  No barrier after the
+// start, and one hop through L2 instead of atomic key, release add, count and key
+// (tiny round: 27 -> 17 us for 8 steps).
 constexpr int kPfThreads = 256;
 
 __global__ void __launch_bounds__(kPfThreads, 1)
@@ -722,42 +702,43 @@ __global__ void __launch_bounds__(kPfThreads, 1)
   const int nblk = gridDim.x;
   const int t_begin = (int)(((long long)blockIdx.x * ntiles) / nblk);
   const int cnt = (int)(((long long)(blockIdx.x + 1) * ntiles) / nblk) - t_begin;
-  const int C = p.C, B = p.B, V = p.V, rc = p.rc;
+  const int C = p.C, B = p.B, V = p.V, rc = p.rc, wp = rc + 4;
   const int v0 = t_begin * 16, nv = cnt * 16;
-  float* Ws = pfs;                                  // [nv][rc]
-  float* Es = Ws + (size_t)nv * rc;                 // [C][rc]
-  __shared__ int s_y[kPMaxC];
-  __shared__ int s_ok;
-  unsigned long long* slots = p.sync;
-  unsigned* counts = reinterpret_cast<unsigned*>(p.sync + (size_t)B * kPMaxC * kSlotStride);
+  float* Ws = pfs;                                  // [nv][wp]
+  float* Es = Ws + (size_t)nv * wp;                 // [C][rc]
   const float* Wc = static_cast<const float*>(p.Wc);
   const float* Ec = static_cast<const float*>(p.Ec);
   const bool sample = p.temperature > 0.f;
   const float inv_temp = sample ? 1.0f / p.temperature : 1.0f;
   const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
+  constexpr unsigned long long kTagMask = (1ull << kTagBits) - 1;
 
-  for (int i = tid; i < nv * rc / 4; i += kPfThreads)
-    reinterpret_cast<float4*>(Ws)[i] = reinterpret_cast<const float4*>(Wc + (size_t)v0 * rc)[i];
-  if (tid < C) {
-    int y = p.prev[(size_t)tid * p.prev_stride];
+  const unsigned epoch = *reinterpret_cast<volatile unsigned*>(p.sync);
+  const int r4 = rc / 4;
+  for (int i = tid; i < nv * r4; i += kPfThreads)
+    *reinterpret_cast<float4*>(Ws + (size_t)(i / r4) * wp + 4 * (i % r4)) = reinterpret_cast<const float4*>(Wc + (size_t)v0 * rc)[i];
+  for (int c = warp; c < C; c += nw) {
+    int y = p.prev[(size_t)c * p.prev_stride];
     if (y < 0 || y >= V) {
-      if (blockIdx.x == 0) set_err(p.err, LSP_DEV_BAD_TOKEN);
+      if (blockIdx.x == 0 && lane == 0) set_err(p.err, LSP_DEV_BAD_TOKEN);
       y = 0;
     }
-    s_y[tid] = y;
+    for (int i = lane; i < rc; i += 32) Es[c * rc + i] = Ec[(size_t)y * rc + i];
   }
-  __syncthreads();
+  __syncthreads();                                  // W_c is here, and every warp has read the epoch
   for (int s = 0; s < B; ++s) {
-    for (int i = tid; i < C * rc; i += kPfThreads) Es[i] = Ec[(size_t)s_y[i / rc] * rc + i % rc];
-    __syncthreads();
+    const unsigned long long tag = (unsigned long long)(epoch + s + 1) & kTagMask;
+    unsigned long long* slots = p.slots + (size_t)(s & 1) * C * nblk;   // [request][CTA]
     for (int c = warp; c < C; c += nw) {
       const float* zr = p.src + ((size_t)c * B + s) * V;
       float bv = -INFINITY;
       int bi = 0x7fffffff;
       for (int v = v0 + lane; v < v0 + nv; v += 32) {
-        const float* w = Ws + (size_t)(v - v0) * rc;
+        const float z0 = zr[v];
+        const float* w = Ws + (size_t)(v - v0) * wp;
         const float* e = Es + (size_t)c * rc;
         float corr = 0.f;
+#pragma unroll 4
         for (int r = 0; r < rc; r += 4) {
           const float4 a = *reinterpret_cast<const float4*>(w + r), b = *reinterpret_cast<const float4*>(e + r);
           corr = fmaf(a.x, b.x, corr);
@@ -765,7 +746,7 @@ __global__ void __launch_bounds__(kPfThreads, 1)
           corr = fmaf(a.z, b.z, corr);
           corr = fmaf(a.w, b.w, corr);
         }
-        const float z = zr[v] + corr;
+        const float z = z0 + corr;
         if (p.dst) p.dst[((size_t)c * B + s) * V + v] = z;
         float sc = z;
         if (sample) {
@@ -775,35 +756,48 @@ __global__ void __launch_bounds__(kPfThreads, 1)
         }
         if (better(sc, v, bv, bi)) { bv = sc; bi = v; }
       }
-      unsigned long long k = nv > 0 && bi != 0x7fffffff ? arg_key(bv, bi) : 0ull;
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1) k = max_u64(k, __shfl_xor_sync(0xffffffffu, k, o));
-      if (lane == 0 && k) atomicMax(&slots[(s * kPMaxC + c) * kSlotStride], k);
+      const unsigned long long k = warp_max_key(bi != 0x7fffffff ? arg_key(bv, bi) : 0ull);
+      if (lane == 0)
+        st_relaxed_u64(slots + (size_t)c * nblk + blockIdx.x,
+                       (k & 0xffffffff00000000ull) | ((k & ((1ull << kIdxBits) - 1)) << kTagBits) | tag);
     }
-    __syncthreads();                                // this CTA's keys of step s are published
     const bool last = s + 1 == B;
-    if (tid == 0) {
-      red_release_add(&counts[s], 1u);
-      s_ok = (last && blockIdx.x != 0) ? 1 : (wait_count(&counts[s], (unsigned)nblk) ? 1 : 0);
-      if (!s_ok) set_err(p.err, LSP_DEV_TIMEOUT);
-    }
-    __syncthreads();
-    if (!s_ok || (last && blockIdx.x != 0)) return;   // only CTA 0 needs y_B
-    if (tid < C) {
-      int y = (int)~(uint32_t)ld_relaxed_u64(&slots[(s * kPMaxC + tid) * kSlotStride]);
-      if (y < 0 || y >= V) {                          // no key arrived: corrupt sync words
-        set_err(p.err, LSP_DEV_TIMEOUT);
-        y = 0;
+    if (last && blockIdx.x != 0) return;            // only CTA 0 needs y_B
+    for (int c = warp; c < C; c += nw) {
+      unsigned long long best = 0ull;
+      for (int c0 = 0; c0 < nblk; c0 += 32 * kLeadBatch) {
+        unsigned long long k[kLeadBatch];
+        const uint64_t t0 = global_ns();
+        for (uint32_t it = 1;; ++it) {
+          bool all = true;
+#pragma unroll
+          for (int u = 0; u < kLeadBatch; ++u) {
+            const int b = c0 + u * 32 + lane;
+            k[u] = tag;
+            if (b < nblk) k[u] = ld_relaxed_u64(slots + (size_t)c * nblk + b);
+          }
+#pragma unroll
+          for (int u = 0; u < kLeadBatch; ++u) all = all && (k[u] & kTagMask) == tag;
+          if (__all_sync(0xffffffffu, all)) break;
+          if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) {
+            if (lane == 0) set_err(p.err, LSP_DEV_TIMEOUT);
+            return;                                 // (the other warps wait for no one but the CTAs' slots)
+          }
+        }
+#pragma unroll
+        for (int u = 0; u < kLeadBatch; ++u) best = max_u64(best, k[u]);
       }
-      s_y[tid] = y;
-      if (blockIdx.x == 0) p.out_tokens[(size_t)tid * B + s] = y;
+      best = warp_max_key(best);
+      int y = (int)(~(uint32_t)(best >> kTagBits) & ((1u << kIdxBits) - 1));
+      if (y >= V) y = 0;                            // (no entry of the row compared)
+      if (blockIdx.x == 0 && lane == 0) p.out_tokens[(size_t)c * B + s] = y;
+      if (!last)
+        for (int i = lane; i < rc; i += 32) Es[c * rc + i] = Ec[(size_t)y * rc + i];
     }
-    __syncthreads();
+    __syncwarp();
   }
-  // CTA 0 after the last step: every CTA has arrived on every counter, so no
-  // one reads the sync words again -- leave them zero for the next launch
-  for (int i = tid; i < B * kPMaxC; i += kPfThreads) slots[i * kSlotStride] = 0ull;
-  for (int i = tid; i < B; i += kPfThreads) counts[i] = 0u;
+  // CTA 0's first warp has read every CTA's last keys of request 0: all of them have read the epoch
+  if (blockIdx.x == 0 && tid == 0) *reinterpret_cast<volatile unsigned*>(p.sync) = epoch + (unsigned)B;
 }
 
 __global__ void __launch_bounds__(kSampThreads) sample_final_kernel(const SampleParams p) {
@@ -851,9 +845,9 @@ size_t sample_slot_bytes(int C, int num_sms) {
   return (size_t)2 * (kAnsCopies * kPMaxC + std::min(C, kPMaxC) * num_sms) * sizeof(unsigned long long);
 }
 
+// The loops' epoch word.  (Kept at its size: lsp_sample_noalloc's documented need counts it.)
 size_t sample_sync_bytes(int B) {
-  return ((size_t)B * kPMaxC * kSlotStride * sizeof(unsigned long long) + (size_t)B * sizeof(unsigned) +
-          255) / 256 * 256;
+  return ((size_t)B * kPMaxC * 16 * sizeof(unsigned long long) + (size_t)B * sizeof(unsigned) + 255) / 256 * 256;
 }
 
 // The bf16 loop's vocabulary tiles, CTAs and shared memory.
@@ -908,7 +902,7 @@ static int launch_persistent_any(const SampleParams& p, cudaStream_t s) {
 }
 
 // The persistent kernel's shape limits (anything else takes the per-step kernel).
-static size_t persistent_f32_smem(int tpc, int rc) { return ((size_t)tpc * 16 + kPMaxC) * rc * sizeof(float); }
+static size_t persistent_f32_smem(int tpc, int rc) { return ((size_t)tpc * 16 * (rc + 4) + kPMaxC * rc) * sizeof(float); }
 
 static bool coop_ok() {
   int dev = 0, coop = 0;
@@ -919,11 +913,12 @@ static bool coop_ok() {
 // fp32 storage: the whole B-step loop in one cooperative launch when the W_c
 // slice of a CTA fits shared memory.
 static bool persistent_f32_ok(const SampleParams& p, int dtype) {
-  if (dtype != LSP_DTYPE_F32 || p.C > kPMaxC || !p.sync || p.num_sms < 1 || p.rc % 4) return false;
+  if (dtype != LSP_DTYPE_F32 || p.C > kPMaxC || !p.sync || !p.slots || p.num_sms < 1 || p.rc % 4) return false;
+  if (p.V > (1 << kIdxBits) || 2 * p.B + 2 > (1 << kTagBits)) return false;
   const int ntiles = p.V / 16;
   const int nblk = std::min(p.num_sms, ntiles);
   const int tpc = (ntiles + nblk - 1) / nblk;
-  return persistent_f32_smem(tpc, p.rc) <= 200 * 1024 && coop_ok();
+  return persistent_f32_smem(tpc, p.rc) <= 220 * 1024 && coop_ok();
 }
 
 static int launch_persistent_f32(const SampleParams& p, cudaStream_t s) {

@@ -252,9 +252,8 @@ struct SampleParams {
   int32_t* out_tokens;    // [C][B]
   float* part_val;        // [2][nblk][C]   (per-step kernel)
   int* part_idx;          // [2][nblk][C]
-  unsigned long long* sync;   // sample_sync_bytes(B), zero at first: the fp32 loop's step keys and
-                              // arrival counts (zero between launches), or the bf16 loop's epoch and answers
-  unsigned long long* slots;  // sample_slot_bytes(C, num_sms), zero at first: the bf16 loop's key slots
+  unsigned long long* sync;   // sample_sync_bytes(B), zero at first: the one-launch loops' epoch
+  unsigned long long* slots;  // sample_slot_bytes(C, num_sms), zero at first: their key slots
   unsigned* err;
   int C, B, V, rc, nblk;
   int num_sms;
