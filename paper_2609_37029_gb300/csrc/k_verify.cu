@@ -19,6 +19,16 @@
 // the request's last chunk merges the chunk winners (its counter resets
 // itself).  One wave of draw CTAs pays the merge latency once.
 //
+// verify_rows_kernel takes the row pass's place where its CTAs make several
+// waves: they come in the order of the positions, the CTA that finishes a
+// position's last chunk decides it, and CTAs of later positions of a request that
+// has rejected one end before they read anything.  Only the rows up to the first
+// rejection carry the result, and a drafter is rejected somewhere in most blocks.
+// Measured at C = 16, B = 16, V = 151936 (T = 1: 321 MB of rows): 64.5 us whatever
+// is accepted before; now 45 us where 4.8 candidates are accepted on average and 62.5
+// where all are; T = 0 30 us before, 13 at 0.5 accepted, 31 at 16.  Chunks twice as long
+// (fewer CTAs): 47 and 60, T = 0 27.
+//
 // Randomness (Philox4x32-10, key = seed): the acceptance uniform of position i
 // is word 0 of counter (0, 2^30 + i, b, round), u = ((x >> 9) + 1/2) 2^-23,
 // accepted iff u q_i(y_i) < p_i(y_i); the draw at position i uses the words of
@@ -166,6 +176,169 @@ __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyP
   }
 }
 
+// ---------------------------------------------------------------- rows up to the first rejection
+constexpr int kRowsCtasPerSm = 4;
+constexpr int kRowsBatch = 8;                 // float4 a thread in flight: 128 KB an SM
+constexpr int kRowsChunk = 2 * kRowsBatch * kVerThreads;   // float4 groups of a row a CTA takes at most
+
+// p.ctr: [C] draw counters, [C] first rejections (B + 1 - i, 0: none so far),
+// [C][B + 1] chunks done of a position; all zero between calls.
+__device__ __forceinline__ unsigned* ver_rej(const VerifyParams& p) { return p.ctr + p.C; }
+__device__ __forceinline__ unsigned* ver_done(const VerifyParams& p) { return p.ctr + 2 * p.C; }
+__device__ __forceinline__ int ver_first(const VerifyParams& p, int b) {   // first rejected position, B if none
+  const unsigned v = *reinterpret_cast<volatile unsigned*>(ver_rej(p) + b);
+  return v ? p.B + 1 - (int)v : p.B;
+}
+// Merged statistics of row r of request b by the eight lanes sub = 0 .. 7.
+__device__ __forceinline__ float ver_row_lse(const VerifyParams& p, int b, int r, int sub, bool on) {
+  const size_t base = ((size_t)b * (2 * p.B + 1) + r) * p.nst;
+  float m = -INFINITY, s = 0.f;
+  if (on)
+    for (int k = sub; k < p.nst; k += 8) lse2_combine(m, s, __ldcg(p.st_a + base + k), __ldcg(p.st_b + base + k));
+  group_lse2<8>(m, s);
+  return m + __log2f(s);
+}
+__device__ __forceinline__ int ver_row_argmax(const VerifyParams& p, int b, int r, int sub) {
+  const size_t base = ((size_t)b * (p.B + 1) + r) * p.nst;
+  float v = -INFINITY;
+  int i = INT_MAX;
+  for (int k = sub; k < p.nst; k += 8) {
+    const float kv = __ldcg(p.st_a + base + k);
+    const int ki = __ldcg(p.st_i + base + k);
+    if (ver_better(kv, ki, v, i)) { v = kv; i = ki; }
+  }
+  group_argmax<8>(v, i);
+  return i;
+}
+// Candidates outside [0, V), up to the 32 that hold the first rejection (one warp).
+__device__ __forceinline__ void flag_tokens(const VerifyParams& p, int b, int first, int lane) {
+  for (int i = lane; i < min(p.B, (first / 32 + 1) * 32); i += 32) {
+    const int y = p.y[(size_t)b * p.B + i];
+    if (y < 0 || y >= p.V) set_err(p.err, LSP_DEV_BAD_TOKEN);
+  }
+}
+__device__ __forceinline__ void ver_reset(const VerifyParams& p, int b, int lane) {
+  for (int i = lane; i <= p.B; i += 32) ver_done(p)[(size_t)b * (p.B + 1) + i] = 0u;
+  if (lane == 0) {
+    ver_rej(p)[b] = 0u;
+    p.ctr[b] = 0u;
+  }
+}
+
+template <bool kGreedy>
+__global__ void __launch_bounds__(kVerThreads, kRowsCtasPerSm) verify_rows_kernel(const VerifyParams p) {
+  __shared__ float sv[kVerThreads / 32];
+  __shared__ int si[kVerThreads / 32];
+  griddep_wait();
+  griddep_launch();
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, B = p.B, nst = p.nst;
+  // position i, then request, then (T > 0) target or draft row, then chunk
+  const int kinds = kGreedy ? 1 : 2, level = p.C * kinds * nst;
+  const int i = min((int)blockIdx.x / level, B);
+  int u = blockIdx.x - i * level;
+  const int nk = i < B ? kinds : 1, ch = u % nst;
+  u /= nst;
+  const int b = u / nk, r = u % nk == 0 ? i : B + 1 + i;
+  if (__syncthreads_or(threadIdx.x == 0 && ver_first(p, b) < i)) return;      // an earlier position was rejected
+  const int ng = p.V / 4;
+  const int g0 = (int)((long long)ch * ng / nst), g1 = (int)((long long)(ch + 1) * ng / nst);
+  const float4* z4 = reinterpret_cast<const float4*>(ver_row(p, b, r));
+  const float it2 = kGreedy ? 1.f : 1.4426950408889634f / p.temperature;     // log2(e) / T
+  float m = -INFINITY, s = 0.f;
+  int bi = INT_MAX;
+  for (int base = g0 + threadIdx.x; base < g1; base += kRowsBatch * kVerThreads) {
+    float4 x[kRowsBatch];
+#pragma unroll
+    for (int k = 0; k < kRowsBatch; ++k) {
+      const int g = base + k * kVerThreads;
+      x[k] = g < g1 ? __ldg(z4 + g) : make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    }
+    if (kGreedy) {
+#pragma unroll
+      for (int k = 0; k < kRowsBatch; ++k) {
+        // indices rise with (k, e) within a thread: a strict > keeps the lowest on ties
+        const int v0 = 4 * (base + k * kVerThreads);
+        if (x[k].x > m) { m = x[k].x; bi = v0; }
+        if (x[k].y > m) { m = x[k].y; bi = v0 + 1; }
+        if (x[k].z > m) { m = x[k].z; bi = v0 + 2; }
+        if (x[k].w > m) { m = x[k].w; bi = v0 + 3; }
+      }
+    } else {
+      float bm = -INFINITY;
+#pragma unroll
+      for (int k = 0; k < kRowsBatch; ++k) bm = fmaxf(bm, fmaxf(fmaxf(x[k].x, x[k].y), fmaxf(x[k].z, x[k].w)));
+      const float nm = fmaxf(m, bm * it2);
+      if (nm > -INFINITY) {
+        float acc = 0.f;
+#pragma unroll
+        for (int k = 0; k < kRowsBatch; ++k)
+          acc += ex2(fmaf(x[k].x, it2, -nm)) + ex2(fmaf(x[k].y, it2, -nm)) + ex2(fmaf(x[k].z, it2, -nm)) +
+                 ex2(fmaf(x[k].w, it2, -nm));
+        s = s * ex2(m - nm) + acc;
+        m = nm;
+      }
+    }
+  }
+  if (kGreedy) group_argmax<32>(m, bi);
+  else group_lse2<32>(m, s);
+  if (lane == 0) {
+    sv[warp] = m;
+    si[warp] = kGreedy ? bi : __float_as_int(s);
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  m = lane < kVerThreads / 32 ? sv[lane] : -INFINITY;
+  if (kGreedy) {
+    bi = lane < kVerThreads / 32 ? si[lane] : INT_MAX;
+    group_argmax<8>(m, bi);
+  } else {
+    s = lane < kVerThreads / 32 ? __int_as_float(si[lane]) : 0.f;
+    group_lse2<8>(m, s);
+  }
+  unsigned last = 0;
+  if (lane == 0) {
+    const size_t o = ((size_t)b * (kGreedy ? B + 1 : 2 * B + 1) + r) * nst + ch;
+    p.st_a[o] = m;
+    if (kGreedy) p.st_i[o] = bi;
+    else p.st_b[o] = s;
+    __threadfence();
+    last = i < B && atomicAdd(ver_done(p) + (size_t)b * (B + 1) + i, 1u) == (unsigned)(kinds * nst) - 1u;
+  }
+  if (!__shfl_sync(kFull, last, 0)) return;
+  // ---- this position's last chunk: accept or reject its candidate
+  __threadfence();
+  int y = p.y[(size_t)b * B + i];
+  bool rej;
+  if (kGreedy) {
+    rej = ver_row_argmax(p, b, i, lane & 7) != y;
+  } else {
+    if (y < 0 || y >= p.V) y = 0;                                   // (flagged by the draw kernel)
+    const float lse = ver_row_lse(p, b, (lane & 8) ? B + 1 + i : i, lane & 7, true);
+    const float lse_t = __shfl_sync(kFull, lse, 0), lse_q = __shfl_sync(kFull, lse, 8);
+    const float lp = p.zt[((size_t)b * (B + 1) + i) * p.V + y] * it2 - lse_t;
+    const float lq = p.zq[((size_t)b * B + i) * p.V + y] * it2 - lse_q;
+    const uint4 x = philox4x32_10(make_uint4(0u, kAcceptStream + (uint32_t)i, (uint32_t)b, p.round),
+                                  make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32)));
+    rej = !(ver_uniform(x.x) * exp2f(lq) < exp2f(lp));
+  }
+  if (lane == 0 && rej) atomicMax(ver_rej(p) + b, (unsigned)(B + 1 - i));
+}
+
+// T = 0 after verify_rows_kernel: the prefix and the emitted token of request blockIdx.x (one warp).
+__global__ void __launch_bounds__(32) verify_emit_kernel(const VerifyParams p) {
+  const int b = blockIdx.x, lane = threadIdx.x;
+  griddep_launch();
+  griddep_wait();
+  const int j = ver_first(p, b), arg = ver_row_argmax(p, b, j, lane & 7);
+  if (lane == 0) {
+    p.accepted[b] = j;
+    p.next_token[b] = arg < p.V ? arg : 0;
+  }
+  flag_tokens(p, b, j, lane);
+  __syncwarp();
+  ver_reset(p, b, lane);
+}
+
 // T = 0, CTA per request: argmax of each position (8 lanes per row), then the
 // greedy prefix and the emitted token.
 __global__ void __launch_bounds__(kVerThreads) verify_greedy_kernel(const VerifyParams p) {
@@ -215,8 +388,10 @@ __global__ void __launch_bounds__(kVerThreads) verify_greedy_kernel(const Verify
 
 // CTA (chunk, b), T > 0: decide j, then the Gumbel-max of the correction /
 // bonus draw over the chunk's vocabulary; the last chunk merges the winners.
+// kDecided: verify_rows_kernel has found j, and only row j's normalisers are needed.
+template <bool kDecided>
 __global__ void __launch_bounds__(kVerThreads, kDrawCtasPerSm) verify_draw_kernel(const VerifyParams p) {
-  __shared__ float s_lse[2 * kVerMaxB + 1];    // base-2 log-normalisers of the request's rows
+  __shared__ float s_lse[kDecided ? 2 : 2 * kVerMaxB + 1];    // base-2 log-normalisers of the request's rows
   __shared__ float sv[32];
   __shared__ int si[32];
   __shared__ int s_j;
@@ -226,10 +401,10 @@ __global__ void __launch_bounds__(kVerThreads, kDrawCtasPerSm) verify_draw_kerne
   const float it2 = 1.4426950408889634f / p.temperature;
   const uint2 key = make_uint2((uint32_t)p.seed, (uint32_t)(p.seed >> 32));
   const int B = p.B, nst = p.nst, rpr = 2 * B + 1;
-  // candidate logits: inputs of the call, complete before the row pass began,
-  // so they load while the row pass finishes
   float zy_t = 0.f, zy_q = 0.f;
-  if (warp == 0 && lane < B) {
+  if (!kDecided && warp == 0 && lane < B) {
+    // candidate logits: inputs of the call, complete before the row pass began,
+    // so they load while the row pass finishes
     int y = p.y[(size_t)b * B + lane];
     if (y < 0 || y >= p.V) {
       set_err(p.err, LSP_DEV_BAD_TOKEN);
@@ -240,51 +415,65 @@ __global__ void __launch_bounds__(kVerThreads, kDrawCtasPerSm) verify_draw_kerne
   }
   griddep_launch();
   griddep_wait();
-  {
-    const int grp = threadIdx.x >> 3, sub = threadIdx.x & 7;
-    const size_t base = (size_t)b * rpr * nst;
-    for (int r0 = 0; r0 < rpr; r0 += kVerThreads / 8) {
-      const int r = r0 + grp;
-      float m = -INFINITY, s = 0.f;
-      if (r < rpr)
-        for (int k = sub; k < nst; k += 8)
-          lse2_combine(m, s, p.st_a[base + (size_t)r * nst + k], p.st_b[base + (size_t)r * nst + k]);
-      group_lse2<8>(m, s);
-      if (r < rpr && sub == 0) s_lse[r] = m + __log2f(s);
-    }
-  }
-  __syncthreads();
-  if (warp == 0) {
-    int j = B;
-    for (int i0 = 0; i0 < B; i0 += 32) {
-      const int i = i0 + lane;
-      bool rej = false;
-      if (i < B) {
-        float zt_i = zy_t, zq_i = zy_q;
-        if (i0 > 0) {   // candidates past the first 32 (f32 configurations with B > 32)
-          int y = p.y[(size_t)b * B + i];
-          if (y < 0 || y >= p.V) {
-            set_err(p.err, LSP_DEV_BAD_TOKEN);
-            y = 0;
-          }
-          zt_i = p.zt[((size_t)b * (B + 1) + i) * p.V + y];
-          zq_i = p.zq[((size_t)b * B + i) * p.V + y];
-        }
-        // p_i(y) = 2^(z_t it2 - lse2_t), q_i(y) = 2^(z_q it2 - lse2_q)
-        const float lp = zt_i * it2 - s_lse[i];
-        const float lq = zq_i * it2 - s_lse[B + 1 + i];
-        const uint4 x = philox4x32_10(make_uint4(0u, kAcceptStream + (uint32_t)i, (uint32_t)b, p.round), key);
-        rej = !(ver_uniform(x.x) * exp2f(lq) < exp2f(lp));
+  if constexpr (kDecided) {
+    if (warp == 0) {
+      const int first = ver_first(p, b);
+      const float lse = ver_row_lse(p, b, (lane & 8) ? B + 1 + first : first, lane & 7, !(lane & 8) || first < B);
+      if (lane == 0) {
+        s_j = first;
+        s_lse[0] = lse;
       }
-      const unsigned rm = __ballot_sync(kFull, rej);
-      if (rm) { j = i0 + __ffs(rm) - 1; break; }
+      if (lane == 8) s_lse[1] = lse;
+      if (ch == 0) flag_tokens(p, b, first, lane);
     }
-    if (lane == 0) s_j = j;
+    __syncthreads();
+  } else {
+    {
+      const int grp = threadIdx.x >> 3, sub = threadIdx.x & 7;
+      const size_t base = (size_t)b * rpr * nst;
+      for (int r0 = 0; r0 < rpr; r0 += kVerThreads / 8) {
+        const int r = r0 + grp;
+        float m = -INFINITY, s = 0.f;
+        if (r < rpr)
+          for (int k = sub; k < nst; k += 8)
+            lse2_combine(m, s, p.st_a[base + (size_t)r * nst + k], p.st_b[base + (size_t)r * nst + k]);
+        group_lse2<8>(m, s);
+        if (r < rpr && sub == 0) s_lse[r] = m + __log2f(s);
+      }
+    }
+    __syncthreads();
+    if (warp == 0) {
+      int j = B;
+      for (int i0 = 0; i0 < B; i0 += 32) {
+        const int i = i0 + lane;
+        bool rej = false;
+        if (i < B) {
+          float zt_i = zy_t, zq_i = zy_q;
+          if (i0 > 0) {   // candidates past the first 32 (f32 configurations with B > 32)
+            int y = p.y[(size_t)b * B + i];
+            if (y < 0 || y >= p.V) {
+              set_err(p.err, LSP_DEV_BAD_TOKEN);
+              y = 0;
+            }
+            zt_i = p.zt[((size_t)b * (B + 1) + i) * p.V + y];
+            zq_i = p.zq[((size_t)b * B + i) * p.V + y];
+          }
+          // p_i(y) = 2^(z_t it2 - lse2_t), q_i(y) = 2^(z_q it2 - lse2_q)
+          const float lp = zt_i * it2 - s_lse[i];
+          const float lq = zq_i * it2 - s_lse[B + 1 + i];
+          const uint4 x = philox4x32_10(make_uint4(0u, kAcceptStream + (uint32_t)i, (uint32_t)b, p.round), key);
+          rej = !(ver_uniform(x.x) * exp2f(lq) < exp2f(lp));
+        }
+        const unsigned rm = __ballot_sync(kFull, rej);
+        if (rm) { j = i0 + __ffs(rm) - 1; break; }
+      }
+      if (lane == 0) s_j = j;
+    }
+    __syncthreads();
   }
-  __syncthreads();
   const int j = s_j;
   const bool corr = j < B;
-  const float lse_t = s_lse[j], lse_q = corr ? s_lse[B + 1 + j] : 0.f;
+  const float lse_t = s_lse[kDecided ? 0 : j], lse_q = corr ? s_lse[kDecided ? 1 : B + 1 + j] : 0.f;
   const float* zt = p.zt + ((size_t)b * (B + 1) + j) * p.V;
   const float* zq = corr ? p.zq + ((size_t)b * B + j) * p.V : zt;
   const int ng = p.V / 4;
@@ -354,10 +543,13 @@ __global__ void __launch_bounds__(kVerThreads, kDrawCtasPerSm) verify_draw_kerne
     if (lane == 0) {
       p.accepted[b] = j;
       p.next_token[b] = i < p.V ? i : 0;
-      atomicExch(&p.ctr[b], 0u);
+      if (!kDecided) atomicExch(&p.ctr[b], 0u);
     }
+    if (kDecided) ver_reset(p, b, lane);      // every CTA of the request has read j
   }
 }
+
+size_t verify_counter_words(int C, int B) { return (size_t)C * (B + 3); }
 
 int verify_max_stat_chunks(int V) { return std::max(1, std::min(kVerMaxStatChunks, V / 8192)); }
 
@@ -366,19 +558,33 @@ int launch_verify(const VerifyParams& p, int num_sms, cudaStream_t s) {
   const bool greedy = !(p.temperature > 0.f);
   const int rpr = greedy ? p.B + 1 : 2 * p.B + 1;
   VerifyParams q = p;
+  cudaError_t e;
+  // one wave of draw CTAs, at least one float4 group per thread
+  const int nch = std::max(1, std::min({kDrawCtasPerSm * num_sms / p.C, kVerMaxDrawChunks, std::max(1, p.V / 4 / kVerThreads)}));
+  // Rows in the order of the positions, where that makes three waves and more: with
+  // fewer CTAs every row is under way before the first position is decided.
+  const int rows_nst = std::min(verify_max_stat_chunks(p.V), (p.V / 4 + kRowsChunk - 1) / kRowsChunk);
+  const long long units = (long long)p.C * rpr * rows_nst;
+  if (units >= 3ll * kRowsCtasPerSm * num_sms && units < (1ll << 31)) {
+    q.nst = rows_nst;
+    const dim3 grid((unsigned)units), threads(kVerThreads);
+    e = greedy ? launch_pdl(verify_rows_kernel<true>, grid, threads, 0, s, q)
+               : launch_pdl(verify_rows_kernel<false>, grid, threads, 0, s, q);
+    if (e == cudaSuccess)
+      e = greedy ? launch_pdl(verify_emit_kernel, dim3(p.C), dim3(32), 0, s, q)
+                 : launch_pdl(verify_draw_kernel<true>, dim3(nch, p.C), threads, 0, s, q);
+    return e == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
+  }
   // about eight chunk CTAs per SM in all (the row pass streams; many chunks keep SMs fed)
   q.nst = std::max(1, std::min(verify_max_stat_chunks(p.V), (8 * num_sms + p.C * rpr - 1) / (p.C * rpr)));
   const dim3 grid(p.C * rpr * q.nst);
-  cudaError_t e;
   if (greedy) {
     e = launch_pdl(verify_stats_kernel<true, 8>, grid, dim3(kVerThreads), 0, s, q, rpr);
     if (e == cudaSuccess) e = launch_pdl(verify_greedy_kernel, dim3(p.C), dim3(kVerThreads), 0, s, q);
   } else {
     e = launch_pdl(verify_stats_kernel<false, 4>, grid, dim3(kVerThreads), 0, s, q, rpr);
-    // one wave of draw CTAs, at least one float4 group per thread
-    const int nch = std::max(1, std::min({kDrawCtasPerSm * num_sms / p.C, kVerMaxDrawChunks, std::max(1, p.V / 4 / kVerThreads)}));
     // (the draw kernel's pre-wait loads need the row pass to trigger after its own wait)
-    if (e == cudaSuccess) e = launch_pdl(verify_draw_kernel, dim3(nch, p.C), dim3(kVerThreads), 0, s, q);
+    if (e == cudaSuccess) e = launch_pdl(verify_draw_kernel<false>, dim3(nch, p.C), dim3(kVerThreads), 0, s, q);
   }
   return e == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;
 }

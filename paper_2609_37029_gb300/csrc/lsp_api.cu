@@ -244,7 +244,7 @@ int lsp_state_create(const lsp_config* cfg, lsp_state** out) {
   const size_t w_vsi = off; off = align256(off + ver_rows * sizeof(int));
   const size_t w_vpv = off; off = align256(off + (size_t)c.C * kVerMaxDrawChunks * sizeof(float));
   const size_t w_vpi = off; off = align256(off + (size_t)c.C * kVerMaxDrawChunks * sizeof(int));
-  const size_t w_vc = off; off = align256(off + (size_t)c.C * sizeof(unsigned));
+  const size_t w_vc = off; off = align256(off + verify_counter_words(c.C, c.B) * sizeof(unsigned));
   if (cudaMalloc(&st->ws, off) != cudaSuccess) { free_state(st); return LSP_ERR_NOMEM; }
   char* w = static_cast<char*>(st->ws);
   st->x = reinterpret_cast<float*>(w + w_x);

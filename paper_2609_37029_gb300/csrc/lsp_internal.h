@@ -228,7 +228,7 @@ struct VerifyParams {
   int nst;                  // chunks per row (set by launch_verify)
   float* part_val;          // draw partials [C][<= kVerMaxDrawChunks]
   int* part_idx;
-  unsigned* ctr;            // [C] self-resetting counters (zero between calls)
+  unsigned* ctr;            // verify_counter_words(C, B) self-resetting counters (zero between calls)
   unsigned* err;
   int C, B, V;
   float temperature;
@@ -239,6 +239,7 @@ constexpr int kVerMaxStatChunks = 32;
 constexpr int kVerMaxDrawChunks = 128;
 constexpr int kVerMaxB = 512;
 int verify_max_stat_chunks(int V);
+size_t verify_counter_words(int C, int B);
 int launch_verify(const VerifyParams& p, int num_sms, cudaStream_t s);
 
 // ------------------------------------------------------------------ sampler
