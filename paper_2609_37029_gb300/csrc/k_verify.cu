@@ -9,9 +9,11 @@
 // verify_stats_kernel: CTA (request, row, chunk) streams every logit row the
 // decision needs and writes the chunk's partial: (max, sum of 2^x) of
 // x = z log2(e) / T over the target and draft rows (T > 0), or the
-// lowest-index argmax of the target rows (T = 0).  verify_greedy_kernel
-// (T = 0): CTA per request -- merges the argmax partials and accepts the prefix
-// of candidates equal to the target argmax.  verify_draw_kernel (T > 0): CTA
+// lowest-index argmax of the target rows (T = 0).  At T = 0 the CTA that
+// finishes a request's last chunk merges the argmax partials and accepts the
+// prefix of candidates equal to the target argmax: one launch, where a second one of
+// one CTA a request made a call of the host 2 us longer (C = 4, V = 32000: 8.9 -> 7.0 us;
+// replayed from a graph 4.6 -> 5.2).  verify_draw_kernel (T > 0): CTA
 // (vocabulary chunk, request) -- merges the request's row partials, tests the
 // B candidates one lane each (the acceptance uniforms are Philox words, so
 // every CTA finds the same first rejected position j), takes the Gumbel-max
@@ -95,10 +97,56 @@ __device__ __forceinline__ void group_lse2(float& m, float& s) {
     lse2_combine(m, s, __shfl_xor_sync(kFull, m, o), __shfl_xor_sync(kFull, s, o));
 }
 
+// T = 0, the CTA that finishes a request's last chunk: argmax of each position (8
+// lanes per row), then the greedy prefix and the emitted token.
+__device__ __forceinline__ void verify_greedy(const VerifyParams& p, int b, int* s_arg) {
+  const int B = p.B, nst = p.nst, rpr = B + 1;
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  const int grp = threadIdx.x >> 3, sub = threadIdx.x & 7;
+  const size_t base = (size_t)b * rpr * nst;
+  for (int r0 = 0; r0 < rpr; r0 += kVerThreads / 8) {
+    const int r = r0 + grp;
+    float v = -INFINITY;
+    int i = INT_MAX;
+    if (r < rpr)
+      for (int k = sub; k < nst; k += 8) {
+        const float kv = __ldcg(p.st_a + base + (size_t)r * nst + k);
+        const int ki = __ldcg(p.st_i + base + (size_t)r * nst + k);
+        if (ver_better(kv, ki, v, i)) { v = kv; i = ki; }
+      }
+    group_argmax<8>(v, i);
+    if (r < rpr && sub == 0) s_arg[r] = i;
+  }
+  __syncthreads();
+  if (warp != 0) return;
+  for (int i0 = 0; i0 <= B; i0 += 32) {
+    const int i = i0 + lane;
+    bool stop = false;
+    if (i < B) {
+      const int y = p.y[(size_t)b * B + i];
+      if (y < 0 || y >= p.V) set_err(p.err, LSP_DEV_BAD_TOKEN);
+      stop = y != s_arg[i];
+    } else if (i == B) {
+      stop = true;
+    }
+    const unsigned m = __ballot_sync(kFull, stop);
+    if (m) {
+      const int j = i0 + __ffs(m) - 1;
+      if (lane == 0) {
+        p.accepted[b] = j;
+        p.next_token[b] = s_arg[j] < p.V ? s_arg[j] : 0;
+      }
+      return;
+    }
+  }
+}
+
 template <bool kGreedy, int kBatch>
 __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyParams p, const int rpr) {
   __shared__ float sv[32];
   __shared__ int si[32];
+  __shared__ int s_arg[kGreedy ? kVerMaxB + 1 : 1];
+  __shared__ int s_last;
   // dependents launch only after this grid's inputs are complete: the draw
   // kernel reads the call's inputs before its own wait
   griddep_wait();
@@ -139,7 +187,14 @@ __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyP
         if (ver_better(sv[w], si[w], bv, bi)) { bv = sv[w]; bi = si[w]; }
       p.st_a[u] = bv;
       p.st_i[u] = bi;
+      __threadfence();
+      s_last = atomicAdd(&p.ctr[b], 1u) == (unsigned)(rpr * p.nst) - 1u;
     }
+    __syncthreads();
+    if (!s_last) return;
+    __threadfence();
+    verify_greedy(p, b, s_arg);
+    if (threadIdx.x == 0) p.ctr[b] = 0u;
   } else {
     const float it2 = 1.4426950408889634f / p.temperature;   // log2(e) / T
     float m = -INFINITY, s = 0.f;
@@ -324,7 +379,9 @@ __global__ void __launch_bounds__(kVerThreads, kRowsCtasPerSm) verify_rows_kerne
   if (lane == 0 && rej) atomicMax(ver_rej(p) + b, (unsigned)(B + 1 - i));
 }
 
-// T = 0 after verify_rows_kernel: the prefix and the emitted token of request blockIdx.x (one warp).
+// T = 0 after verify_rows_kernel: the prefix and the emitted token of request
+// blockIdx.x (one warp).  A launch of its own: a count of every CTA of the request, so that
+// the last one emits, took 2.5 us more than it saves.
 __global__ void __launch_bounds__(32) verify_emit_kernel(const VerifyParams p) {
   const int b = blockIdx.x, lane = threadIdx.x;
   griddep_launch();
@@ -337,53 +394,6 @@ __global__ void __launch_bounds__(32) verify_emit_kernel(const VerifyParams p) {
   flag_tokens(p, b, j, lane);
   __syncwarp();
   ver_reset(p, b, lane);
-}
-
-// T = 0, CTA per request: argmax of each position (8 lanes per row), then the
-// greedy prefix and the emitted token.
-__global__ void __launch_bounds__(kVerThreads) verify_greedy_kernel(const VerifyParams p) {
-  __shared__ int s_arg[kVerMaxB + 1];
-  griddep_launch();
-  griddep_wait();
-  const int b = blockIdx.x, B = p.B, nst = p.nst, rpr = B + 1;
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  const int grp = threadIdx.x >> 3, sub = threadIdx.x & 7;
-  const size_t base = (size_t)b * rpr * nst;
-  for (int r0 = 0; r0 < rpr; r0 += kVerThreads / 8) {
-    const int r = r0 + grp;
-    float v = -INFINITY;
-    int i = INT_MAX;
-    if (r < rpr)
-      for (int k = sub; k < nst; k += 8)
-        if (ver_better(p.st_a[base + (size_t)r * nst + k], p.st_i[base + (size_t)r * nst + k], v, i)) {
-          v = p.st_a[base + (size_t)r * nst + k];
-          i = p.st_i[base + (size_t)r * nst + k];
-        }
-    group_argmax<8>(v, i);
-    if (r < rpr && sub == 0) s_arg[r] = i;
-  }
-  __syncthreads();
-  if (warp != 0) return;
-  for (int i0 = 0; i0 <= B; i0 += 32) {
-    const int i = i0 + lane;
-    bool stop = false;
-    if (i < B) {
-      const int y = p.y[(size_t)b * B + i];
-      if (y < 0 || y >= p.V) set_err(p.err, LSP_DEV_BAD_TOKEN);
-      stop = y != s_arg[i];
-    } else if (i == B) {
-      stop = true;
-    }
-    const unsigned m = __ballot_sync(kFull, stop);
-    if (m) {
-      const int j = i0 + __ffs(m) - 1;
-      if (lane == 0) {
-        p.accepted[b] = j;
-        p.next_token[b] = s_arg[j] < p.V ? s_arg[j] : 0;
-      }
-      return;
-    }
-  }
 }
 
 // CTA (chunk, b), T > 0: decide j, then the Gumbel-max of the correction /
@@ -580,7 +590,6 @@ int launch_verify(const VerifyParams& p, int num_sms, cudaStream_t s) {
   const dim3 grid(p.C * rpr * q.nst);
   if (greedy) {
     e = launch_pdl(verify_stats_kernel<true, 8>, grid, dim3(kVerThreads), 0, s, q, rpr);
-    if (e == cudaSuccess) e = launch_pdl(verify_greedy_kernel, dim3(p.C), dim3(kVerThreads), 0, s, q);
   } else {
     e = launch_pdl(verify_stats_kernel<false, 4>, grid, dim3(kVerThreads), 0, s, q, rpr);
     // (the draw kernel's pre-wait loads need the row pass to trigger after its own wait)
