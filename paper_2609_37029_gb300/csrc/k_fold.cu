@@ -41,18 +41,21 @@
 // only when a score passes it by 24 in base-2 units (one compare a score and
 // one barrier a block instead of a maximum across the 128 lanes for every
 // query and block).  The accumulator is drained into registers every
-// kFlushBlocks blocks and when ref moves: tcgen05 accumulation drops low bits,
-// and a short run keeps its error below that of the 2048-row segments of the
-// mma.sync kernel this replaces.
+// kFlushBlocks blocks and when ref moves, and the remainders' MMAs of a block go
+// first: tcgen05 accumulation drops low bits.  Relative error of m against 64
+// bits at 131072 / 2048 / 1999 rows: 2.8e-6 / 4.9e-7 / 2.3e-6 with 8 blocks and
+// the parts in turn, 2.1e-6 / 4.0e-7 / 2.1e-6 with 2 or 1 and the remainders
+// first (the mma.sync kernel this replaces: 4.6e-6 / 8.3e-7 / 2.0e-6); the call of
+// 131072 rows takes 450.6, 452.1 and 453.9 us with 8, 2 and 1 (460 with the
+// parts in turn).
 //
 // fold_merge_kernel merges a unit's pieces (one per CTA share that touches
 // it) and the stored state, in share order: deterministic.
 //
 // Measured (GB300, Qwen3-8B heads, 5 layers): lsp_prefill of 131072 rows
-// (2.68 GB) 745 us with the mma.sync kernel, 397 + 7 us now (6.8 TB/s, the copy
+// (2.68 GB) 745 us with the mma.sync kernel, 386 + 7 us now (6.9 TB/s, the copy
 // bandwidth); lsp_view_update of 2048 rows 232 -> 22 us for one request, 423 ->
-// 162 us for 16.  Relative error of m against 64 bits at 131072 rows: 4.6e-6 ->
-// 2.8e-6.
+// 162 us for 16.
 #include <algorithm>
 #include <type_traits>
 
@@ -69,7 +72,7 @@ constexpr int kFoldCopy = 64;                // threads that copy the window (2 
 constexpr int kFoldThreads = kFoldSoftmax + 64 + kFoldCopy;
 constexpr int kFoldSlot = kFoldKeys * 256;   // bytes of one K or V block
 constexpr int kFoldRec = 16 + 16 * kFoldD;   // floats per (piece, query head): eta[16], m[16][d]
-constexpr int kFlushBlocks = 8;
+constexpr int kFlushBlocks = 2;
 constexpr float kRefSlack = 24.f;            // log2 units a score may pass its reference by
 constexpr int kFoldMaxC = 64;
 constexpr int kCopyBatch = 4;                // window vectors a copying lane has in flight (K and V each)
@@ -364,11 +367,15 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
         const uint32_t sv = s_ring + (uint32_t)s * kFoldSlot;
         const uint32_t keep = uniform(*sfresh ? 0u : 1u);   // fresh: the accumulator was drained
         if (elect_one()) {
+          // remainders first: the accumulator is small while they are added, so the
+          // bits that each MMA's addition drops are theirs
 #pragma unroll
-          for (int ks = 0; ks < kFoldKeys / 16; ++ks) {
-            const uint64_t ad = fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2);
-            umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)ks * 2048u, 16384u), id_o, ks > 0 ? 1u : keep);
-            umma_f16(t_o, ad, fold_desc_mn(s_p + (uint32_t)(NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o, 1u);
+          for (int part = 1; part >= 0; --part) {
+#pragma unroll
+            for (int ks = 0; ks < kFoldKeys / 16; ++ks)
+              umma_f16(t_o, fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2),
+                       fold_desc_mn(s_p + (uint32_t)(part * NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o,
+                       part == 0 || ks > 0 ? 1u : keep);
           }
           umma_commit(b_empty(s));
           umma_commit(b_pv);
