@@ -267,8 +267,8 @@ def prefill_leg(wl, rows, hbm, dist, reps=5):
     del k, v, h
     return {"rows": rows, "us_per_request": us, "kv_bytes": kv, "achieved_gbs": kv / us * 1e-3,
             "frac_hbm": kv / us * 1e-3 / hbm, "flops": flops,
-            "note": "mma.sync score and value products (P V as bf16 high + remainder): "
-                    "tensor-issue bound on the legacy path, not HBM"}
+            "note": "tcgen05 score and value products (P V as bf16 high + remainder): HBM; "
+                    "the state's export copy to the host is not in it"}
 
 
 def verify_leg(wl, hbm, dist, reps=20):
@@ -294,15 +294,21 @@ def verify_leg(wl, hbm, dist, reps=20):
         e1.record()
         torch.cuda.synchronize()
         us = dist.max(e0.elapsed_time(e1) * 1e3 / reps)
-        # every row read once for its statistics, plus the emitting rows re-read by the draw
-        rows = s.C * (2 * s.B + 3) if T > 0 else s.C * (s.B + 1)
+        # the rows up to each request's first rejection (later ones are not needed), plus
+        # the emitting rows re-read by the draw
+        taken = [int(a) for a in acc.tolist()]
+        if T > 0:
+            rows = sum(2 * min(a + 1, s.B) + 2 for a in taken)
+        else:
+            rows = sum(a + 1 for a in taken)
         nbytes = rows * s.V * 4
         out[name] = {"us": us, "bytes": nbytes, "achieved_gbs": nbytes / us * 1e-3,
                      "frac_hbm": nbytes / us * 1e-3 / hbm}
     assert lsp.lsp_get_error(st) == (lsp.LSP_OK, 0)
     lsp.lsp_state_destroy(st)
     out["note"] = ("inputs %.0f MB > L2 (no flush needed); T = 1 reads target and draft rows, "
-                   "T = 0 the target rows only" % (s.C * (2 * s.B + 1) * s.V * 4 / 1e6))
+                   "T = 0 the target rows only, up to each request's first rejection"
+                   % (s.C * (2 * s.B + 1) * s.V * 4 / 1e6))
     return out
 
 

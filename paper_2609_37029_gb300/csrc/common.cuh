@@ -122,14 +122,6 @@ __device__ __forceinline__ uint64_t policy_evict_last() {
   return p;
 }
 
-// Fetch a tile of a tensor map into L2 only (no shared memory, no barrier).
-__device__ __forceinline__ void tma_prefetch_l2(const void* tmap, int x, int y) {
-  asm volatile("cp.async.bulk.prefetch.tensor.2d.L2.global.tile [%0, {%1, %2}];" ::"l"(
-                   reinterpret_cast<uint64_t>(tmap)),
-               "r"(x), "r"(y)
-               : "memory");
-}
-
 // ---------------------------------------------------------------- programmatic dependent launch
 // Wait until the preceding grid in the stream has completed and its writes are
 // visible (a no-op when the kernel was not launched as a dependent).

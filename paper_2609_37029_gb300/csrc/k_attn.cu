@@ -503,7 +503,7 @@ __global__ void __launch_bounds__(256) attn_simple_kernel(const AttnParams p) {
 // query, dims c, c + lpq, ...); the rows' padding puts those on distinct banks.
 // P V runs its four chains (context rows r = u mod 4) on four lanes and adds them as
 // (0 + 1) + (2 + 3).  Each score and output is the sum it was with one CTA a head
-// (tiny round: attention stage 35.1 -> 14.7 us, round 94.2 -> 71).
+// (tiny round: attention stage 35.1 -> 14.7 us of a 94 us round).
 constexpr int kWholeThreads = 512;
 
 struct WholeLayout {
