@@ -280,6 +280,15 @@ __global__ void __launch_bounds__(kSampThreads, 2) sample_step_kernel(const Samp
 
 // ------------------------------------------------------------------ persistent kernel
 constexpr int kPWarps = 16;                          // compute warps
+// A CTA takes 16 tiles, one a compute warp, before there are more than 32 CTAs,
+// and up to 32 every CTA reads all keys itself, a lane a CTA: one hop through
+// L2 instead of two, and fewer words to poll.  Spread over all SMs with
+// leaders -> so (us): C = 6, V = 1584, B = 16 T = 0 49.1 -> 38.0; C = 2, V = 1024
+// T = 1 40.5 -> 34.5; C = 14, V = 39200, B = 8 T = 0 46.6 -> 38.0; C = 16, V = 32000,
+// B = 16 T = 1 83.6 -> 70.4.  (Two groups at T = 0 with a middling vocabulary are
+// where the atomic exchange of before was quicker: 35.5 and, at V = 16000, 30.4
+// against 33.5 now.)
+constexpr int kPFewCtas = 32;
 constexpr int kPMaxGroups = 2;                       // request groups of eight
 constexpr int kPPairsPerWarp = 2;
 constexpr int kPMaxPairs = kPWarps * kPPairsPerWarp; // 32-row vocabulary tiles a CTA: 1024 rows
@@ -602,7 +611,8 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   // T = 1).  The answers go out in 8 copies, a 128-byte line each, that 19 CTAs read:
   // polls of one line by every CTA hold up the store they wait for (C = 8:
   // 84 us with one copy, 78 with 8, 80 with 32).  Slots alternate between two sets: a CTA writes step s + 2 only after
-  // the answer of step s + 1, which its leader gives after reading step s.
+  // the answer of step s + 1, which its leader gives after reading step s (without
+  // leaders: after every CTA's word of step s + 1).
   // Tags go on from launch to launch (the epoch word), so nothing is cleared.
   unsigned long long* answers = p.slots;                                // [2][kAnsCopies][kPMaxC]
   constexpr unsigned long long kTagMask = (1ull << kTagBits) - 1;
@@ -622,45 +632,76 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
     }
     __syncwarp();
     bool ok = true;
-    // ---- leader: the best of all CTAs
-    for (int r = r0 + ((int)blockIdx.x - r0 % nblk + nblk) % nblk; r < r0 + Cg && ok; r += nblk) {
-      unsigned long long best = 0ull;
-      for (int c0 = 0; c0 < nblk && ok; c0 += 32 * kLeadBatch) {
-        unsigned long long k[kLeadBatch];
+    const bool last = s + 1 == B;
+    unsigned long long k = tag;                                         // lane r: the best key of request r0 + r
+    if (nblk <= kPFewCtas) {
+      // ---- few CTAs: one lane a CTA, all requests at once, no leader
+      const bool writes = (int)blockIdx.x < Cg || nblk < Cg;            // (block 0 writes in both groups)
+      if (!last || writes) {
+        unsigned long long v[kPGroup];
         const uint64_t t0 = global_ns();
         for (uint32_t it = 1;; ++it) {
           bool all = true;
 #pragma unroll
-          for (int u = 0; u < kLeadBatch; ++u) {
-            const int c = c0 + u * 32 + lane;
-            k[u] = c < nblk ? ld_relaxed_u64(slots + (size_t)r * nblk + c) : tag;
-          }
+          for (int u = 0; u < kPGroup; ++u)
+            v[u] = u < Cg && lane < nblk ? ld_relaxed_u64(slots + (size_t)(r0 + u) * nblk + lane) : tag;
 #pragma unroll
-          for (int u = 0; u < kLeadBatch; ++u) all = all && (k[u] & kTagMask) == tag;
+          for (int u = 0; u < kPGroup; ++u) all = all && (v[u] & kTagMask) == tag;
           if (__all_sync(0xffffffffu, all)) break;
           if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
         }
 #pragma unroll
-        for (int u = 0; u < kLeadBatch; ++u) best = max_u64(best, k[u]);
+        for (int u = 0; u < kPGroup; ++u) {
+          const unsigned long long best = warp_max_key(v[u]);
+          if (lane == u) k = best;
+        }
+        if (ok && lane < Cg && lane % nblk == (int)blockIdx.x) {
+          const int t = (int)(~(uint32_t)(k >> kTagBits) & ((1u << kIdxBits) - 1));
+          p.out_tokens[(size_t)(r0 + lane) * B + s] = t < V ? t : 0;
+        }
       }
-      best = warp_max_key(best);
-      if (ok && lane < kAnsCopies) st_relaxed_u64(ans + lane * kPMaxC + r, best);
-      if (ok && lane == 0) {
-        const int t = (int)(~(uint32_t)(best >> kTagBits) & ((1u << kIdxBits) - 1));
-        p.out_tokens[(size_t)r * B + s] = t < V ? t : 0;
+      if (last && ok) break;
+    } else {
+      // ---- leader: the best of all CTAs
+      for (int r = r0 + ((int)blockIdx.x - r0 % nblk + nblk) % nblk; r < r0 + Cg && ok; r += nblk) {
+        unsigned long long best = 0ull;
+        for (int c0 = 0; c0 < nblk && ok; c0 += 32 * kLeadBatch) {
+          unsigned long long k[kLeadBatch];
+          const uint64_t t0 = global_ns();
+          for (uint32_t it = 1;; ++it) {
+            bool all = true;
+#pragma unroll
+            for (int u = 0; u < kLeadBatch; ++u) {
+              const int c = c0 + u * 32 + lane;
+              k[u] = c < nblk ? ld_relaxed_u64(slots + (size_t)r * nblk + c) : tag;
+            }
+#pragma unroll
+            for (int u = 0; u < kLeadBatch; ++u) all = all && (k[u] & kTagMask) == tag;
+            if (__all_sync(0xffffffffu, all)) break;
+            if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
+          }
+#pragma unroll
+          for (int u = 0; u < kLeadBatch; ++u) best = max_u64(best, k[u]);
+        }
+        best = warp_max_key(best);
+        if (ok && lane < kAnsCopies) st_relaxed_u64(ans + lane * kPMaxC + r, best);
+        if (ok && lane == 0) {
+          const int t = (int)(~(uint32_t)(best >> kTagBits) & ((1u << kIdxBits) - 1));
+          p.out_tokens[(size_t)r * B + s] = t < V ? t : 0;
+        }
+      }
+      if (last && ok) break;
+      // ---- everyone: the answers
+      if (ok) {
+        const uint64_t t0 = global_ns();
+        for (uint32_t it = 1;; ++it) {
+          if (lane < Cg) k = ld_relaxed_u64(ans + ((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane);
+          if (__all_sync(0xffffffffu, (k & kTagMask) == tag)) break;
+          if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
+        }
       }
     }
-    const bool last = s + 1 == B;
-    if (last && ok) break;
-    // ---- everyone: the answers
     if (ok) {
-      const uint64_t t0 = global_ns();
-      unsigned long long k = tag;
-      for (uint32_t it = 1;; ++it) {
-        if (lane < Cg) k = ld_relaxed_u64(ans + ((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane);
-        if (__all_sync(0xffffffffu, (k & kTagMask) == tag)) break;
-        if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
-      }
       y = (int)(~(uint32_t)(k >> kTagBits) & ((1u << kIdxBits) - 1));
       if (y >= V) y = 0;                                                // (no entry of the row compared)
     }
@@ -858,7 +899,7 @@ struct PersistentPlan {
 static PersistentPlan persistent_plan(const SampleParams& p) {
   PersistentPlan q;
   q.npairs = (p.V + 31) / 32;
-  q.nblk = std::min(p.num_sms, q.npairs);
+  q.nblk = std::min(std::min(p.num_sms, q.npairs), std::max(kPFewCtas, (q.npairs + kPWarps - 1) / kPWarps));
   q.tpc = (q.npairs + q.nblk - 1) / q.nblk;
   q.groups = p.C > kPGroup ? 2 : 1;
   const size_t rb = (size_t)p.rc * 2;
