@@ -383,7 +383,6 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   uint8_t* Es = reinterpret_cast<uint8_t*>(Zs + (size_t)NG * kPGroup * zpitch);              // [NG][8][RB]
   unsigned long long* red = reinterpret_cast<unsigned long long*>(Es + NG * kPGroup * RB);   // [NG][warps][8]
   unsigned long long* zbar = red + NG * kPWarps * kPGroup;                        // [NG] the group's logits have landed
-  volatile int* abort_flag = reinterpret_cast<volatile int*>(zbar + NG);
   const bf16* Wc = static_cast<const bf16*>(p.Wc);
   const bf16* Ec = static_cast<const bf16*>(p.Ec);
   const int C = p.C, B = p.B, V = p.V, rc = p.rc;
@@ -400,7 +399,6 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   for (int i = tid; i < NG * kPGroup * RB / 16; i += kThreads)
     reinterpret_cast<uint4*>(Es)[i] = make_uint4(0u, 0u, 0u, 0u);
   if (tid == 0) {
-    *abort_flag = 0;
     for (int h = 0; h < NG; ++h) mbar_init(smem_u32(zbar + h), 1);
     fence_barrier_init();
   }
@@ -486,22 +484,15 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
 
   if (warp < kPWarps) {
     // ================= compute warps: the groups in turn, so that one group's
-    // exchange and logits traffic run under the other's scoring and noise
+    // exchange and logits traffic run under the other's scoring and noise.  Every
+    // role passes the same barriers in every step, whatever happens: a control warp
+    // that gives up waiting goes on without the exchange, so no warp is ever left
+    // at a barrier that another has not reached.
     for (int s = 0; s < B; ++s) {
       const bool more = s + 1 < B;
 #pragma unroll
       for (int h = 0; h < NG; ++h) {
-        if (s > 0) {
-          named_bar(3 + h, kPBar);
-          if (*abort_flag) {                                            // the others wait for keys, and see the flag
-#pragma unroll
-            for (int u = 0; u < NG; ++u) {
-              named_arrive(1 + u, kPBar);
-              named_arrive(5 + u, kPBar);
-            }
-            return;
-          }
-        }
+        if (s > 0) named_bar(3 + h, kPBar);
         // B operand: E_c(y) row g of the group over this lane's k range
         uint32_t eb[2 * KS];
 #pragma unroll
@@ -582,10 +573,6 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
     // 16 requests, the bandwidth's time, with nothing under them)
     for (int s = 0; s < B; ++s) {
       named_bar(5 + grp, kPBar);
-      if (*abort_flag) {
-        mbar_wait(smem_u32(zbar + grp), (uint32_t)s & 1u, p.err);       // the load of step s may be in flight
-        return;
-      }
       if (lane < Cg && p.dst) {
         asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(
                          p.dst + ((size_t)(grp * kPGroup + lane) * B + s) * V + first),
@@ -617,12 +604,17 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   unsigned long long* answers = p.slots;                                // [2][kAnsCopies][kPMaxC]
   constexpr unsigned long long kTagMask = (1ull << kTagBits) - 1;
   const int r0 = grp * kPGroup;
+  bool ok = true;                                                       // false: a wait has given up
   for (int s = 0; s < B; ++s) {
     const unsigned long long tag = (unsigned long long)(epoch + s + 1) & kTagMask;
     unsigned long long* slots = p.slots + 2 * kAnsCopies * kPMaxC + (size_t)(s & 1) * C * nblk;   // [request][CTA]
     unsigned long long* ans = answers + (s & 1) * kAnsCopies * kPMaxC;
+    const bool last = s + 1 == B;
     named_bar(1 + grp, kPBar);
-    if (*abort_flag) return;                                            // the other group has given up
+    if (!ok) {                                                          // nothing is published any more; the others' waits end too
+      if (!last) named_arrive(3 + grp, kPBar);
+      continue;
+    }
     if (lane < Cg) {
       unsigned long long k = 0ull;
 #pragma unroll
@@ -631,8 +623,6 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
                      (k & 0xffffffff00000000ull) | ((k & ((1ull << kIdxBits) - 1)) << kTagBits) | tag);
     }
     __syncwarp();
-    bool ok = true;
-    const bool last = s + 1 == B;
     unsigned long long k = tag;                                         // lane r: the best key of request r0 + r
     if (nblk <= kPFewCtas) {
       // ---- few CTAs: one lane a CTA, all requests at once, no leader
@@ -660,7 +650,6 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
           p.out_tokens[(size_t)(r0 + lane) * B + s] = t < V ? t : 0;
         }
       }
-      if (last && ok) break;
     } else {
       // ---- leader: the best of all CTAs
       for (int r = r0 + ((int)blockIdx.x - r0 % nblk + nblk) % nblk; r < r0 + Cg && ok; r += nblk) {
@@ -690,9 +679,8 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
           p.out_tokens[(size_t)r * B + s] = t < V ? t : 0;
         }
       }
-      if (last && ok) break;
       // ---- everyone: the answers
-      if (ok) {
+      if (ok && !last) {
         const uint64_t t0 = global_ns();
         for (uint32_t it = 1;; ++it) {
           if (lane < Cg) k = ld_relaxed_u64(ans + ((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane);
@@ -701,25 +689,18 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
         }
       }
     }
+    if (!ok && lane == 0) set_err(p.err, LSP_DEV_TIMEOUT);
+    if (last) break;
     if (ok) {
       y = (int)(~(uint32_t)(k >> kTagBits) & ((1u << kIdxBits) - 1));
       if (y >= V) y = 0;                                                // (no entry of the row compared)
+      gather_e<CH>(Ec, y, Cg, rc, Es + grp * kPGroup * RB, lane);
     }
-    if (!ok) {
-      if (lane == 0) {
-        set_err(p.err, LSP_DEV_TIMEOUT);
-        *abort_flag = 1;
-      }
-      __syncwarp();
-      if (!last) named_arrive(3 + grp, kPBar);                          // releases the compute warps, and they the others
-      return;
-    }
-    gather_e<CH>(Ec, y, Cg, rc, Es + grp * kPGroup * RB, lane);
     __syncwarp();
     named_arrive(3 + grp, kPBar);
   }
   // every CTA has read the epoch before its first keys, and those have arrived here
-  if (blockIdx.x == 0 && grp == 0 && lane == 0) *reinterpret_cast<volatile unsigned*>(p.sync) = epoch + (unsigned)B;
+  if (ok && blockIdx.x == 0 && grp == 0 && lane == 0) *reinterpret_cast<volatile unsigned*>(p.sync) = epoch + (unsigned)B;
 }
 
 // ------------------------------------------------------------------ persistent kernel, fp32 storage
@@ -904,7 +885,7 @@ static PersistentPlan persistent_plan(const SampleParams& p) {
   q.groups = p.C > kPGroup ? 2 : 1;
   const size_t rb = (size_t)p.rc * 2;
   q.smem = (size_t)q.tpc * 32 * rb + (size_t)q.groups * kPGroup * (z_pitch(q.tpc) * sizeof(float) + rb) +
-           (size_t)q.groups * (kPWarps * kPGroup + 1) * sizeof(unsigned long long) + 16;
+           (size_t)q.groups * (kPWarps * kPGroup + 1) * sizeof(unsigned long long);
   return q;
 }
 
