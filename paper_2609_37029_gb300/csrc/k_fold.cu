@@ -30,8 +30,9 @@
 //               layout their producer writes, so nothing is transposed.
 //   warps 0-7   softmax: a thread owns one key (TMEM lane) and half of the
 //               queries, P = 2^((s - ref) log2(e) / sqrt(d)) is written as a
-//               bf16 high part and a bf16 remainder (two MMAs, ~16
-//               significant bits), and the sums stay in registers.
+//               bf16 high part and one or two bf16 remainders (two MMAs, ~16
+//               significant bits, or three, ~24: see fold_parts), and the sums
+//               stay in registers.
 //   warps 10-11 the window ring and the boundary rows; the softmax warps join
 //               them when their blocks are done
 //
@@ -83,21 +84,22 @@ struct FoldLayout {
   uint32_t off_p, off_ring, off_misc, bytes;
 };
 
-// bytes: G [2][16 REP][128 B], P high and remainder [64-query blocks][128][128 B],
+// bytes: G [2][16 REP][128 B], P in parts [64-query blocks][128][128 B],
 // the ring, then references, scales, block counts, rows and slots, barriers
-__host__ __device__ constexpr FoldLayout fold_layout(int rep) {
+__host__ __device__ constexpr FoldLayout fold_layout(int rep, int parts) {
   FoldLayout L{};
   const int nb = (16 * rep + 63) / 64;
   L.off_p = (uint32_t)rep * 4096u;
-  L.off_ring = L.off_p + 2u * (uint32_t)nb * 16384u;
-  const uint32_t misc = 2u * 128u * 4u + 272u + 2u * kFoldMaxC * 4u + 160u;
+  L.off_ring = L.off_p + (uint32_t)(parts * nb) * 16384u;
+  const uint32_t misc = 2u * 16u * (uint32_t)rep * 4u + 272u + 2u * kFoldMaxC * 4u + 160u;
   const int fit = (int)((227u * 1024u - 1024u - misc - L.off_ring) / (uint32_t)kFoldSlot);
   L.slots = fit < kFoldMaxSlots ? fit : kFoldMaxSlots;
   L.off_misc = L.off_ring + (uint32_t)L.slots * kFoldSlot;
   L.bytes = L.off_misc + misc + 1024u;
   return L;
 }
-static_assert(fold_layout(8).slots >= 4 && fold_layout(4).slots == 5, "K and V of two blocks fit the ring");
+static_assert(fold_layout(8, 2).slots >= 4 && fold_layout(4, 3).slots == 5, "K and V of two blocks fit the ring");
+static_assert(fold_layout(8, 3).slots >= 3, "K and V of a block and the next K fit the ring");
 
 __host__ __device__ constexpr uint32_t fold_tmem_cols(int rep) {
   uint32_t c = 32;
@@ -235,20 +237,20 @@ __device__ __forceinline__ FoldPiece fold_piece(const int* pre, int nreq, int LG
   return q;
 }
 
-template <int REP>
+template <int REP, int PARTS>
 __global__ void __launch_bounds__(kFoldThreads, 1)
     fold_tc_kernel(const __grid_constant__ CUtensorMap mk, const __grid_constant__ CUtensorMap mv, const FoldParams p) {
   constexpr int Q = 16 * REP, QH = 8 * REP;               // queries; a softmax thread's share of them
   constexpr int CW = REP <= 5 ? QH : (REP == 7 ? 8 : 16); // score columns a thread holds at a time
-  constexpr FoldLayout L = fold_layout(REP);
+  constexpr FoldLayout L = fold_layout(REP, PARTS);
   constexpr int NS = L.slots, NB = (Q + 63) / 64;
   extern __shared__ uint8_t fsm_raw[];
   uint8_t* sm = reinterpret_cast<uint8_t*>((reinterpret_cast<uintptr_t>(fsm_raw) + 1023) & ~static_cast<uintptr_t>(1023));
   const uint32_t s_g = smem_u32(sm), s_p = s_g + L.off_p, s_ring = s_g + L.off_ring;
   float* sref = reinterpret_cast<float*>(sm + L.off_misc);   // reference of each query
-  float* sscale = sref + 128;                                // factor of a reference that moved; at a piece's end 1 / sum
+  float* sscale = sref + Q;                                  // factor of a reference that moved; at a piece's end 1 / sum
   float* sinv = sscale;
-  int* pre = reinterpret_cast<int*>(sscale + 128);           // [65]
+  int* pre = reinterpret_cast<int*>(sscale + Q);             // [65]
   int* srows = pre + 68;                                     // new rows of each request
   int* sslot = srows + kFoldMaxC;                            // and its first window slot
   uint64_t* bars = reinterpret_cast<uint64_t*>(sslot + kFoldMaxC);
@@ -370,12 +372,12 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
           // remainders first: the accumulator is small while they are added, so the
           // bits that each MMA's addition drops are theirs
 #pragma unroll
-          for (int part = 1; part >= 0; --part) {
+          for (int part = PARTS - 1; part >= 0; --part) {
 #pragma unroll
             for (int ks = 0; ks < kFoldKeys / 16; ++ks)
               umma_f16(t_o, fold_desc_mn(sv + (uint32_t)ks * 2048u, kFoldSlot / 2),
                        fold_desc_mn(s_p + (uint32_t)(part * NB * 16384) + (uint32_t)ks * 2048u, 16384u), id_o,
-                       part == 0 || ks > 0 ? 1u : keep);
+                       part < PARTS - 1 || ks > 0 ? 1u : keep);
           }
           umma_commit(b_empty(s));
           umma_commit(b_pv);
@@ -511,10 +513,10 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
             }
           }
         }
-        // P = high + remainder (bf16 each), eight queries a 16-byte store; where a
-        // thread holds all its scores, P is formed under the previous block's
-        // MMAs and waits for them only here
-        auto weights = [&](int cc, int c, uint32_t* hi, uint32_t* lo) {
+        // P in PARTS bf16 parts, each the rounded rest of those before, eight queries a
+        // 16-byte store; where a thread holds all its scores, P is formed under the
+        // previous block's MMAs and waits for them only here
+        auto weights = [&](int cc, int c, uint32_t (&w)[PARTS][4]) {
           const float4 ra = *reinterpret_cast<const float4*>(sref + c0 + cc + c);
           const float4 rb = *reinterpret_cast<const float4*>(sref + c0 + cc + c + 4);
           const float r[8] = {ra.x, ra.y, ra.z, ra.w, rb.x, rb.y, rb.z, rb.w};
@@ -523,32 +525,38 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
             const float x0 = fold_ex2((s[c + e] - r[e]) * sl2), x1 = fold_ex2((s[c + e + 1] - r[e + 1]) * sl2);
             sum[cc + c + e] += x0;
             sum[cc + c + e + 1] += x1;
-            const uint32_t h = pack_bf16(x0, x1);
-            hi[e >> 1] = h;
-            lo[e >> 1] = pack_bf16(x0 - __uint_as_float(h << 16), x1 - __uint_as_float(h & 0xffff0000u));
+            float y0 = x0, y1 = x1;
+#pragma unroll
+            for (int part = 0; part < PARTS; ++part) {
+              const uint32_t h = pack_bf16(y0, y1);
+              w[part][e >> 1] = h;
+              y0 -= __uint_as_float(h << 16);
+              y1 -= __uint_as_float(h & 0xffff0000u);
+            }
           }
         };
-        auto store_p = [&](int col, const uint32_t* hi, const uint32_t* lo) {
+        auto store_p = [&](int col, const uint32_t (&w)[PARTS][4]) {
           const uint32_t a = prow + (uint32_t)(col >> 6) * 16384u + (uint32_t)((((col & 63) >> 3) ^ (j & 7)) << 4);
-          st_v4(a, hi[0], hi[1], hi[2], hi[3]);
-          st_v4(a + (uint32_t)(NB * 16384), lo[0], lo[1], lo[2], lo[3]);
+#pragma unroll
+          for (int part = 0; part < PARTS; ++part)
+            st_v4(a + (uint32_t)(part * NB * 16384), w[part][0], w[part][1], w[part][2], w[part][3]);
         };
         if constexpr (CW == QH) {
-          uint32_t hi[QH / 2], lo[QH / 2];
+          uint32_t w[QH / 8][PARTS][4];
 #pragma unroll
-          for (int c = 0; c < QH; c += 8) weights(0, c, hi + c / 2, lo + c / 2);
+          for (int c = 0; c < QH; c += 8) weights(0, c, w[c / 8]);
           if (i > 0) fold_wait(b_pv, (uint32_t)(n - 1) & 1u, stop, p.err);
 #pragma unroll
-          for (int c = 0; c < QH; c += 8) store_p(c0 + c, hi + c / 2, lo + c / 2);
+          for (int c = 0; c < QH; c += 8) store_p(c0 + c, w[c / 8]);
         } else {
 #pragma unroll
           for (int cc = 0; cc < QH; cc += CW) {
             load(cc);
 #pragma unroll
             for (int c = 0; c < CW; c += 8) {
-              uint32_t hi[4], lo[4];
-              weights(cc, c, hi, lo);
-              store_p(c0 + cc + c, hi, lo);
+              uint32_t w[PARTS][4];
+              weights(cc, c, w);
+              store_p(c0 + cc + c, w);
             }
           }
         }
@@ -720,15 +728,34 @@ __global__ void __launch_bounds__(256) fold_merge_kernel(const FoldParams p, con
   if ((threadIdx.x & 15) == 0) p.eta[q] = mx + logf(w);
 }
 
-template <int REP>
+template <int REP, int PARTS>
 int launch_rep(const FoldParams& p, const CUtensorMap& mk, const CUtensorMap& mv, int grid, cudaStream_t s) {
-  constexpr FoldLayout L = fold_layout(REP);
+  constexpr FoldLayout L = fold_layout(REP, PARTS);
   static_assert(L.bytes <= 227 * 1024, "one CTA's shared memory");
   static const cudaError_t attr =
-      cudaFuncSetAttribute(fold_tc_kernel<REP>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
+      cudaFuncSetAttribute(fold_tc_kernel<REP, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
   if (attr != cudaSuccess) return LSP_ERR_CUDA;
-  return launch_pdl(fold_tc_kernel<REP>, dim3(grid), dim3(kFoldThreads), L.bytes, s, mk, mv, p) == cudaSuccess ? LSP_OK
-                                                                                                               : LSP_ERR_CUDA;
+  return launch_pdl(fold_tc_kernel<REP, PARTS>, dim3(grid), dim3(kFoldThreads), L.bytes, s, mk, mv, p) == cudaSuccess
+             ? LSP_OK
+             : LSP_ERR_CUDA;
+}
+
+// Parts of P.  Two leave 2^-18 on a weight, 2.0e-6 on m against 64 bits whatever the
+// length, three 1e-7 at 100 rows to 6e-7 at 60000.  Three are taken where two would be
+// less exact than the kernel that the call took without this one: view updates whose
+// 8 to 128 queries a KV head are no multiple of 16 (fp32 FMA: 6.2e-7 at 1126 rows, 40 queries,
+// where two parts leave 2.1e-6 and three 5.1e-7), and folds so short that the mma.sync
+// kernels' own two parts were their only error (prefill of 84, 1999, 4096, 60000 rows: 1.97e-6,
+// 2.08e-6, 2.29e-6, 3.1e-6; update of 100, 200 rows: 1.79e-6, 1.96e-6).  Their cost: 24.2 -> 26.0 us at
+// those 40 queries, prefill of 1999 rows 20.5 -> 21.6; at 60000 rows it would be 124 -> 141.
+int fold_parts(const FoldParams& p) {
+  const bool fma = !p.replace && (p.nq / p.nkv * p.R) % 16 != 0;
+  return fma || p.rows <= (p.replace ? 4096 : 256) ? 3 : 2;
+}
+
+template <int REP>
+int launch_parts(const FoldParams& p, const CUtensorMap& mk, const CUtensorMap& mv, int grid, cudaStream_t s) {
+  return fold_parts(p) == 3 ? launch_rep<REP, 3>(p, mk, mv, grid, s) : launch_rep<REP, 2>(p, mk, mv, grid, s);
 }
 
 }  // namespace
@@ -755,14 +782,14 @@ int launch_fold(const FoldParams& p, int num_sms, cudaStream_t s) {
   const long long blocks = (long long)p.nreq * p.L * p.nkv * ((p.rows + kFoldKeys - 1) / kFoldKeys);
   const int grid = (int)std::max(1ll, std::min((long long)num_sms, blocks));
   switch (p.nq / p.nkv) {
-    case 1: rc = launch_rep<1>(p, mk, mv, grid, s); break;
-    case 2: rc = launch_rep<2>(p, mk, mv, grid, s); break;
-    case 3: rc = launch_rep<3>(p, mk, mv, grid, s); break;
-    case 4: rc = launch_rep<4>(p, mk, mv, grid, s); break;
-    case 5: rc = launch_rep<5>(p, mk, mv, grid, s); break;
-    case 6: rc = launch_rep<6>(p, mk, mv, grid, s); break;
-    case 7: rc = launch_rep<7>(p, mk, mv, grid, s); break;
-    case 8: rc = launch_rep<8>(p, mk, mv, grid, s); break;
+    case 1: rc = launch_parts<1>(p, mk, mv, grid, s); break;
+    case 2: rc = launch_parts<2>(p, mk, mv, grid, s); break;
+    case 3: rc = launch_parts<3>(p, mk, mv, grid, s); break;
+    case 4: rc = launch_parts<4>(p, mk, mv, grid, s); break;
+    case 5: rc = launch_parts<5>(p, mk, mv, grid, s); break;
+    case 6: rc = launch_parts<6>(p, mk, mv, grid, s); break;
+    case 7: rc = launch_parts<7>(p, mk, mv, grid, s); break;
+    case 8: rc = launch_parts<8>(p, mk, mv, grid, s); break;
     default: return LSP_ERR_UNSUPPORTED;
   }
   if (rc != LSP_OK) return rc;
