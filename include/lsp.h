@@ -111,7 +111,9 @@ typedef struct lsp_config {
  *   k[b][l][j][0..nkv)[0..d)   key rows as cached by the target (rotary applied)
  *   v[b][l][j][0..nkv)[0..d)   value rows
  *   h[b][l][j][0..H)           hidden state at that row (only row accepted_len-1 is read)
- * All three are device pointers of dtype with row capacity `rows` per (b, l);
+ * All three are device pointers of dtype with row capacity `rows` per (b, l)
+ * (the counts are on the device, so the capacity chooses the kernel: one near
+ * the counts, say B + 1 in a round, is the quickest);
  * h may be null (and is not read) with LSP_NO_BOUNDARY.
  * h_rows: rows of h per (b, l).  0 (the default when the struct is zeroed) or
  * `rows`: the layout above.  1: h[b][l][0..H) holds only the boundary row --

@@ -48,7 +48,7 @@
 // the parts in turn, 2.1e-6 / 4.0e-7 / 2.1e-6 with 2 or 1 and the remainders
 // first (the mma.sync kernel this replaces: 4.6e-6 / 8.3e-7 / 2.0e-6); the call of
 // 131072 rows takes 450.6, 452.1 and 453.9 us with 8, 2 and 1 (460 with the
-// parts in turn).
+// parts in turn).  (With three parts the 1999 rows leave 4.9e-7.)
 //
 // fold_merge_kernel merges a unit's pieces (one per CTA share that touches
 // it) and the stored state, in share order: deterministic.
@@ -78,6 +78,7 @@ constexpr float kRefSlack = 24.f;            // log2 units a score may pass its 
 constexpr int kFoldMaxC = 64;
 constexpr int kCopyBatch = 4;                // window vectors a copying lane has in flight (K and V each)
 constexpr int kFoldMaxSlots = 5;
+constexpr int kFoldSmall = 128;              // rows of a prefill up to which it takes fold_small_kernel
 
 struct FoldLayout {
   int slots;
@@ -93,12 +94,13 @@ __host__ __device__ constexpr FoldLayout fold_layout(int rep, int parts) {
   L.off_ring = L.off_p + (uint32_t)(parts * nb) * 16384u;
   const uint32_t misc = 2u * 16u * (uint32_t)rep * 4u + 272u + 2u * kFoldMaxC * 4u + 160u;
   const int fit = (int)((227u * 1024u - 1024u - misc - L.off_ring) / (uint32_t)kFoldSlot);
-  L.slots = fit < kFoldMaxSlots ? fit : kFoldMaxSlots;
+  const int most = parts == 2 ? kFoldMaxSlots : kFoldMaxSlots - 1;   // (three: room for CTAs of the merge to wait in)
+  L.slots = fit < most ? fit : most;
   L.off_misc = L.off_ring + (uint32_t)L.slots * kFoldSlot;
   L.bytes = L.off_misc + misc + 1024u;
   return L;
 }
-static_assert(fold_layout(8, 2).slots >= 4 && fold_layout(4, 3).slots == 5, "K and V of two blocks fit the ring");
+static_assert(fold_layout(8, 2).slots >= 4 && fold_layout(4, 3).slots == 4, "K and V of two blocks fit the ring");
 static_assert(fold_layout(8, 3).slots >= 3, "K and V of a block and the next K fit the ring");
 
 __host__ __device__ constexpr uint32_t fold_tmem_cols(int rep) {
@@ -235,6 +237,199 @@ __device__ __forceinline__ FoldPiece fold_piece(const int* pre, int nreq, int LG
   q.n = min(nb - q.blk, f_end - f);
   q.unit = i * LG + q.lg;
   return q;
+}
+
+// Window ring (row q of the prefix in slot q mod W): a warp copies the chunks of
+// kCopyBatch x 32 vectors that next() names.  The walk goes over `longest` rows of every
+// (request, layer), the most that any request has for its window, and skips what lies past
+// a request's own (over W rows it took 6 us more at 16 requests of one row each, W = 256).
+template <typename F>
+__device__ __forceinline__ void fold_copy_window(const FoldParams& p, int longest, const int* srows, const int* sslot, int lane, F next) {
+  const int vpr = p.nkv * (kFoldD / 8), span = longest * vpr;   // 16-byte vectors of a row (all KV heads), of the rows walked
+  const int items = p.nreq * p.L * span;
+  for (;;) {
+    const long long first = next() * (kCopyBatch * 32);
+    if (first >= items) break;
+    const int k0 = (int)first + lane;
+    uint4 xk[kCopyBatch], xv[kCopyBatch];
+    size_t dst[kCopyBatch];
+    bool on[kCopyBatch];
+#pragma unroll
+    for (int u = 0; u < kCopyBatch; ++u) {
+      const int k = k0 + u * 32, ul = k / span, w = k - ul * span, r = w / vpr, v = w - r * vpr;
+      const int i = ul / p.L, l = ul - i * p.L;
+      on[u] = k < items && r < min(srows[i], p.W);
+      if (on[u]) {
+        const int n = srows[i];
+        int slot = sslot[i] + r;
+        if (slot >= p.W) slot -= p.W;
+        dst[u] = ((((size_t)(p.b0 + i) * p.L + l) * p.nkv + (v >> 4)) * p.W + slot) * kFoldD + (size_t)(v & 15) * 8;
+        const size_t src = (((size_t)ul * p.rows + (n - min(n, p.W)) + r) * vpr + v) * 8;
+        xk[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.k) + src);
+        xv[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.v) + src);
+      }
+    }
+#pragma unroll
+    for (int u = 0; u < kCopyBatch; ++u)
+      if (on[u]) {
+        *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_k) + dst[u]) = xk[u];
+        *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_v) + dst[u]) = xv[u];
+      }
+  }
+}
+
+// Boundary rows: the (request, layer) pairs first, first + step, .. by nthr threads.
+__device__ __forceinline__ void fold_copy_boundary(const FoldParams& p, const int* srows, int first, int step, int t, int nthr) {
+  for (int ul = first; ul < p.nreq * p.L; ul += step) {
+    const int i = ul / p.L, n = srows[i];
+    if (n == 0) continue;
+    const bf16* hin = static_cast<const bf16*>(p.hid) + ((size_t)ul * p.h_rows + (p.h_rows == 1 ? 0 : n - 1)) * p.H;
+    bf16* hout = static_cast<bf16*>(p.h) + ((size_t)p.b0 * p.L + ul) * p.H;
+    for (int k = t * 8; k < p.H; k += nthr * 8) *reinterpret_cast<uint4*>(hout + k) = *reinterpret_cast<const uint4*>(hin + k);
+  }
+}
+
+// The summary over at most kFoldSmall rows, of one layer l and query head h, by a CTA of
+// 256 threads: scores, weights and values in shared memory, products with mma.sync,
+// weights in three parts (see fold_parts).  What bounds it is latency: one round trip
+// for K, V and G and three barriers.
+constexpr int kSmallLd = kFoldD + 8, kSmallPLd = kFoldSmall + 8, kSmallSLd = kFoldSmall + 4;
+struct alignas(16) SmallSmem {
+  bf16 k[kFoldSmall * kSmallLd], v[kFoldSmall * kSmallLd];
+  union {
+    bf16 g[16 * kSmallLd];
+    bf16 p[3][16 * kSmallPLd];
+  };
+  float s[16 * kSmallSLd];
+  float sum[16];
+};
+
+__device__ __forceinline__ void fold_small(const FoldParams& p, SmallSmem& sm, int l, int h) {
+  const int tid = threadIdx.x, warp = warp_index(), lane = tid & 31, r = tid >> 4, c = tid & 15, n = p.rows;
+  const size_t row = (size_t)p.nkv * kFoldD, in = (size_t)l * n * row + (size_t)(h / (p.nq / p.nkv)) * kFoldD;
+  const size_t q0 = (((size_t)p.b0 * p.L + l) * p.nq + h) * p.R;
+  const bf16* k = static_cast<const bf16*>(p.k) + in;
+  const bf16* v = static_cast<const bf16*>(p.v) + in;
+  const bf16* G = static_cast<const bf16*>(p.G) + ((size_t)l * p.nq + h) * p.R * kFoldD;
+  const uint4 zero = make_uint4(0u, 0u, 0u, 0u);
+  uint4 xk[kFoldSmall / 16], xv[kFoldSmall / 16];
+#pragma unroll
+  for (int u = 0; u < kFoldSmall / 16; ++u) {
+    const int j = r + u * 16;
+    xk[u] = j < n ? *reinterpret_cast<const uint4*>(k + j * row + c * 8) : zero;
+    xv[u] = j < n ? *reinterpret_cast<const uint4*>(v + j * row + c * 8) : zero;
+  }
+  const uint4 xg = r < p.R ? *reinterpret_cast<const uint4*>(G + r * kFoldD + c * 8) : zero;
+#pragma unroll
+  for (int u = 0; u < kFoldSmall / 16; ++u) {
+    *reinterpret_cast<uint4*>(sm.k + (r + u * 16) * kSmallLd + c * 8) = xk[u];
+    *reinterpret_cast<uint4*>(sm.v + (r + u * 16) * kSmallLd + c * 8) = xv[u];
+  }
+  *reinterpret_cast<uint4*>(sm.g + r * kSmallLd + c * 8) = xg;
+  __syncthreads();
+  const int g = lane >> 2;
+  for (int j0 = 8 * warp; j0 < n; j0 += 64) {                 // scores of eight keys
+    float sc[4] = {};
+#pragma unroll
+    for (int kk = 0; kk < kFoldD; kk += 32) {
+      uint32_t b[4], a[4];
+      ldsm_x4(b, sm.k + (j0 + (lane & 7)) * kSmallLd + kk + (lane >> 3) * 8);
+#pragma unroll
+      for (int e = 0; e < 2; ++e) {
+        ldsm_x4(a, sm.g + (lane & 15) * kSmallLd + kk + e * 16 + (lane >> 4) * 8);
+        mma_bf16(sc, a, b[2 * e], b[2 * e + 1]);
+      }
+    }
+    float* o = sm.s + g * kSmallSLd + j0 + 2 * (lane & 3);
+    *reinterpret_cast<float2*>(o) = make_float2(sc[0], sc[1]);
+    *reinterpret_cast<float2*>(o + 8 * kSmallSLd) = make_float2(sc[2], sc[3]);
+  }
+  __syncthreads();
+  const float isd = rsqrtf((float)kFoldD), sl2 = 1.4426950408889634f * isd;
+  float x[kFoldSmall / 16], mx = -INFINITY, sum = 0.f;
+#pragma unroll
+  for (int u = 0; u < kFoldSmall / 16; ++u) {
+    x[u] = c + 16 * u < n ? sm.s[r * kSmallSLd + c + 16 * u] : -INFINITY;
+    mx = fmaxf(mx, x[u]);
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) mx = fmaxf(mx, __shfl_xor_sync(0xffffffffu, mx, o));
+  if (mx == -INFINITY) mx = 0.f;                              // no finite score
+#pragma unroll
+  for (int u = 0; u < kFoldSmall / 16; ++u) {
+    x[u] = exp2f((x[u] - mx) * sl2);
+    sum += x[u];
+#pragma unroll
+    for (int part = 0; part < 3; ++part) {                    // (g has been read)
+      const bf16 y = __float2bfloat16_rn(x[u]);
+      sm.p[part][r * kSmallPLd + c + 16 * u] = y;
+      x[u] -= __bfloat162float(y);
+    }
+  }
+#pragma unroll
+  for (int o = 8; o > 0; o >>= 1) sum += __shfl_xor_sync(0xffffffffu, sum, o);
+  if (c == 0) {
+    sm.sum[r] = sum;
+    if (r < p.R) p.eta[q0 + r] = mx * isd + logf(sum);
+  }
+  __syncthreads();
+  float o[2][4] = {};                                         // rows g and g + 8, dims 16 warp + 8 t + 2 (lane & 3) and the next
+#pragma unroll
+  for (int ks = 0; ks < kFoldSmall / 16; ++ks) {
+    if (16 * ks >= n) break;
+    uint32_t b[4], a[4];
+    ldsm_x4_t(b, sm.v + (16 * ks + (lane & 15)) * kSmallLd + warp * 16 + (lane >> 4) * 8);
+#pragma unroll
+    for (int part = 2; part >= 0; --part) {
+      ldsm_x4(a, sm.p[part] + (lane & 15) * kSmallPLd + 16 * ks + (lane >> 4) * 8);
+      mma_bf16(o[0], a, b[0], b[1]);
+      mma_bf16(o[1], a, b[2], b[3]);
+    }
+  }
+#pragma unroll
+  for (int hh = 0; hh < 2; ++hh) {
+    const int q = g + 8 * hh;
+    if (q >= p.R) continue;
+    const float inv = 1.0f / sm.sum[q];
+#pragma unroll
+    for (int t = 0; t < 2; ++t)
+      *reinterpret_cast<float2*>(p.m + (q0 + q) * kFoldD + warp * 16 + 8 * t + 2 * (lane & 3)) =
+          make_float2(o[t][2 * hh] * inv, o[t][2 * hh + 1] * inv);
+  }
+}
+
+// A prefill of at most kFoldSmall rows: CTA (layer, query head), then `ncopy` CTAs that copy
+// the window and the boundary rows; CTA 0 sets t (a prefill reads none).  The two kernels
+// below pay 11 to 14 us for tensor memory, records and the merge whatever the rows are,
+// more than the mma.sync kernels before them.  Device time in us (those, the two below, this
+// one): 5 layers of 32 heads 7.1, 13.8, 3.9 at 1 row, 11.8, 14.0, 5.5 at 84, 13.8, 13.6, 6.5 at 128;
+// 3 layers of 8 heads 9.1, 11.0, 4.3 at 128 rows.
+__global__ void __launch_bounds__(256) fold_small_kernel(const FoldParams p, const int ncopy) {
+  extern __shared__ __align__(16) uint8_t small_raw[];
+  griddep_launch();
+  griddep_wait();
+  const int nsum = (int)gridDim.x - ncopy;
+  if (blockIdx.x == 0 && threadIdx.x == 0) p.t[p.b0] = p.rows;
+  if ((int)blockIdx.x < nsum) {
+    if (p.R > 0)
+      fold_small(p, *reinterpret_cast<SmallSmem*>(small_raw), (int)blockIdx.x / p.nq, (int)blockIdx.x % p.nq);
+    return;
+  }
+  int* srows = reinterpret_cast<int*>(small_raw);
+  int* sslot = srows + 1;
+  const int cta = (int)blockIdx.x - nsum, warp = threadIdx.x >> 5, lane = threadIdx.x & 31, nw = min(p.rows, p.W);
+  if (threadIdx.x == 0) {
+    srows[0] = p.rows;
+    sslot[0] = p.W > 0 ? (p.rows - nw) % p.W : 0;
+  }
+  __syncthreads();
+  long long chunk = (long long)cta * 8 + warp;
+  fold_copy_window(p, nw, srows, sslot, lane, [&] {
+    const long long c = chunk;
+    chunk += (long long)ncopy * 8;
+    return c;
+  });
+  if (p.h) fold_copy_boundary(p, srows, cta, ncopy, threadIdx.x, 256);
 }
 
 template <int REP, int PARTS>
@@ -601,56 +796,20 @@ __global__ void __launch_bounds__(kFoldThreads, 1)
     }
   }
 
-  // ---- window ring (row q of the prefix in slot q mod W) and boundary rows: warps
-  // 10 and 11 from the start, and the softmax warps once their blocks are done
-  // (a long fold hides the copy under its blocks, in a short one it is most of the
-  // work).  A warp takes kCopyBatch x 32 vectors of the CTA's share at a time.
+  // ---- window ring and boundary rows: warps 10 and 11 from the start, and the softmax
+  // warps once their blocks are done (a long fold hides the copy under its blocks, in
+  // a short one it is most of the work), a chunk of the CTA's share at a time
   if (warp < 8 || warp >= 10) {
     if (p.acc && blockIdx.x == 0 && warp == 10)
       for (int i = lane; i < p.nreq; i += 32)
         if (p.acc[i] < 0 || p.acc[i] > p.rows) set_err(p.err, LSP_DEV_BAD_DELTA);
-    const int vpr = p.nkv * (kFoldD / 8), span = p.W * vpr;     // 16-byte vectors of a row (all KV heads), of a window
-    const int items = p.nreq * p.L * span;
-    for (;;) {
-      int c = lane == 0 ? atomicAdd(scopy, 1) : 0;
-      c = __shfl_sync(0xffffffffu, c, 0);
-      const long long first = ((long long)c * gridDim.x + blockIdx.x) * (kCopyBatch * 32);
-      if (first >= items) break;
-      const int k0 = (int)first + lane;
-      uint4 xk[kCopyBatch], xv[kCopyBatch];
-      size_t dst[kCopyBatch];
-      bool on[kCopyBatch];
-#pragma unroll
-      for (int u = 0; u < kCopyBatch; ++u) {
-        const int k = k0 + u * 32, ul = k / span, w = k - ul * span, r = w / vpr, v = w - r * vpr;
-        const int i = ul / p.L, l = ul - i * p.L;
-        on[u] = k < items && r < min(srows[i], p.W);
-        if (on[u]) {
-          const int n = srows[i];
-          int slot = sslot[i] + r;
-          if (slot >= p.W) slot -= p.W;
-          dst[u] = ((((size_t)(p.b0 + i) * p.L + l) * p.nkv + (v >> 4)) * p.W + slot) * kFoldD + (size_t)(v & 15) * 8;
-          const size_t src = (((size_t)ul * p.rows + (n - min(n, p.W)) + r) * vpr + v) * 8;
-          xk[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.k) + src);
-          xv[u] = *reinterpret_cast<const uint4*>(static_cast<const bf16*>(p.v) + src);
-        }
-      }
-#pragma unroll
-      for (int u = 0; u < kCopyBatch; ++u)
-        if (on[u]) {
-          *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_k) + dst[u]) = xk[u];
-          *reinterpret_cast<uint4*>(static_cast<bf16*>(p.win_v) + dst[u]) = xv[u];
-        }
-    }
-    if (p.h && warp >= 10)
-      for (int ul = (int)blockIdx.x; ul < p.nreq * p.L; ul += (int)gridDim.x) {
-        const int i = ul / p.L, n = srows[i];
-        if (n == 0) continue;
-        const bf16* hin = static_cast<const bf16*>(p.hid) + ((size_t)ul * p.h_rows + (p.h_rows == 1 ? 0 : n - 1)) * p.H;
-        bf16* hout = static_cast<bf16*>(p.h) + ((size_t)p.b0 * p.L + ul) * p.H;
-        for (int k = (tid - (kFoldSoftmax + 64)) * 8; k < p.H; k += kFoldCopy * 8)
-          *reinterpret_cast<uint4*>(hout + k) = *reinterpret_cast<const uint4*>(hin + k);
-      }
+    const int n0 = lane < p.nreq ? srows[lane] : 0, n1 = lane + 32 < p.nreq ? srows[lane + 32] : 0;
+    const int longest = min(__reduce_max_sync(0xffffffffu, max(n0, n1)), p.W);
+    fold_copy_window(p, longest, srows, sslot, lane, [&] {
+      const int c = lane == 0 ? atomicAdd(scopy, 1) : 0;
+      return (long long)__shfl_sync(0xffffffffu, c, 0) * gridDim.x + blockIdx.x;
+    });
+    if (p.h && warp >= 10) fold_copy_boundary(p, srows, (int)blockIdx.x, (int)gridDim.x, tid - (kFoldSoftmax + 64), kFoldCopy);
   }
 
   tc_fence_before();
@@ -745,9 +904,11 @@ int launch_rep(const FoldParams& p, const CUtensorMap& mk, const CUtensorMap& mv
 // less exact than the kernel that the call took without this one: view updates whose
 // 8 to 128 queries a KV head are no multiple of 16 (fp32 FMA: 6.2e-7 at 1126 rows, 40 queries,
 // where two parts leave 2.1e-6 and three 5.1e-7), and folds so short that the mma.sync
-// kernels' own two parts were their only error (prefill of 84, 1999, 4096, 60000 rows: 1.97e-6,
-// 2.08e-6, 2.29e-6, 3.1e-6; update of 100, 200 rows: 1.79e-6, 1.96e-6).  Their cost: 24.2 -> 26.0 us at
-// those 40 queries, prefill of 1999 rows 20.5 -> 21.6; at 60000 rows it would be 124 -> 141.
+// kernels' own two parts were their only error (prefill of 421, 1999, 4096, 60000 rows: 2.03e-6,
+// 2.08e-6, 2.29e-6, 3.1e-6; update of 100, 200 rows: 1.79e-6, 1.96e-6).  Their cost, device
+// time in us: 38.6 -> 41.8 at 40 queries and 4 x 1024 rows, prefill of 512 rows 15.1 -> 14.7,
+// 2048 20.9 -> 22.0, 4096 28.5 -> 31.4 (the ring is one slot shorter, so that CTAs of the merge
+// can wait on the SMs); prefill of 60000 rows it would be 124 -> 141.
 int fold_parts(const FoldParams& p) {
   const bool fma = !p.replace && (p.nq / p.nkv * p.R) % 16 != 0;
   return fma || p.rows <= (p.replace ? 4096 : 256) ? 3 : 2;
@@ -773,6 +934,17 @@ size_t fold_ws_floats(int C, int L, int nq, int nkv, int num_sms) {
 int launch_fold(const FoldParams& p, int num_sms, cudaStream_t s) {
   if (p.rows < 1 || p.nreq < 1 || p.nreq > kFoldMaxC || !p.ws) return LSP_ERR_UNSUPPORTED;
   if (p.H % 8) return LSP_ERR_SHAPE;
+  // what the tensor maps refuse, also where none is made
+  if ((reinterpret_cast<uintptr_t>(p.k) | reinterpret_cast<uintptr_t>(p.v)) & 15) return LSP_ERR_SHAPE;
+  if (p.replace && p.rows <= kFoldSmall) {
+    const int items = std::min(p.rows, p.W) * p.L * p.nkv * (kFoldD / 8);
+    const int ncopy = std::max(p.L, (items + 8 * kCopyBatch * 32 - 1) / (8 * kCopyBatch * 32));
+    constexpr size_t smem = sizeof(SmallSmem);
+    static const cudaError_t attr = cudaFuncSetAttribute(fold_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (attr != cudaSuccess) return LSP_ERR_CUDA;
+    return launch_pdl(fold_small_kernel, dim3(p.L * p.nq + ncopy), dim3(256), smem, s, p, ncopy) == cudaSuccess ? LSP_OK
+                                                                                                               : LSP_ERR_CUDA;
+  }
   CUtensorMap mk, mv;
   const uint64_t rows = (uint64_t)p.nreq * p.L * p.rows, pitch = (uint64_t)p.nkv * kFoldD;
   int rc;

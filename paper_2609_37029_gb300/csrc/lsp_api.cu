@@ -321,7 +321,10 @@ static int feats_h_rows(const lsp_target_feats* f) {
 // (about 4 us a pass); the fold pays a fixed price for each such unit an SM gets
 // a piece of.  Measured at the Qwen3-8B heads, 5 layers (per-unit kernel vs
 // fold, us): C = 1: 14.1 vs 14.3 at 64 rows, 24.0 vs 14.7 at 128; C = 4: 50.6
-// vs 25.8 at 256; C = 16: 78.9 vs 88 at 256, 128 vs 101 at 512.
+// vs 25.8 at 256; C = 16: 78.9 vs 88 at 256, 128 vs 101 at 512.  The counts are on the
+// device, so the capacity decides: rows that are few in a large one pay the fold's
+// price (C = 16, one row each in a capacity of 512: 10.9 vs 52), so a caller gives each
+// call the capacity that it needs.
 static bool fold_pays(const lsp_state* st, int rows) {
   const lsp_config& c = st->cfg;
   return st->fold_ws && c.R > 0 && rows >= 64 + 64ll * c.C * c.L * c.nkv / st->num_sms;
