@@ -264,8 +264,8 @@ int lsp_sample(lsp_state* st, const float* base_logits, const int32_t* prev_toke
  * array's device address and the SM count (a failed lookup is retried by the
  * next call); make that first call before any stream capture on the device.
  * Every call shares the array: calls that overlap on the GPU (other streams
- * or threads) race, so the caller must serialise them.  The step counters are
- * cleared on the caller's stream before each launch.  Allocates nothing and
+ * or threads) race, so the caller must serialise them.  The words that the CTAs
+ * exchange are cleared on the caller's stream before each call.  Allocates nothing and
  * calls no allocating CUDA or library routine. */
 int lsp_sample_noalloc(const float* base_logits, const int32_t* prev_token, const void* Ec,
                        const void* Wc, int dtype, int C, int B, int V, int rc,

@@ -8,7 +8,8 @@
 // Two kernels compute the same thing.
 //
 // sample_persistent_kernel (bf16, C <= 16, rc in {32, 64}, vocabulary slice
-// fits shared memory): one cooperative launch for all B steps, one CTA per SM.
+// fits shared memory): one cooperative launch for all B steps, one CTA per SM
+// (32 CTAs for a small vocabulary).
 // Each CTA owns a contiguous slice of 32-row vocabulary tiles and keeps its
 // W_c rows resident in shared memory for the whole launch.  The requests form one
 // or two groups of eight, which sixteen compute warps take in turn: the
@@ -280,22 +281,22 @@ __global__ void __launch_bounds__(kSampThreads, 2) sample_step_kernel(const Samp
 
 // ------------------------------------------------------------------ persistent kernel
 constexpr int kPWarps = 16;                          // compute warps
-// A CTA takes 16 tiles, one a compute warp, before there are more than 32 CTAs,
-// and up to 32 every CTA reads all keys itself, a lane a CTA: one hop through
-// L2 instead of two, and fewer words to poll.  Spread over all SMs with
-// leaders -> so (us): C = 6, V = 1584, B = 16 T = 0 49.1 -> 38.0; C = 2, V = 1024
-// T = 1 40.5 -> 34.5; C = 14, V = 39200, B = 8 T = 0 46.6 -> 38.0; C = 16, V = 32000,
-// B = 16 T = 1 83.6 -> 70.4.  (Two groups at T = 0 with a middling vocabulary are
-// where the atomic exchange of before was quicker: 35.5 and, at V = 16000, 30.4
-// against 33.5 now.)
+// A vocabulary of few tiles goes to 32 CTAs, and every CTA reads all keys itself, a lane a
+// CTA: one hop through L2 instead of two, and fewer words to poll.  Beyond, all SMs and
+// leaders.  The lines are where both take about the same time (us, B = 8, 32 CTAs against
+// 152): one group of requests, C = 8, 23.2 and 26.8 at V = 6400, 25.1 and 26.7 at 9984, 26.9 and
+// 27.2 at 16000 (T = 0; T = 1: 29.1 and 27.3); two, C = 16, 25.1 and 29.1 at 4096, 27.1 and 29.4 at 8000,
+// 31.4 and 29.4 at 16000 (T = 1: 35.5 and 30.8).
 constexpr int kPFewCtas = 32;
+__host__ __device__ constexpr int few_pairs(int groups) { return kPFewCtas * (groups == 1 ? 10 : 8); }
 constexpr int kPMaxGroups = 2;                       // request groups of eight
 constexpr int kPPairsPerWarp = 2;
 constexpr int kPMaxPairs = kPWarps * kPPairsPerWarp; // 32-row vocabulary tiles a CTA: 1024 rows
 constexpr int kPGroup = 8;                           // requests of a group (mma N)
 constexpr int kPMaxC = kPGroup * kPMaxGroups;
 constexpr int kIdxBits = 20, kTagBits = 12;          // low half of an exchanged key: ~index, step tag
-constexpr int kAnsCopies = 8;                        // copies of the answers
+constexpr int kAnsCopies = 4;                        // copies of the answers
+constexpr int kLineWords = 16;                       // 64-bit words of a 128-byte line
 constexpr int kLeadBatch = 5;                        // slots a leader's lane has in flight (152 CTAs in one go)
 // named barriers of the compute warps with one more warp: 1 + group, a step's keys (-> control); 3 + group,
 // E_c(y) (control ->); 5 + group, a step's corrected rows (-> I/O)
@@ -329,6 +330,14 @@ __device__ __forceinline__ unsigned long long ld_relaxed_u64(const unsigned long
   unsigned long long v;
   asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
   return v;
+}
+
+// Four words of a 32-byte sector at once (each one of them relaxed).
+__device__ __forceinline__ void ld_relaxed_4xu64(const unsigned long long* p, unsigned long long* v) {
+  asm volatile("ld.relaxed.gpu.global.v4.u64 {%0, %1, %2, %3}, [%4];"
+               : "=l"(v[0]), "=l"(v[1]), "=l"(v[2]), "=l"(v[3])
+               : "l"(p)
+               : "memory");
 }
 
 __device__ __forceinline__ void st_relaxed_u64(unsigned long long* p, unsigned long long v) {
@@ -595,20 +604,28 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   // and answers with a tagged word that every CTA reads: no counter, no
   // fence and no atomic, so the words do not queue behind the step's logits
   // traffic (the atomic key, release add and count of before: 3.6 + 1.3 us a step at
-  // T = 1).  The answers go out in 8 copies, a 128-byte line each, that 19 CTAs read:
-  // polls of one line by every CTA hold up the store they wait for (C = 8:
-  // 84 us with one copy, 78 with 8, 80 with 32).  Slots alternate between two sets: a CTA writes step s + 2 only after
+  // T = 1).  Each answer has a 128-byte line of its own, in kAnsCopies copies that the
+  // CTAs share: answers of several leaders in one line, which every CTA polls, are stored
+  // one after the other wherever the line's home is the far die (C = 16, V = 151936, B = 8
+  // T = 0: 49 or 68 us by the page that the workspace had got, now 52 on any).
+  // Slots alternate between two sets: a CTA writes step s + 2 only after
   // the answer of step s + 1, which its leader gives after reading step s (without
   // leaders: after every CTA's word of step s + 1).
   // Tags go on from launch to launch (the epoch word), so nothing is cleared.
-  unsigned long long* answers = p.slots;                                // [2][kAnsCopies][kPMaxC]
+  unsigned long long* answers = p.slots;                                // [2][kAnsCopies][kPMaxC], a line each
   constexpr unsigned long long kTagMask = (1ull << kTagBits) - 1;
   const int r0 = grp * kPGroup;
+  const bool direct = nblk <= kPFewCtas;
+  // direct: a CTA's words lie together, in a 32-byte sector up to four requests and a line
+  // of their own beyond: one store and one or two loads for all requests.  (As rows of a
+  // request, 16 CTAs a line: 23 or 29 us by the page at C = 8, V = 8000, B = 8, 23 now.)
+  const int cw = Cg <= 4 ? 4 : kLineWords;
   bool ok = true;                                                       // false: a wait has given up
   for (int s = 0; s < B; ++s) {
     const unsigned long long tag = (unsigned long long)(epoch + s + 1) & kTagMask;
-    unsigned long long* slots = p.slots + 2 * kAnsCopies * kPMaxC + (size_t)(s & 1) * C * nblk;   // [request][CTA]
-    unsigned long long* ans = answers + (s & 1) * kAnsCopies * kPMaxC;
+    unsigned long long* slots = p.slots + 2 * kAnsCopies * kPMaxC * kLineWords + (size_t)(s & 1) * C * nblk;   // [request][CTA]
+    unsigned long long* lines = p.slots + (size_t)((s & 1) * kPMaxGroups + grp) * kPFewCtas * kLineWords;   // direct: [CTA][cw]
+    unsigned long long* ans = answers + (s & 1) * kAnsCopies * kPMaxC * kLineWords;
     const bool last = s + 1 == B;
     named_bar(1 + grp, kPBar);
     if (!ok) {                                                          // nothing is published any more; the others' waits end too
@@ -619,27 +636,33 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
       unsigned long long k = 0ull;
 #pragma unroll
       for (int w = 0; w < kPWarps; ++w) k = max_u64(k, red[(grp * kPWarps + w) * kPGroup + lane]);
-      st_relaxed_u64(slots + (size_t)(r0 + lane) * nblk + blockIdx.x,
+      st_relaxed_u64(direct ? lines + (int)blockIdx.x * cw + lane : slots + (size_t)(r0 + lane) * nblk + blockIdx.x,
                      (k & 0xffffffff00000000ull) | ((k & ((1ull << kIdxBits) - 1)) << kTagBits) | tag);
     }
     __syncwarp();
     unsigned long long k = tag;                                         // lane r: the best key of request r0 + r
-    if (nblk <= kPFewCtas) {
+    if (direct) {
       // ---- few CTAs: one lane a CTA, all requests at once, no leader
       const bool writes = (int)blockIdx.x < Cg || nblk < Cg;            // (block 0 writes in both groups)
       if (!last || writes) {
         unsigned long long v[kPGroup];
-        const uint64_t t0 = global_ns();
-        for (uint32_t it = 1;; ++it) {
-          bool all = true;
+        const unsigned long long* w = lines + min(lane, nblk - 1) * cw;
+        auto poll = [&](auto load) {
+          const uint64_t t0 = global_ns();
+          for (uint32_t it = 1;; ++it) {
+            bool all = true;
+            load();
 #pragma unroll
-          for (int u = 0; u < kPGroup; ++u)
-            v[u] = u < Cg && lane < nblk ? ld_relaxed_u64(slots + (size_t)(r0 + u) * nblk + lane) : tag;
-#pragma unroll
-          for (int u = 0; u < kPGroup; ++u) all = all && (v[u] & kTagMask) == tag;
-          if (__all_sync(0xffffffffu, all)) break;
-          if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
-        }
+            for (int u = 0; u < kPGroup; ++u) {
+              if (u >= Cg) v[u] = tag;
+              all = all && (v[u] & kTagMask) == tag;
+            }
+            if (__all_sync(0xffffffffu, all)) return true;
+            if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) return false;
+          }
+        };
+        ok = Cg <= 4 ? poll([&] { ld_relaxed_4xu64(w, v); })
+                     : poll([&] { ld_relaxed_4xu64(w, v); ld_relaxed_4xu64(w + 4, v + 4); });
 #pragma unroll
         for (int u = 0; u < kPGroup; ++u) {
           const unsigned long long best = warp_max_key(v[u]);
@@ -673,7 +696,7 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
           for (int u = 0; u < kLeadBatch; ++u) best = max_u64(best, k[u]);
         }
         best = warp_max_key(best);
-        if (ok && lane < kAnsCopies) st_relaxed_u64(ans + lane * kPMaxC + r, best);
+        if (ok && lane < kAnsCopies) st_relaxed_u64(ans + (lane * kPMaxC + r) * kLineWords, best);
         if (ok && lane == 0) {
           const int t = (int)(~(uint32_t)(best >> kTagBits) & ((1u << kIdxBits) - 1));
           p.out_tokens[(size_t)r * B + s] = t < V ? t : 0;
@@ -683,7 +706,7 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
       if (ok && !last) {
         const uint64_t t0 = global_ns();
         for (uint32_t it = 1;; ++it) {
-          if (lane < Cg) k = ld_relaxed_u64(ans + ((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane);
+          if (lane < Cg) k = ld_relaxed_u64(ans + (((int)blockIdx.x % kAnsCopies) * kPMaxC + r0 + lane) * kLineWords);
           if (__all_sync(0xffffffffu, (k & kTagMask) == tag)) break;
           if ((it & 63u) == 0 && __any_sync(0xffffffffu, global_ns() - t0 > kWaitLimitNs)) { ok = false; break; }
         }
@@ -864,7 +887,8 @@ static cudaError_t launch_step(const SampleParams& p, int step, size_t smem, cud
 
 // The bf16 loop's exchange: two sets of answers (copies x requests) and of (request, CTA) key slots.
 size_t sample_slot_bytes(int C, int num_sms) {
-  return (size_t)2 * (kAnsCopies * kPMaxC + std::min(C, kPMaxC) * num_sms) * sizeof(unsigned long long);
+  static_assert(kPMaxGroups * kPFewCtas <= kAnsCopies * kPMaxC, "without leaders the words take the answers' room");
+  return (size_t)2 * (kAnsCopies * kPMaxC * kLineWords + std::min(C, kPMaxC) * num_sms) * sizeof(unsigned long long);
 }
 
 // The loops' epoch word.  (Kept at its size: lsp_sample_noalloc's documented need counts it.)
@@ -880,9 +904,9 @@ struct PersistentPlan {
 static PersistentPlan persistent_plan(const SampleParams& p) {
   PersistentPlan q;
   q.npairs = (p.V + 31) / 32;
-  q.nblk = std::min(std::min(p.num_sms, q.npairs), std::max(kPFewCtas, (q.npairs + kPWarps - 1) / kPWarps));
-  q.tpc = (q.npairs + q.nblk - 1) / q.nblk;
   q.groups = p.C > kPGroup ? 2 : 1;
+  q.nblk = std::min(std::min(p.num_sms, q.npairs), q.npairs <= few_pairs(q.groups) ? kPFewCtas : q.npairs);
+  q.tpc = (q.npairs + q.nblk - 1) / q.nblk;
   const size_t rb = (size_t)p.rc * 2;
   q.smem = (size_t)q.tpc * 32 * rb + (size_t)q.groups * kPGroup * (z_pitch(q.tpc) * sizeof(float) + rb) +
            (size_t)q.groups * (kPWarps * kPGroup + 1) * sizeof(unsigned long long);

@@ -7,10 +7,10 @@
 // framework's caching allocator, or code that must not create a state object
 // (lsp_state_create allocates the interface and a workspace).  The sampler's
 // only scratch is the per-CTA argmax partials of two consecutive steps and the
-// per-step keys and arrival counters of the persistent kernel, so this variant
+// epoch word, key slots and answers of the one-launch loops, so this variant
 // keeps them in a fixed file-scope __device__ array instead.  Every GPU that
-// loads the library holds that array until the process exits.  The counters
-// are cleared on the caller's stream before every launch, so a launch that
+// loads the library holds that array until the process exits.  The words of the
+// loops are cleared on the caller's stream before every call, so a launch that
 // gave up waiting cannot affect the next one.
 #include <cmath>
 #include <algorithm>
@@ -74,20 +74,20 @@ extern "C" int lsp_sample_noalloc(const float* base_logits, const int32_t* prev_
   const int rc_setup = scratch_for_current_device(&scratch, &num_sms);
   if (rc_setup != LSP_OK) return rc_setup;
   // Layout: argmax partials of two consecutive steps (values, then indices), then the
-  // persistent kernel's step keys and arrival counters -- align256(16 nblk C) +
-  // sample_sync_bytes(B) bytes, which must fit the array.
+  // words of the one-launch loops.  The documented need, align256(16 nblk C) +
+  // sample_sync_bytes(B) bytes, must fit the array.
   const int nblk = lsp::sample_blocks(num_sms);
   const size_t part = (size_t)2 * nblk * C;
   const size_t sync_off = (part * (sizeof(float) + sizeof(int)) + 255) / 256 * 256;
   const size_t sync_bytes = lsp::sample_sync_bytes(B);
   if (sync_off + sync_bytes > kStaticScratchBytes) return LSP_ERR_SHAPE;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The bf16 loop's key slots take the room of the partials, or what is left
-  // behind the sync words (the per-step kernel runs where neither holds them).
-  const size_t slot_bytes = lsp::sample_slot_bytes(C, num_sms), slot_off = slot_bytes <= sync_off ? 0 : sync_off + sync_bytes;
-  const bool slots = slot_off + slot_bytes <= kStaticScratchBytes;
-  const size_t clear = std::max(sync_off + sync_bytes, slots ? slot_off + slot_bytes : 0);
-  if (cudaMemsetAsync(scratch, 0, clear, s) != cudaSuccess) return LSP_ERR_CUDA;
+  // The one-launch loops' epoch word and, from the next 256 bytes on, their key slots
+  // and answers; all zero before a launch, whose tags begin at 1.  (The per-step kernel
+  // runs where they do not fit; it reads no partial that it has not written.)
+  const size_t slot_off = sync_off + 256, slot_end = slot_off + lsp::sample_slot_bytes(C, num_sms);
+  const bool slots = slot_end <= kStaticScratchBytes;
+  if (slots && cudaMemsetAsync(scratch + sync_off, 0, slot_end - sync_off, s) != cudaSuccess) return LSP_ERR_CUDA;
   lsp::SampleParams p = {};
   p.src = base_logits;
   p.dst = out_logits;
