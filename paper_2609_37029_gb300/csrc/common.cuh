@@ -265,6 +265,10 @@ __device__ __forceinline__ void tma_store_3d_hint(const void* tmap, uint32_t src
       : "memory");
 }
 
+// bytes (a multiple of 16) of shared memory to global memory, both on 16-byte boundaries.
+__device__ __forceinline__ void bulk_store(void* dst, uint32_t src, uint32_t bytes) {
+  asm volatile("cp.async.bulk.global.shared::cta.bulk_group [%0], [%1], %2;" ::"l"(dst), "r"(src), "r"(bytes) : "memory");
+}
 __device__ __forceinline__ void bulk_commit() { asm volatile("cp.async.bulk.commit_group;" ::: "memory"); }
 
 // Wait until at most N committed bulk groups still read shared memory.

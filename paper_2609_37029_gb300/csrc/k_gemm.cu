@@ -162,17 +162,66 @@ __device__ __forceinline__ void epilogue_f32(const GemmParams& p, const CUtensor
       if (issuer) bulk_commit();
     } else {
       // no tensor map describes Y (its row pitch or address is no multiple of
-      // 16 bytes): a warp writes its own 32 rows, lanes along the features
-      __syncwarp();
-      const int lane = row & 31, row0 = row - lane, f = w.col0 + c + lane;
-      float* Y = static_cast<float*>(p.Y) + (p.mode == EPI_PARTIAL ? (size_t)w.split * p.M * p.ldy : 0);
-      const int rows = min(min(32, p.tile_tok - row0), p.M - tok0 - row0);
-      if (f < p.N)
-        for (int i = 0; i < rows; ++i)
-          Y[(size_t)(tok0 + row0 + i) * p.ldy + f] =
-              *reinterpret_cast<const float*>(buf + (size_t)(row0 + i) * 128 + (((lane >> 2) ^ (i & 7)) << 4) + (lane & 3) * 4);
-      __syncwarp();
+      // 16 bytes): the group's four warps take the tile's rows in turn, lanes along the
+      // features.  (A warp's own 32 rows each left three of them idle at 16 tokens.)
+      named_bar(bar, kEpiGroup);
+      const int lane = row & 31, f = w.col0 + c + lane, rows = min(p.tile_tok, p.M - tok0);
+      float* y = static_cast<float*>(p.Y) + (p.mode == EPI_PARTIAL ? (size_t)w.split * p.M * p.ldy : 0) + (size_t)tok0 * p.ldy + f;
+      for (int i0 = row >> 5; i0 < rows; i0 += 16) {
+        float x[4];
+#pragma unroll
+        for (int u = 0; u < 4; ++u) {
+          const int i = i0 + 4 * u;                       // (a row past the tile is in the buffer all the same)
+          x[u] = *reinterpret_cast<const float*>(buf + (size_t)(i & (kTileTok - 1)) * 128 + (((lane >> 2) ^ (i & 7)) << 4) + (lane & 3) * 4);
+        }
+#pragma unroll
+        for (int u = 0; u < 4; ++u)
+          if (i0 + 4 * u < rows && f < p.N) y[(size_t)(i0 + 4 * u) * p.ldy] = x[u];
+      }
+      if (nbuf == 1) named_bar(bar, kEpiGroup);           // (else the next chunk's barrier frees this buffer)
     }
+  }
+}
+
+// The same for an output that no tensor map describes (its row pitch or address is no
+// multiple of 16 bytes), where a CTA has one item and its ring is idle: `cb` features of
+// every token row are staged where they lie against a 16-byte boundary in the output, and a
+// thread a row copies the part between the boundaries in bulk.  Stores of registers
+// pass about 32 bytes a cycle and SM: 206 x 30561 x 416 takes 14.6 us, 17.6 with them (11.4 by
+// tensor map at N = 30560), 300 x 5001 x 2048 17.5 and 19.1.
+__device__ __forceinline__ void epilogue_rows(const GemmParams& p, uint8_t* smem, uint32_t acc, const GemmItem& w, int cb, int tile,
+                                              int c_first, int c_step, int row, int thread) {
+  const int pitch = cb + 4;                             // floats; rows begin on 16 bytes
+  const size_t out0 = (p.mode == EPI_PARTIAL ? (size_t)w.split * p.M * p.ldy : 0) + (size_t)w.tok0 * p.ldy + w.col0;
+  float* stage = reinterpret_cast<float*>(smem);
+  auto shift = [&](int r, int c) {                      // floats of row r, feature c past a 16-byte boundary
+    return (int)((reinterpret_cast<uintptr_t>(static_cast<float*>(p.Y) + out0 + (size_t)r * p.ldy + c) >> 2) & 3);
+  };
+  for (int c0 = 0; c0 < w.cols; c0 += cb) {
+    const int n = min(min(cb, w.cols - c0), p.N - w.col0 - c0);
+    const int r0 = tile * p.tile_tok + row;
+    float* dst = stage + (size_t)r0 * pitch + shift(r0, c0);
+    for (int c = c_first * kChunk; c < min(cb, w.cols - c0); c += c_step * kChunk) {
+      float v[32];
+      tmem_ld32(acc + (uint32_t)(c0 + c), v);
+      if (row < p.tile_tok) {
+#pragma unroll
+        for (int e = 0; e < 32; ++e) dst[c + e] = v[e];
+      }
+    }
+    fence_proxy_async_smem();
+    named_bar(3, 2 * kEpiGroup);
+    if (thread < min(p.m_pad, p.M - w.tok0) && n > 0) {
+      float* y = static_cast<float*>(p.Y) + out0 + (size_t)thread * p.ldy + c0;
+      const int a = shift(thread, c0), head = min((4 - a) & 3, n), mid = (n - head) & ~3;
+      const float* src = stage + (size_t)thread * pitch + a;
+      if (mid > 0) bulk_store(y + head, smem_u32(src + head), (uint32_t)mid * 4u);
+      bulk_commit();
+      for (int i = 0; i < head; ++i) y[i] = src[i];
+      for (int i = head + mid; i < n; ++i) y[i] = src[i];
+      bulk_wait_read<0>();                              // the rows are staged again, or the CTA ends
+    }
+    if (c0 + cb < w.cols) named_bar(3, 2 * kEpiGroup);
   }
 }
 
@@ -426,6 +475,8 @@ __global__ void __launch_bounds__(kTwoRings ? kGemmThreads : kGemmThreads - 32, 
           tma_store_3d(&to, smem_u32(tile), w.row0 / 2, tok, 0);
           bulk_commit();
         }
+      } else if (p.row_cols > 0) {
+        epilogue_rows(p, smem, acc, w, p.row_cols, t, two ? 0 : grp, two ? 1 : 2, row, grp * kEpiGroup + row);
       } else {
         epilogue_f32(p, &to, stg, p.n_stg, chunks, acc, w, w.tok0 + t * p.tile_tok, two ? 0 : grp, two ? 1 : 2, row, 1 + grp);
       }
@@ -678,15 +729,16 @@ static void ring_stages(int width, int m_pad, bool persistent, int* w, int* x) {
 // each of four steps and each token tile) with 150 cycles of waits and commits,
 // and the round trip of a stage (2 us) over the weight stages.  A CTA costs
 // about 2 us to start; writing an item out takes 0.7 us and 0.35 us a 32-feature
-// chunk (a burst of all CTAs), under the next item's MMAs where a walk has two accumulator
+// chunk (a burst of all CTAs; register stores of many tokens longer), under the next item's MMAs where a walk has two accumulator
 // sets, partly exposed where it has one.
 static double tiling_cost(int width, int m_pad, int tok_tiles, int kblocks, long long items, int num_sms, int stages,
-                          bool persistent) {
+                          bool persistent, bool mapped) {
   const double in = (width + m_pad) * 128.0 / 115.0;
   const double hbm = width * 128.0 * (double)std::min<long long>(items, num_sms) / 6400.0;
   const double mma = (tok_tiles * 4 * std::max(width / 2, 50) + 150) / 1.9, trip = 2000.0 / stages;
   const double kb = kblocks * std::max(std::max(in, hbm), std::max(mma, trip));
-  const double waves = (double)((items + num_sms - 1) / num_sms), out = 700.0 + 11.0 * width;
+  const double waves = (double)((items + num_sms - 1) / num_sms);
+  const double out = 700.0 + (mapped || !persistent ? 11.0 : std::max(11.0, 0.13 * m_pad)) * width;
   if (!persistent) return waves * (kb + 2000.0 + out);
   const bool two_sets = 2 * tok_tiles * ((width + 31) / 32 * 32) <= 512;
   return (two_sets ? waves * std::max(kb, out) : waves * kb + (waves - 1) * 0.6 * out) + 2000.0 + out;
@@ -696,7 +748,7 @@ static double tiling_cost(int width, int m_pad, int tok_tiles, int kblocks, long
 // rows (a chunk of the epilogue is 32), for gate/up twice an odd multiple of
 // eight features.  CTAs walk the items where these make more than one wave.
 static Tiling choose_width(int mode, const int* seg_rows, int nseg, int m_pad, int tok_tiles, int groups, int splits,
-                           int kblocks, int num_sms) {
+                           int kblocks, int num_sms, bool mapped) {
   Tiling best = {};
   double cost = 1e30;
   const bool gu = mode == EPI_SWIGLU;
@@ -709,7 +761,7 @@ static Tiling choose_width(int mode, const int* seg_rows, int nseg, int m_pad, i
     int ws, xs;
     ring_stages(width, m_pad, persistent, &ws, &xs);
     if (ws < 2) continue;
-    const double c = tiling_cost(width, m_pad, tok_tiles, kb, items, num_sms, ws, persistent);
+    const double c = tiling_cost(width, m_pad, tok_tiles, kb, items, num_sms, ws, persistent, mapped);
     if (c < cost - 1e-9) {
       cost = c;
       best = {width, tiles, ws, xs, persistent};
@@ -743,7 +795,8 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   p.m_pad = ((M + p.tok_groups - 1) / p.tok_groups + 15) / 16 * 16;
   p.tok_tiles = p.m_pad > kTileTok ? 2 : 1;
   p.tile_tok = p.m_pad / p.tok_tiles;
-  const Tiling t = choose_width(mode, seg_rows, nseg, p.m_pad, p.tok_tiles, p.tok_groups, splits, p.kblocks, num_sms);
+  const bool mapped = ((reinterpret_cast<uintptr_t>(Y) | (uintptr_t)ldy * 4u) & 15) == 0;   // (fp32 outputs)
+  const Tiling t = choose_width(mode, seg_rows, nseg, p.m_pad, p.tok_tiles, p.tok_groups, splits, p.kblocks, num_sms, mapped);
   if (t.w_stages < 2) return LSP_ERR_SHAPE;
   p.width = t.width;
   p.n_tiles = t.tiles;
@@ -784,8 +837,8 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   int rc;
   const int box = gu ? p.width / 2 : p.width;
   for (int i = 0; i < 3; ++i) {
-    const int si = i < nseg ? i : 0;
-    if ((rc = make_map(&op->a[i], dtype, W[si], K, seg_rows[si], box)) != LSP_OK) return rc;
+    if (i >= nseg) op->a[i] = op->a[0];      // unused placeholder (an encoding takes the host 0.2 us)
+    else if ((rc = make_map(&op->a[i], dtype, W[i], K, seg_rows[i], box)) != LSP_OK) return rc;
   }
   if ((rc = make_map(&op->b, dtype, X, K, M, p.m_pad)) != LSP_OK) return rc;
   // TMA-store epilogue when the output view can be described (else per-thread stores)
@@ -795,7 +848,10 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
     p.tma_out = 1;
   } else {
     p.tma_out = make_out_map(&op->out, true, true, Y, p.N, M, splits, ldy, kChunk, p.tile_tok) == LSP_OK;
-    if (!p.tma_out) op->out = op->b;       // unused placeholder
+    if (!p.tma_out) {
+      op->out = op->b;                     // unused placeholder
+      if (!t.persistent) p.row_cols = std::min(p.width, (ring / (4 * p.m_pad) - 4) / kChunk * kChunk);
+    }
   }
   return LSP_OK;
 }

@@ -51,7 +51,8 @@ struct GemmParams {
   int m_pad, tok_tiles, tile_tok;   // token rows of a group, its accumulators, token rows of one
   int w_stages, x_stages, tmem_cols, tile_cols, acc_cols, n_acc;   // TMEM columns of a tile and of an accumulator set; sets
   int off_stg, n_stg, stg_tile, off_bar;   // shared memory: staging (buffers a group), SwiGLU tile bytes, barriers
-  int tma_out;          // 1: chunks leave by TMA stores (else by per-thread stores)
+  int tma_out;          // 1: chunks leave by TMA stores (else by per-thread stores,
+  int row_cols;         // or, if not 0, by bulk copies of rows, so many features at a time)
   int late_trigger;     // 1: let the next kernel launch only after this one's dependency wait
   void* Y;
   int ldy;
