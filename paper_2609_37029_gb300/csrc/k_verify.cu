@@ -12,8 +12,10 @@
 // lowest-index argmax of the target rows (T = 0).  At T = 0 the CTA that
 // finishes a request's last chunk merges the argmax partials and accepts the
 // prefix of candidates equal to the target argmax: one launch, where a second one of
-// one CTA a request made a call of the host 2 us longer (C = 4, V = 32000: 8.9 -> 7.0 us;
-// replayed from a graph 4.6 -> 5.2).  verify_draw_kernel (T > 0): CTA
+// one CTA a request makes a call of the host 1.5 us longer (C = 4, V = 32000: 9.9 -> 8.3 us).
+// In a graph, where the second one costs the device less than finding the last chunk
+// (4.55 against 4.9 us; C = 8, V = 35424 5.0 and 5.9; C = 2, V = 151936 7.0 and 7.6), a call that
+// is being captured takes two (verify_greedy_kernel).  verify_draw_kernel (T > 0): CTA
 // (vocabulary chunk, request) -- merges the request's row partials, tests the
 // B candidates one lane each (the acceptance uniforms are Philox words, so
 // every CTA finds the same first rejected position j), takes the Gumbel-max
@@ -141,11 +143,12 @@ __device__ __forceinline__ void verify_greedy(const VerifyParams& p, int b, int*
   }
 }
 
-template <bool kGreedy, int kBatch>
+// kDecide (T = 0): the CTA that finishes a request's last chunk decides it.
+template <bool kGreedy, int kBatch, bool kDecide>
 __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyParams p, const int rpr) {
   __shared__ float sv[32];
   __shared__ int si[32];
-  __shared__ int s_arg[kGreedy ? kVerMaxB + 1 : 1];
+  __shared__ int s_arg[kDecide ? kVerMaxB + 1 : 1];
   __shared__ int s_last;
   // dependents launch only after this grid's inputs are complete: the draw
   // kernel reads the call's inputs before its own wait
@@ -187,14 +190,18 @@ __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyP
         if (ver_better(sv[w], si[w], bv, bi)) { bv = sv[w]; bi = si[w]; }
       p.st_a[u] = bv;
       p.st_i[u] = bi;
-      __threadfence();
-      s_last = atomicAdd(&p.ctr[b], 1u) == (unsigned)(rpr * p.nst) - 1u;
+      if (kDecide) {
+        __threadfence();
+        s_last = atomicAdd(&p.ctr[b], 1u) == (unsigned)(rpr * p.nst) - 1u;
+      }
     }
-    __syncthreads();
-    if (!s_last) return;
-    __threadfence();
-    verify_greedy(p, b, s_arg);
-    if (threadIdx.x == 0) p.ctr[b] = 0u;
+    if constexpr (kDecide) {
+      __syncthreads();
+      if (!s_last) return;
+      __threadfence();
+      verify_greedy(p, b, s_arg);
+      if (threadIdx.x == 0) p.ctr[b] = 0u;
+    }
   } else {
     const float it2 = 1.4426950408889634f / p.temperature;   // log2(e) / T
     float m = -INFINITY, s = 0.f;
@@ -229,6 +236,14 @@ __global__ void __launch_bounds__(kVerThreads) verify_stats_kernel(const VerifyP
       p.st_b[u] = s;
     }
   }
+}
+
+// T = 0, CTA per request, after a row pass that does not decide.
+__global__ void __launch_bounds__(kVerThreads) verify_greedy_kernel(const VerifyParams p) {
+  __shared__ int s_arg[kVerMaxB + 1];
+  griddep_launch();
+  griddep_wait();
+  verify_greedy(p, blockIdx.x, s_arg);
 }
 
 // ---------------------------------------------------------------- rows up to the first rejection
@@ -589,9 +604,18 @@ int launch_verify(const VerifyParams& p, int num_sms, cudaStream_t s) {
   q.nst = std::max(1, std::min(verify_max_stat_chunks(p.V), (8 * num_sms + p.C * rpr - 1) / (p.C * rpr)));
   const dim3 grid(p.C * rpr * q.nst);
   if (greedy) {
-    e = launch_pdl(verify_stats_kernel<true, 8>, grid, dim3(kVerThreads), 0, s, q, rpr);
+    // one launch where the host's time bounds the call (6 us of HBM and less), two where the
+    // device's does, or the call is captured
+    cudaStreamCaptureStatus cap = cudaStreamCaptureStatusNone;
+    if ((long long)p.C * rpr * p.V > 10000000ll ||
+        (cudaStreamIsCapturing(s, &cap) == cudaSuccess && cap == cudaStreamCaptureStatusActive)) {
+      e = launch_pdl(verify_stats_kernel<true, 8, false>, grid, dim3(kVerThreads), 0, s, q, rpr);
+      if (e == cudaSuccess) e = launch_pdl(verify_greedy_kernel, dim3(p.C), dim3(kVerThreads), 0, s, q);
+    } else {
+      e = launch_pdl(verify_stats_kernel<true, 8, true>, grid, dim3(kVerThreads), 0, s, q, rpr);
+    }
   } else {
-    e = launch_pdl(verify_stats_kernel<false, 4>, grid, dim3(kVerThreads), 0, s, q, rpr);
+    e = launch_pdl(verify_stats_kernel<false, 4, false>, grid, dim3(kVerThreads), 0, s, q, rpr);
     // (the draw kernel's pre-wait loads need the row pass to trigger after its own wait)
     if (e == cudaSuccess) e = launch_pdl(verify_draw_kernel<false>, dim3(nch, p.C), dim3(kVerThreads), 0, s, q);
   }
