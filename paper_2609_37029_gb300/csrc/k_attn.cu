@@ -786,23 +786,18 @@ int launch_attention(const AttnParams& p, int dtype, cudaStream_t s, const AttnT
     AttnLayout a = attn_layout(p.B, p.W, p.nq, p.nkv, ks);
     if (a.bytes > 227 * 1024 || (size_t)a.rep * (ks - 1) * kMergeRec * sizeof(float) > a.bytes - a.off_kbw)
       return LSP_ERR_SHAPE;
-    static bool attr_set = false;
-    if (!attr_set) {
-      cudaFuncSetAttribute(attn_mma_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      attr_set = true;
-    }
+    static SmemOptIn once;
+    if (smem_opt_in(once, attn_mma_kernel, 227 * 1024) != cudaSuccess) return LSP_ERR_CUDA;
     if (launch_pdl(attn_mma_kernel, dim3(p.C * p.nkv), dim3(a.nwarps * 32), a.bytes, s, p, a.rep, ks,
                    a.rows_bw) != cudaSuccess)
       return LSP_ERR_CUDA;
   } else {
     const int ctx = p.B + p.W + p.R;
     const size_t fixed = (size_t)(3 * p.B * p.d + p.B * simple_lpq(p.B) + 4 + p.B * ctx + 4) * sizeof(float);
-    static bool attr32 = false;
-    if (!attr32) {
-      cudaFuncSetAttribute(attn_simple_kernel<float>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      cudaFuncSetAttribute(attn_whole_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024);
-      attr32 = true;
-    }
+    static SmemOptIn once, once_whole;
+    if (smem_opt_in(once, attn_simple_kernel<float>, 227 * 1024) != cudaSuccess ||
+        smem_opt_in(once_whole, attn_whole_kernel, 227 * 1024) != cudaSuccess)
+      return LSP_ERR_CUDA;
     // all rows at once where they fit (16-byte copies; the block's queries two a
     // CTA, more where that makes more CTAs than about one an SM), else
     // kSimpleChunk rows at a time

@@ -527,15 +527,10 @@ int attn_tc_plan(AttnTcPlan* pl, const AttnParams& p) {
 int launch_attention_tc(const AttnParams& p, const AttnTcPlan& pl, cudaStream_t s) {
   if (!pl.ok) return LSP_ERR_SHAPE;
   const TcLayout L = tc_layout(p.W, p.nq / p.nkv);
-  static bool attr_set = false;
-  if (!attr_set) {
-    if (cudaFuncSetAttribute(attn_tc_kernel<1>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
-            cudaSuccess ||
-        cudaFuncSetAttribute(attn_tc_kernel<2>, cudaFuncAttributeMaxDynamicSharedMemorySize, 227 * 1024) !=
-            cudaSuccess)
-      return LSP_ERR_CUDA;
-    attr_set = true;
-  }
+  static SmemOptIn once1, once2;
+  if ((L.dup == 2 ? smem_opt_in(once2, attn_tc_kernel<2>, 227 * 1024) : smem_opt_in(once1, attn_tc_kernel<1>, 227 * 1024)) !=
+      cudaSuccess)
+    return LSP_ERR_CUDA;
   const cudaError_t e =
       L.dup == 2 ? launch_pdl(attn_tc_kernel<2>, dim3(p.C * p.nkv), dim3(kTcThreads), (size_t)L.bytes, s, pl.wk,
                               pl.wv, pl.g, p, pl.wbox)

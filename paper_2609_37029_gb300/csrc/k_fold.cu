@@ -891,9 +891,8 @@ template <int REP, int PARTS>
 int launch_rep(const FoldParams& p, const CUtensorMap& mk, const CUtensorMap& mv, int grid, cudaStream_t s) {
   constexpr FoldLayout L = fold_layout(REP, PARTS);
   static_assert(L.bytes <= 227 * 1024, "one CTA's shared memory");
-  static const cudaError_t attr =
-      cudaFuncSetAttribute(fold_tc_kernel<REP, PARTS>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)L.bytes);
-  if (attr != cudaSuccess) return LSP_ERR_CUDA;
+  static SmemOptIn once;
+  if (smem_opt_in(once, fold_tc_kernel<REP, PARTS>, L.bytes) != cudaSuccess) return LSP_ERR_CUDA;
   return launch_pdl(fold_tc_kernel<REP, PARTS>, dim3(grid), dim3(kFoldThreads), L.bytes, s, mk, mv, p) == cudaSuccess
              ? LSP_OK
              : LSP_ERR_CUDA;
@@ -940,8 +939,8 @@ int launch_fold(const FoldParams& p, int num_sms, cudaStream_t s) {
     const int items = std::min(p.rows, p.W) * p.L * p.nkv * (kFoldD / 8);
     const int ncopy = std::max(p.L, (items + 8 * kCopyBatch * 32 - 1) / (8 * kCopyBatch * 32));
     constexpr size_t smem = sizeof(SmallSmem);
-    static const cudaError_t attr = cudaFuncSetAttribute(fold_small_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (attr != cudaSuccess) return LSP_ERR_CUDA;
+    static SmemOptIn once;
+    if (smem_opt_in(once, fold_small_kernel, smem) != cudaSuccess) return LSP_ERR_CUDA;
     return launch_pdl(fold_small_kernel, dim3(p.L * p.nq + ncopy), dim3(256), smem, s, p, ncopy) == cudaSuccess ? LSP_OK
                                                                                                                : LSP_ERR_CUDA;
   }

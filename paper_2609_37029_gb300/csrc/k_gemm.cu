@@ -858,10 +858,8 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
 
 template <typename T, bool kTwoRings>
 static int launch_t(const GemmOp* op, cudaStream_t s) {
-  static std::once_flag once;
-  std::call_once(once, [] {
-    cudaFuncSetAttribute(gemm_kernel<T, kTwoRings>, cudaFuncAttributeMaxDynamicSharedMemorySize, kSmemBudget);
-  });
+  static SmemOptIn once;
+  if (smem_opt_in(once, gemm_kernel<T, kTwoRings>, kSmemBudget) != cudaSuccess) return LSP_ERR_CUDA;
   const cudaError_t e = launch_pdl(gemm_kernel<T, kTwoRings>, op->grid, dim3(kTwoRings ? kGemmThreads : kGemmThreads - 32),
                                    op->smem, s, op->a[0], op->a[1], op->a[2], op->b, op->out, op->p);
   return e == cudaSuccess ? LSP_OK : LSP_ERR_CUDA;

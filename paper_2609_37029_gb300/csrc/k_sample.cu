@@ -875,13 +875,9 @@ static size_t sample_smem(int rc, int es) {
 
 template <typename T, int KG>
 static cudaError_t launch_step(const SampleParams& p, int step, size_t smem, cudaStream_t s) {
-  static size_t attr = 0;                 // largest dynamic shared memory granted so far
-  if (smem > attr) {
-    const cudaError_t e = cudaFuncSetAttribute(sample_step_kernel<T, KG>,
-                                               cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    attr = smem;
-  }
+  static SmemOptIn once;
+  const cudaError_t e = smem_opt_in(once, sample_step_kernel<T, KG>, smem);
+  if (e != cudaSuccess) return e;
   return launch_pdl(sample_step_kernel<T, KG>, dim3(p.nblk), dim3(kSampThreads), smem, s, p, step);
 }
 
@@ -917,13 +913,8 @@ template <int KS, int NG>
 static int launch_persistent(const SampleParams& p, cudaStream_t s) {
   const PersistentPlan q = persistent_plan(p);
   const int threads = (kPWarps + 2 * NG) * 32;
-  static size_t attr = 0;
-  if (q.smem > attr) {
-    if (cudaFuncSetAttribute(sample_persistent_kernel<KS, NG>, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)q.smem) != cudaSuccess)
-      return LSP_ERR_CUDA;
-    attr = q.smem;
-  }
+  static SmemOptIn once;
+  if (smem_opt_in(once, sample_persistent_kernel<KS, NG>, q.smem) != cudaSuccess) return LSP_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample_persistent_kernel<KS, NG>, threads, q.smem) !=
       cudaSuccess)
@@ -972,13 +963,8 @@ static int launch_persistent_f32(const SampleParams& p, cudaStream_t s) {
   const int nblk = std::min(p.num_sms, ntiles);
   const int tpc = (ntiles + nblk - 1) / nblk;
   const size_t smem = persistent_f32_smem(tpc, p.rc);
-  static size_t attr = 0;
-  if (smem > attr) {
-    if (cudaFuncSetAttribute(sample_persistent_f32_kernel, cudaFuncAttributeMaxDynamicSharedMemorySize,
-                             (int)smem) != cudaSuccess)
-      return LSP_ERR_CUDA;
-    attr = smem;
-  }
+  static SmemOptIn once;
+  if (smem_opt_in(once, sample_persistent_f32_kernel, smem) != cudaSuccess) return LSP_ERR_CUDA;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, sample_persistent_f32_kernel, kPfThreads,
                                                     smem) != cudaSuccess)

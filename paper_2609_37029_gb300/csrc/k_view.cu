@@ -480,13 +480,8 @@ __global__ void __launch_bounds__(MT * 32, vu_min_blocks(MT)) view_update_mma_ke
 template <int MT>
 static int launch_mma(const ViewParams& p, cudaStream_t s) {
   const size_t smem = vu_smem_bytes(MT);
-  static size_t attr = 0;
-  if (smem > attr) {
-    if (cudaFuncSetAttribute(view_update_mma_kernel<MT>, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem) !=
-        cudaSuccess)
-      return LSP_ERR_CUDA;
-    attr = smem;
-  }
+  static SmemOptIn once;
+  if (smem_opt_in(once, view_update_mma_kernel<MT>, smem) != cudaSuccess) return LSP_ERR_CUDA;
   return launch_pdl(view_update_mma_kernel<MT>, dim3(p.C * p.L * p.nkv), dim3(MT * 32), smem, s, p) ==
                  cudaSuccess
              ? LSP_OK

@@ -7,6 +7,7 @@
 #include <stdint.h>
 
 #include "../../include/lsp.h"
+#include "smem_opt_in.h"
 
 namespace lsp {
 
@@ -28,6 +29,17 @@ inline cudaError_t launch_pdl(void (*kernel)(KArgs...), dim3 grid, dim3 block, s
   cfg.attrs = attr;
   cfg.numAttrs = 1;
   return cudaLaunchKernelEx(&cfg, kernel, args...);
+}
+
+// `bytes` of dynamic shared memory for `kernel` on the current device (one SmemOptIn a kernel).
+template <typename... KArgs>
+inline cudaError_t smem_opt_in(SmemOptIn& once, void (*kernel)(KArgs...), size_t bytes) {
+  int dev = 0;
+  const cudaError_t e = cudaGetDevice(&dev);
+  if (e != cudaSuccess) return e;
+  return static_cast<cudaError_t>(once.ensure(dev, bytes, [&] {
+    return static_cast<int>(cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)bytes));
+  }));
 }
 
 // ------------------------------------------------------------------ GEMM
