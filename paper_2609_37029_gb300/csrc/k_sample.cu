@@ -741,13 +741,13 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
 constexpr int kPfThreads = 256;
 
 __global__ void __launch_bounds__(kPfThreads, 1)
-    sample_persistent_f32_kernel(const SampleParams p, const int ntiles) {
+    sample_persistent_f32_kernel(const SampleParams p, const int ntiles, const int pad) {
   extern __shared__ __align__(16) float pfs[];
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, nw = kPfThreads / 32;
   const int nblk = gridDim.x;
   const int t_begin = (int)(((long long)blockIdx.x * ntiles) / nblk);
   const int cnt = (int)(((long long)(blockIdx.x + 1) * ntiles) / nblk) - t_begin;
-  const int C = p.C, B = p.B, V = p.V, rc = p.rc, wp = rc + 4;
+  const int C = p.C, B = p.B, V = p.V, rc = p.rc, wp = rc + pad;
   const int v0 = t_begin * 16, nv = cnt * 16;
   float* Ws = pfs;                                  // [nv][wp]
   float* Es = Ws + (size_t)nv * wp;                 // [C][rc]
@@ -939,7 +939,13 @@ static int launch_persistent_any(const SampleParams& p, cudaStream_t s) {
 }
 
 // The persistent kernel's shape limits (anything else takes the per-step kernel).
-static size_t persistent_f32_smem(int tpc, int rc) { return ((size_t)tpc * 16 * (rc + 4) + kPMaxC * rc) * sizeof(float); }
+static size_t persistent_f32_smem(int tpc, int rc, int pad) {
+  return ((size_t)tpc * 16 * (rc + pad) + kPMaxC * rc) * sizeof(float);
+}
+// Floats between two W_c rows: a vector, or none where only that fits (slices that fit
+// without padding had become B + 1 launches: V = 240000, rc = 32).
+constexpr size_t kPfSmem = 220 * 1024;
+static int persistent_f32_pad(int tpc, int rc) { return persistent_f32_smem(tpc, rc, 4) <= kPfSmem ? 4 : 0; }
 
 static bool coop_ok() {
   int dev = 0, coop = 0;
@@ -955,14 +961,15 @@ static bool persistent_f32_ok(const SampleParams& p, int dtype) {
   const int ntiles = p.V / 16;
   const int nblk = std::min(p.num_sms, ntiles);
   const int tpc = (ntiles + nblk - 1) / nblk;
-  return persistent_f32_smem(tpc, p.rc) <= 220 * 1024 && coop_ok();
+  return persistent_f32_smem(tpc, p.rc, persistent_f32_pad(tpc, p.rc)) <= kPfSmem && coop_ok();
 }
 
 static int launch_persistent_f32(const SampleParams& p, cudaStream_t s) {
   const int ntiles = p.V / 16;
   const int nblk = std::min(p.num_sms, ntiles);
   const int tpc = (ntiles + nblk - 1) / nblk;
-  const size_t smem = persistent_f32_smem(tpc, p.rc);
+  const int pad = persistent_f32_pad(tpc, p.rc);
+  const size_t smem = persistent_f32_smem(tpc, p.rc, pad);
   static SmemOptIn once;
   if (smem_opt_in(once, sample_persistent_f32_kernel, smem) != cudaSuccess) return LSP_ERR_CUDA;
   int per_sm = 0;
@@ -980,7 +987,7 @@ static int launch_persistent_f32(const SampleParams& p, cudaStream_t s) {
   attr_c[0].val.cooperative = 1;
   cfg.attrs = attr_c;
   cfg.numAttrs = 1;
-  return cudaLaunchKernelEx(&cfg, sample_persistent_f32_kernel, p, ntiles) == cudaSuccess ? LSP_OK
+  return cudaLaunchKernelEx(&cfg, sample_persistent_f32_kernel, p, ntiles, pad) == cudaSuccess ? LSP_OK
                                                                                          : LSP_ERR_CUDA;
 }
 
