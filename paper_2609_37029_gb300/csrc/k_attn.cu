@@ -802,7 +802,7 @@ int launch_attention(const AttnParams& p, int dtype, cudaStream_t s, const AttnT
     // CTA, more where that makes more CTAs than about one an SM), else
     // kSimpleChunk rows at a time
     int nqs = std::min(2, 32 / simple_lpq(p.B));
-    while (nqs < p.B && 2 * nqs * simple_lpq(p.B) <= 32 && p.C * p.nq * ((p.B + nqs - 1) / nqs) > 152) nqs *= 2;
+    while (nqs < p.B && 2 * nqs * simple_lpq(p.B) <= 32 && p.C * p.nq * ((p.B + nqs - 1) / nqs) > p.num_sms) nqs *= 2;
     int pad = 1;                         // (rows without padding where only those fit)
     if (whole_layout(p.B, p.d, p.W + p.R, nqs, pad).bytes > 227 * 1024) pad = 0;
     const WholeLayout L = whole_layout(p.B, p.d, p.W + p.R, nqs, pad);

@@ -521,7 +521,7 @@ int lsp_draft(lsp_state* st, const int32_t* block_tokens, const lsp_weights* w,
     ap.qkv = st->qkv;
     ap.win_k = st->win_k; ap.win_v = st->win_v; ap.G = st->G; ap.m = st->m; ap.t = st->t;
     ap.out = st->o; ap.C = c.C; ap.B = c.B; ap.L = c.L; ap.nq = c.nq; ap.nkv = c.nkv; ap.d = c.d;
-    ap.W = c.W; ap.R = c.R; ap.layer = c.layer_map[j]; ap.eps = c.rms_eps; ap.err = st->err;
+    ap.W = c.W; ap.R = c.R; ap.layer = c.layer_map[j]; ap.num_sms = st->num_sms; ap.eps = c.rms_eps; ap.err = st->err;
     ap.part = st->part; ap.splits = st->qkv_op[j].p.splits; ap.q_norm = lw.q_norm; ap.k_norm = lw.k_norm;
     ap.rope = st->rope;
     if ((rc = launch_attention(ap, c.dtype, s, &st->attn_tc)) != LSP_OK) return rc;

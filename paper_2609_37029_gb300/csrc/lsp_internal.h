@@ -172,7 +172,7 @@ struct AttnParams {
   const float* m;         // [C][L][nq][R][d]
   const int64_t* t;       // [C]
   void* out;              // [M][nq d]
-  int C, B, L, nq, nkv, d, W, R, layer;
+  int C, B, L, nq, nkv, d, W, R, layer, num_sms;
   float eps;
   unsigned* err;          // device error word (a bounded wait that gave up)
   // tcgen05 kernel only: the q/k/v projection's split partials, finalised
