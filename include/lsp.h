@@ -330,11 +330,30 @@ size_t lsp_linear_workspace_bytes(int M, int N, int splits);
  *   fused gate/up projection with N = F (gate and up each [F][K]).
  *   *splits: split-K factor (it fixes the order of the fp32 sums);
  *   *tok_groups: groups of *tokens_per_group consecutive token rows (a
- *   multiple of 16) that the plan's cost model divides M into.
+ *   multiple of 16) that the model which chooses the factor divides M into.
+ *   A launch has groups of its own (lsp_gemm_launch_info).
  * LSP_ERR_ARG for null outputs, M outside [1, 512], N, K or num_sms < 1 or
  * an unknown dtype. */
 int lsp_gemm_plan_info(int dtype, int M, int N, int K, int swiglu, int num_sms, int* splits,
                        int* tok_groups, int* tokens_per_group);
+
+/* Diagnostic, host only (needs no GPU): how the projection GEMM is launched for
+ * the same arguments (splits = 0: the factor above; the output is taken to
+ * begin on 16 bytes).  A CTA works on items of tile_rows weight rows (swiglu: half of
+ * them gate rows, half up) x tokens_per_group token rows x one split; there are
+ * tiles x token_groups x splits items, one a CTA, or `ctas` = num_sms CTAs that walk
+ * them.  `accumulators` of tokens_per_group / accumulators token rows each take an item, in
+ * accumulator_sets sets of tensor memory columns (tmem_columns in all);
+ * weight_stages and activation_stages k-blocks are in flight (the same stages up to 128
+ * tokens a group) in smem_bytes of shared memory.  LSP_ERR_ARG as above, LSP_ERR_SHAPE
+ * where no launch fits. */
+typedef struct lsp_gemm_launch {
+  int splits, token_groups, tokens_per_group, accumulators;
+  int tile_rows, tiles, ctas, weight_stages, activation_stages;
+  int accumulator_sets, tmem_columns, smem_bytes;
+} lsp_gemm_launch;
+int lsp_gemm_launch_info(int dtype, int M, int N, int K, int swiglu, int splits, int num_sms,
+                         lsp_gemm_launch* out);
 int lsp_linear(const void* X, const void* W, float* Y, int M, int N, int K, int dtype,
                int splits, void* workspace, size_t workspace_bytes, lsp_stream_t stream);
 

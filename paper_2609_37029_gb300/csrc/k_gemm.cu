@@ -770,9 +770,8 @@ static Tiling choose_width(int mode, const int* seg_rows, int nseg, int m_pad, i
   return best;
 }
 
-int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* const* W,
-              const int* seg_rows, int nseg, int mode, void* Y, int ldy, unsigned* err,
-              int num_sms, int splits) {
+int gemm_layout(GemmParams* pp, size_t* smem, int* ctas, int dtype, int M, int K, const int* seg_rows, int nseg, int mode,
+                int num_sms, int splits, bool mapped) {
   if (M < 1 || M > 512 || K < 1 || nseg < 1 || nseg > 3) return LSP_ERR_SHAPE;
   const bool gu = mode == EPI_SWIGLU;
   if (gu && nseg != 2) return LSP_ERR_SHAPE;
@@ -780,7 +779,7 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   if ((K * es) % 16) return LSP_ERR_SHAPE;
   for (int i = 0; i + 1 < nseg && !gu; ++i)
     if (seg_rows[i] % kTileRows) return LSP_ERR_SHAPE;
-  GemmParams& p = op->p;
+  GemmParams& p = *pp;
   p = GemmParams{};
   p.M = M;
   p.K = K;
@@ -795,7 +794,6 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   p.m_pad = ((M + p.tok_groups - 1) / p.tok_groups + 15) / 16 * 16;
   p.tok_tiles = p.m_pad > kTileTok ? 2 : 1;
   p.tile_tok = p.m_pad / p.tok_tiles;
-  const bool mapped = ((reinterpret_cast<uintptr_t>(Y) | (uintptr_t)ldy * 4u) & 15) == 0;   // (fp32 outputs)
   const Tiling t = choose_width(mode, seg_rows, nseg, p.m_pad, p.tok_tiles, p.tok_groups, splits, p.kblocks, num_sms, mapped);
   if (t.w_stages < 2) return LSP_ERR_SHAPE;
   p.width = t.width;
@@ -817,10 +815,6 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   p.n_acc = t.persistent && 2 * p.acc_cols <= 512 ? 2 : 1;
   p.tmem_cols = 32;
   while (p.tmem_cols < p.n_acc * p.acc_cols) p.tmem_cols *= 2;
-  p.Y = Y;
-  p.ldy = ldy;
-  p.err = err;
-  op->dtype = dtype;
   // shared memory: activation ring | weight ring | staging of a walk | barriers;
   // an accumulator of fewer than 128 tokens reads past its activation tile
   // (lanes nobody looks at), into the weight ring or what follows
@@ -831,10 +825,26 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
   if (gu && p.tok_tiles * p.stg_tile > ring) return LSP_ERR_SHAPE;
   p.off_bar = std::max(ring + (t.persistent ? kStgBytes : 0), (p.x_stages * p.m_pad - p.tile_tok + kTileTok) * 128);
   if (!gu && !t.persistent) p.off_bar = std::max(p.off_bar, p.n_stg * kStgBytes);
-  op->smem = (size_t)p.off_bar + kBarBytes + 1024;
-  if (op->smem > (size_t)kSmemBudget) return LSP_ERR_SHAPE;
-  op->grid = dim3((unsigned)(t.persistent ? num_sms : p.items), 1, 1);
-  int rc;
+  if (!gu && !mapped && !t.persistent) p.row_cols = std::min(p.width, (ring / (4 * p.m_pad) - 4) / kChunk * kChunk);
+  *smem = (size_t)p.off_bar + kBarBytes + 1024;
+  if (*smem > (size_t)kSmemBudget) return LSP_ERR_SHAPE;
+  *ctas = t.persistent ? num_sms : p.items;
+  return LSP_OK;
+}
+
+int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* const* W,
+              const int* seg_rows, int nseg, int mode, void* Y, int ldy, unsigned* err,
+              int num_sms, int splits) {
+  const bool gu = mode == EPI_SWIGLU;
+  const bool mapped = ((reinterpret_cast<uintptr_t>(Y) | (uintptr_t)ldy * 4u) & 15) == 0;   // (fp32 outputs)
+  GemmParams& p = op->p;
+  int ctas = 0, rc;
+  if ((rc = gemm_layout(&p, &op->smem, &ctas, dtype, M, K, seg_rows, nseg, mode, num_sms, splits, mapped)) != LSP_OK) return rc;
+  op->grid = dim3((unsigned)ctas, 1, 1);
+  op->dtype = dtype;
+  p.Y = Y;
+  p.ldy = ldy;
+  p.err = err;
   const int box = gu ? p.width / 2 : p.width;
   for (int i = 0; i < 3; ++i) {
     if (i >= nseg) op->a[i] = op->a[0];      // unused placeholder (an encoding takes the host 0.2 us)
@@ -847,11 +857,8 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
       return rc;
     p.tma_out = 1;
   } else {
-    p.tma_out = make_out_map(&op->out, true, true, Y, p.N, M, splits, ldy, kChunk, p.tile_tok) == LSP_OK;
-    if (!p.tma_out) {
-      op->out = op->b;                     // unused placeholder
-      if (!t.persistent) p.row_cols = std::min(p.width, (ring / (4 * p.m_pad) - 4) / kChunk * kChunk);
-    }
+    p.tma_out = make_out_map(&op->out, true, true, Y, p.N, M, p.splits, ldy, kChunk, p.tile_tok) == LSP_OK;
+    if (!p.tma_out) op->out = op->b;       // unused placeholder
   }
   return LSP_OK;
 }

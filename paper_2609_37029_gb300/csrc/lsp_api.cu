@@ -574,6 +574,31 @@ int lsp_gemm_plan_info(int dtype, int M, int N, int K, int swiglu, int num_sms, 
   return LSP_OK;
 }
 
+int lsp_gemm_launch_info(int dtype, int M, int N, int K, int swiglu, int splits, int num_sms, lsp_gemm_launch* out) {
+  if (!out || M < 1 || M > 512 || N < 1 || K < 1 || num_sms < 1 || splits < 0) return LSP_ERR_ARG;
+  if (dtype != LSP_DTYPE_BF16 && dtype != LSP_DTYPE_F32) return LSP_ERR_ARG;
+  const int rows[2] = {N, N};
+  GemmParams p;
+  size_t smem = 0;
+  int ctas = 0;
+  const int rc = gemm_layout(&p, &smem, &ctas, dtype, M, K, rows, swiglu ? 2 : 1, swiglu ? EPI_SWIGLU : EPI_PARTIAL, num_sms,
+                             splits, N % 4 == 0);
+  if (rc != LSP_OK) return rc;
+  out->splits = p.splits;
+  out->token_groups = p.tok_groups;
+  out->tokens_per_group = p.m_pad;
+  out->accumulators = p.tok_tiles;
+  out->tile_rows = p.width;
+  out->tiles = p.n_tiles;
+  out->ctas = ctas;
+  out->weight_stages = p.w_stages;
+  out->activation_stages = p.x_stages;
+  out->accumulator_sets = p.n_acc;
+  out->tmem_columns = p.tmem_cols;
+  out->smem_bytes = (int)smem;
+  return LSP_OK;
+}
+
 size_t lsp_linear_workspace_bytes(int M, int N, int splits) {
   if (M < 1 || N < 1 || splits < 1) return 0;
   return splits == 1 ? 0 : (size_t)splits * M * N * sizeof(float);

@@ -90,12 +90,16 @@ int gemm_plan(GemmOp* op, int dtype, const void* X, int M, int K, const void* co
               const int* seg_rows, int nseg, int mode, void* Y, int ldy, unsigned* err,
               int num_sms, int splits);
 int gemm_launch(const GemmOp* op, cudaStream_t s);
-// The split-K factor gemm_plan uses (input <= 0 = choose), and the token
-// groups it splits M into (groups may be null).
+// What of a plan needs no pointer: tiles, rings, accumulators, shared memory and CTAs.
+// mapped: a tensor map can describe the output (16-byte aligned rows).
+int gemm_layout(GemmParams* p, size_t* smem, int* ctas, int dtype, int M, int K, const int* seg_rows, int nseg, int mode,
+                int num_sms, int splits, bool mapped);
+// The split-K factor gemm_plan uses (input <= 0 = choose), and the token groups
+// of the model that chooses it (groups may be null; the launch's own are GemmParams').
 void gemm_choose(int dtype, int M, int K, int n_tiles, int mode, int num_sms, int* splits,
                  int* groups = nullptr);
 int gemm_tiles(int mode, const int* seg_rows, int nseg);
-// Token rows one token group of M rows split G ways covers (a multiple of 16).
+// Token rows that one of G token groups of that model covers (a multiple of 16).
 int gemm_group_rows(int M, int G);
 // occ_max: CTAs one SM can hold (1-3) for this tile shape.
 int gemm_auto_splits(int n_ctas, int kblocks, int num_sms, double per_split_cost, int max_splits,

@@ -57,6 +57,11 @@ class lsp_sample_params(Structure):
     _fields_ = [("temperature", c_float), ("round", c_uint32), ("seed", c_uint64)]
 
 
+class lsp_gemm_launch(Structure):
+    _fields_ = [(n, c_int) for n in "splits token_groups tokens_per_group accumulators tile_rows tiles ctas weight_stages "
+                "activation_stages accumulator_sets tmem_columns smem_bytes".split()]
+
+
 class LspError(RuntimeError):
     def __init__(self, status: int, where: str):
         self.status = status
@@ -92,6 +97,8 @@ _f = {
     "lsp_linear_workspace_bytes": _sig("lsp_linear_workspace_bytes", c_size_t, c_int, c_int, c_int),
     "lsp_gemm_plan_info": _sig("lsp_gemm_plan_info", c_int, c_int, c_int, c_int, c_int, c_int, c_int,
                                POINTER(c_int), POINTER(c_int), POINTER(c_int)),
+    "lsp_gemm_launch_info": _sig("lsp_gemm_launch_info", c_int, c_int, c_int, c_int, c_int, c_int, c_int, c_int,
+                                 POINTER(lsp_gemm_launch)),
     "lsp_linear": _sig("lsp_linear", c_int, c_void_p, c_void_p, c_void_p, c_int, c_int, c_int, c_int,
                        c_int, c_void_p, c_size_t, c_void_p),
     "lsp_philox_words": _sig("lsp_philox_words", c_int, c_uint64, c_uint32, c_uint32, c_uint32,
@@ -234,11 +241,19 @@ def lsp_linear_workspace_bytes(M: int, N: int, splits: int) -> int:
 
 
 def lsp_gemm_plan_info(dtype, M, N, K, swiglu, num_sms):
-    """(splits, token groups, token rows per group) of the projection GEMM's plan (host only)."""
+    """(splits, token groups, token rows per group) of the split-K model (host only)."""
     s, g, r = c_int(0), c_int(0), c_int(0)
     _check(_f["lsp_gemm_plan_info"](dtype, M, N, K, int(bool(swiglu)), num_sms, ctypes.byref(s),
                                     ctypes.byref(g), ctypes.byref(r)), "lsp_gemm_plan_info")
     return s.value, g.value, r.value
+
+
+def lsp_gemm_launch_info(dtype, M, N, K, swiglu, splits, num_sms) -> lsp_gemm_launch:
+    """How the projection GEMM is launched (host only); splits = 0: the drafter's factor."""
+    out = lsp_gemm_launch()
+    _check(_f["lsp_gemm_launch_info"](dtype, M, N, K, int(bool(swiglu)), splits, num_sms, ctypes.byref(out)),
+           "lsp_gemm_launch_info")
+    return out
 
 
 def lsp_linear(X, W, Y, M, N, K, dtype, splits=1, workspace=None, workspace_bytes=0,
