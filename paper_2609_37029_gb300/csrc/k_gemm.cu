@@ -729,8 +729,10 @@ static void ring_stages(int width, int m_pad, bool persistent, int* w, int* x) {
 // each of four steps and each token tile) with 150 cycles of waits and commits,
 // and the round trip of a stage (2 us) over the weight stages.  A CTA costs
 // about 2 us to start; writing an item out takes 0.7 us and 0.35 us a 32-feature
-// chunk (a burst of all CTAs; register stores of many tokens longer), under the next item's MMAs where a walk has two accumulator
-// sets, partly exposed where it has one.
+// chunk (a burst of all CTAs), under the next item's MMAs where a walk has two accumulator
+// sets, partly exposed where it has one.  A walk that stores from registers takes 2.2 us
+// and, from 85 tokens on, longer a chunk (22 x 10875 x 3344 in 6 splits: 20.8 -> 18.1 us by the width
+// that this chooses).
 static double tiling_cost(int width, int m_pad, int tok_tiles, int kblocks, long long items, int num_sms, int stages,
                           bool persistent, bool mapped) {
   const double in = (width + m_pad) * 128.0 / 115.0;
@@ -738,7 +740,7 @@ static double tiling_cost(int width, int m_pad, int tok_tiles, int kblocks, long
   const double mma = (tok_tiles * 4 * std::max(width / 2, 50) + 150) / 1.9, trip = 2000.0 / stages;
   const double kb = kblocks * std::max(std::max(in, hbm), std::max(mma, trip));
   const double waves = (double)((items + num_sms - 1) / num_sms);
-  const double out = 700.0 + (mapped || !persistent ? 11.0 : std::max(11.0, 0.13 * m_pad)) * width;
+  const double out = mapped || !persistent ? 700.0 + 11.0 * width : 2200.0 + std::max(11.0, 0.13 * m_pad) * width;
   if (!persistent) return waves * (kb + 2000.0 + out);
   const bool two_sets = 2 * tok_tiles * ((width + 31) / 32 * 32) <= 512;
   return (two_sets ? waves * std::max(kb, out) : waves * kb + (waves - 1) * 0.6 * out) + 2000.0 + out;
