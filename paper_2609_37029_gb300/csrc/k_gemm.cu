@@ -827,7 +827,11 @@ int gemm_layout(GemmParams* pp, size_t* smem, int* ctas, int dtype, int M, int K
   if (gu && p.tok_tiles * p.stg_tile > ring) return LSP_ERR_SHAPE;
   p.off_bar = std::max(ring + (t.persistent ? kStgBytes : 0), (p.x_stages * p.m_pad - p.tile_tok + kTileTok) * 128);
   if (!gu && !t.persistent) p.off_bar = std::max(p.off_bar, p.n_stg * kStgBytes);
-  if (!gu && !mapped && !t.persistent) p.row_cols = std::min(p.width, (ring / (4 * p.m_pad) - 4) / kChunk * kChunk);
+  // (copies of narrow tiles' rows cost more than the registers' stores: width 32, 500 x 2001 x
+  // 300 9.8 us against 9.2; 64, one accumulator, 64 x 3001 x 4096 11.1 and 10.2, but two, 250 x 9001 x
+  // 512, 8.3 and 8.8; 96, 300 x 5001 x 2048, 16.6 and 17.5)
+  if (!gu && !mapped && !t.persistent && p.width >= (p.tok_tiles == 2 ? 64 : 96))
+    p.row_cols = std::min(p.width, (ring / (4 * p.m_pad) - 4) / kChunk * kChunk);
   *smem = (size_t)p.off_bar + kBarBytes + 1024;
   if (*smem > (size_t)kSmemBudget) return LSP_ERR_SHAPE;
   *ctas = t.persistent ? num_sms : p.items;
