@@ -53,10 +53,10 @@
 // fold_merge_kernel merges a unit's pieces (one per CTA share that touches
 // it) and the stored state, in share order: deterministic.
 //
-// Measured (GB300, Qwen3-8B heads, 5 layers): lsp_prefill of 131072 rows
-// (2.68 GB) 745 us with the mma.sync kernel, 386 + 7 us now (6.9 TB/s, the copy
-// bandwidth); lsp_view_update of 2048 rows 232 -> 22 us for one request, 423 ->
-// 162 us for 16.
+// Measured (GB300, Qwen3-8B heads, 5 layers, in a graph): lsp_prefill of 131072
+// rows (2.68 GB) 738 us with the mma.sync kernel, 399 us now with the merge (6.7
+// TB/s, the copy bandwidth), of 1999 rows 44 -> 23 us; lsp_view_update of 2048 rows
+// 231 -> 22 us for one request, 421 -> 162 us for 16.
 #include <algorithm>
 #include <type_traits>
 

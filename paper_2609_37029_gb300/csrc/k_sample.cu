@@ -607,7 +607,7 @@ __global__ void __launch_bounds__((kPWarps + 4) * 32, 1)
   // T = 1).  Each answer has a 128-byte line of its own, in kAnsCopies copies that the
   // CTAs share: answers of several leaders in one line, which every CTA polls, are stored
   // one after the other wherever the line's home is the far die (C = 16, V = 151936, B = 8
-  // T = 0: 49 or 68 us by the page that the workspace had got, now 52 on any).
+  // T = 0: 49 or 68 us by the page that the workspace had got, now 50 on any).
   // Slots alternate between two sets: a CTA writes step s + 2 only after
   // the answer of step s + 1, which its leader gives after reading step s (without
   // leaders: after every CTA's word of step s + 1).

@@ -30,7 +30,7 @@
 // rejection carry the result, and a drafter is rejected somewhere in most blocks.
 // Measured at C = 16, B = 16, V = 151936 (T = 1: 321 MB of rows): 64.5 us whatever
 // is accepted before; now 45 us where 4.8 candidates are accepted on average and 62.5
-// where all are; T = 0 30 us before, 13 at 0.5 accepted, 31 at 16.  Chunks twice as long
+// where all are; T = 0 30 us before, 13 at 0.5 accepted, 30.4 at 16.  Chunks twice as long
 // (fewer CTAs): 47 and 60, T = 0 27.
 //
 // Randomness (Philox4x32-10, key = seed): the acceptance uniform of position i
